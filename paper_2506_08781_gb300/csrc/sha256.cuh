@@ -40,8 +40,26 @@ __device__ __forceinline__ uint32_t rotr32(uint32_t x, uint32_t n) { return __fu
 // Big-endian load helper: byte-swap a little-endian 32-bit word.
 __device__ __forceinline__ uint32_t bswap32(uint32_t x) { return __byte_perm(x, 0, 0x0123); }
 
+// a + b on the IMAD pipe: a product by a 1 that the compiler cannot see through.
+static __device__ __constant__ uint32_t kShaOne = 1u;
+__device__ __forceinline__ uint32_t imad_add(uint32_t a, uint32_t b, uint32_t one) {
+  uint32_t r;
+  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(one), "r"(b));
+  return r;
+}
+
 // One compression of the 16 big-endian message words w (clobbered) into state st.
+//
+// Bound by the ALU pipe (rotations, logic and three-input additions at one instruction per two
+// cycles and SM quarter), with the IMAD pipe beside it idle: the additions whose operands are
+// all registers go there.  1,088 ALU and 473 IMAD instructions a compression instead of 1,265
+// and 119: 2,264 cycles against 2,580 at full occupancy (0.96 of the ALU pipe's rate).  The
+// additions of a round constant stay, since an IMAD takes either the constant or the hidden 1
+// as its one non-register operand, and a third register operand costs more in register-port
+// conflicts (2,547 cycles) than the pipe change gives; right shifts as high products lose too
+// (2,298: a high product takes the IMAD pipe for four cycles).
 __device__ __forceinline__ void sha256_compress(uint32_t st[8], uint32_t w[16]) {
+  const uint32_t one = kShaOne;
   uint32_t a = st[0], b = st[1], c = st[2], d = st[3], e = st[4], f = st[5], g = st[6], h = st[7];
 #pragma unroll
   for (int i = 0; i < 64; ++i) {
@@ -52,16 +70,17 @@ __device__ __forceinline__ void sha256_compress(uint32_t st[8], uint32_t w[16]) 
       const uint32_t x = w[(i + 1) & 15], y = w[(i + 14) & 15];
       const uint32_t s0 = rotr32(x, 7) ^ rotr32(x, 18) ^ (x >> 3);
       const uint32_t s1 = rotr32(y, 17) ^ rotr32(y, 19) ^ (y >> 10);
-      wi = w[i & 15] + s0 + w[(i + 9) & 15] + s1;
+      wi = imad_add(s1, imad_add(s0, imad_add(w[i & 15], w[(i + 9) & 15], one), one), one);
       w[i & 15] = wi;
     }
     const uint32_t S1 = rotr32(e, 6) ^ rotr32(e, 11) ^ rotr32(e, 25);
     const uint32_t ch = (e & f) ^ (~e & g);
-    const uint32_t t1 = h + S1 + ch + kSha256K[i] + wi;
+    const uint32_t t0 = h + wi + kSha256K[i];
+    const uint32_t t1 = imad_add(S1, imad_add(ch, t0, one), one);
     const uint32_t S0 = rotr32(a, 2) ^ rotr32(a, 13) ^ rotr32(a, 22);
     const uint32_t maj = (a & b) ^ (a & c) ^ (b & c);
-    h = g; g = f; f = e; e = d + t1;
-    d = c; c = b; b = a; a = t1 + S0 + maj;
+    h = g; g = f; f = e; e = imad_add(d, t1, one);
+    d = c; c = b; b = a; a = imad_add(S0, imad_add(maj, t1, one), one);
   }
   st[0] += a; st[1] += b; st[2] += c; st[3] += d; st[4] += e; st[5] += f; st[6] += g; st[7] += h;
 }
