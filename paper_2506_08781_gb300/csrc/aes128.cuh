@@ -7,7 +7,7 @@
 // (2 S(a), S(a), S(a), 3 S(a)) as a big-endian word (rows 0..3); the contributions of rows
 // 1, 2, 3 are T rotated right by 8, 16, 24 bits.  S(a) itself is byte 2 (and byte 1) of T[a].
 //
-// Shared memory.  The table has 32 copies, entry a of copy c at word 32 a + c, i.e. in bank
+// Shared memory.  The table of the kernels with few encryptions has 32 copies, entry a of copy c at word 32 a + c, i.e. in bank
 // c: lane c of a warp reads only copy c, so data-dependent lookups never conflict (32 KiB
 // per block).  Each block builds it at start from the S-box definition (the inverse in
 // GF(2^8) followed by the affine map of FIPS-197 Sec. 5.1.1); no table is stored anywhere.
@@ -67,26 +67,82 @@ __device__ __forceinline__ void aes_tables_init(AesShared& sh) {
   __syncthreads();
 }
 
+__device__ __forceinline__ uint32_t ror32(uint32_t x, uint32_t n) { return __funnelshift_r(x, x, n); }
+
 // Table reads: entry (byte K of w) of the lane's copy; a byte permute isolates the byte in one
-// instruction (13 % faster on GB300 than shift-and-mask; the kernel is bound by the ALU pipe,
-// 78 % busy, with the shared-memory pipe at 45 %).  Explicit byte-offset addressing, with or
-// without ld.shared, measured no faster.
+// instruction.  The three members are the steps of a round: an output column from the four
+// input columns' bytes, S-box values alone (bytes 3..0 from S of byte 3 of a, byte 2 of b,
+// byte 1 of c, byte 0 of d), and SubWord(RotWord(w)) (S of bytes 2, 1, 0, 3 of w).
 struct AesCtx {
   const AesShared* sh;
   uint32_t lane;
   template <int K>
   __device__ __forceinline__ uint32_t T(uint32_t w) const { return sh->t[__byte_perm(w, 0u, 0x4440u | K)][lane]; }
+  // S is byte 2 of a table entry
+  __device__ __forceinline__ static uint32_t join(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    return (a & 0x00ff0000u) << 8 | (b & 0x00ff0000u) | (c & 0x00ff0000u) >> 8 | (d & 0x00ff0000u) >> 16;
+  }
+  __device__ __forceinline__ uint32_t column(uint32_t a, uint32_t b, uint32_t c, uint32_t d) const {
+    return T<3>(a) ^ ror32(T<2>(b), 8) ^ ror32(T<1>(c), 16) ^ ror32(T<0>(d), 24);
+  }
+  __device__ __forceinline__ uint32_t sub4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) const {
+    return join(T<3>(a), T<2>(b), T<1>(c), T<0>(d));
+  }
+  __device__ __forceinline__ uint32_t sub_rot(uint32_t w) const { return join(T<2>(w), T<1>(w), T<0>(w), T<3>(w)); }
 };
 
 __device__ __forceinline__ AesCtx aes_ctx(const AesShared* sh) { return AesCtx{sh, threadIdx.x & 31u}; }
 
-__device__ __forceinline__ uint32_t ror32(uint32_t x, uint32_t n) { return __funnelshift_r(x, x, n); }
+// The message hashing's tables (k_hash, where all but a few of the encryptions are): T and its
+// three rotations, 32 copies each, 128 KiB of dynamic shared memory per block.  Rows v of T0 and
+// T1 are the two halves of 256 bytes at 256 v, T2 and T3 follow at 64 KiB, so a lookup's
+// address is one byte permute -- byte 1 is the state byte, byte 0 the lane's word in the row --
+// and the load, and a column needs no rotations: 20 permutes, 20 loads and 15 other
+// instructions a round (at one table: two more address steps a lookup and 12 rotations).
+// What bounds it: the shared-memory pipe at one load a cycle and SM (200 loads an encryption,
+// 800 cycles for the four SM quarters' warps) and next to it the ALU pipe (about 700).
+constexpr uint32_t kAesWideBytes = 4u * 256u * 128u;
+extern __shared__ __align__(16) uint8_t aes_wide_smem[];
 
-// Four S-box values assembled into one word: bytes 3..0 from S of byte 3 of a, byte 2 of b,
-// byte 1 of c, byte 0 of d (S is byte 2 of a table entry).
-__device__ __forceinline__ uint32_t aes_sub4(const AesCtx& c, uint32_t a, uint32_t b, uint32_t cc, uint32_t d) {
-  return (c.T<3>(a) & 0x00ff0000u) << 8 | (c.T<2>(b) & 0x00ff0000u) | (c.T<1>(cc) & 0x00ff0000u) >> 8 |
-         (c.T<0>(d) & 0x00ff0000u) >> 16;
+struct AesWide {
+  uint32_t lane;   // byte 0: 4 x lane, byte 1: 4 x lane + 128, bytes 2 and 3: 0
+  // table R (T rotated right by 8 R bits) at byte K of w
+  template <int K, int R>
+  __device__ __forceinline__ uint32_t T(uint32_t w) const {
+    const uint32_t o = __byte_perm(w, lane, 0x7600u | K << 4 | (4 + (R & 1)));
+    return *reinterpret_cast<const uint32_t*>(aes_wide_smem + (R >> 1) * 65536 + o);
+  }
+  // bytes 3, 2, 1, 0 of entries whose S-box value lies in that byte
+  __device__ __forceinline__ static uint32_t join(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    return __byte_perm(__byte_perm(a, b, 0x3600u), __byte_perm(c, d, 0x0014u), 0x3254u);
+  }
+  __device__ __forceinline__ uint32_t column(uint32_t a, uint32_t b, uint32_t c, uint32_t d) const {
+    return T<3, 0>(a) ^ T<2, 1>(b) ^ T<1, 2>(c) ^ T<0, 3>(d);
+  }
+  // S is byte 3 of T2 and T3, byte 2 of T0 and T3, byte 1 of T0 and T1, byte 0 of T1 and T2
+  __device__ __forceinline__ uint32_t sub4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) const {
+    return join(T<3, 2>(a), T<2, 3>(b), T<1, 0>(c), T<0, 1>(d));
+  }
+  __device__ __forceinline__ uint32_t sub_rot(uint32_t w) const {
+    return join(T<2, 2>(w), T<1, 3>(w), T<0, 0>(w), T<3, 1>(w));
+  }
+};
+
+// Every thread of the block must call this (it ends with a barrier).
+__device__ __forceinline__ AesWide aes_wide_init() {
+  __shared__ uint32_t t0[256];
+  for (uint32_t a = threadIdx.x; a < 256; a += blockDim.x) {
+    const uint32_t s = aes_sbox_entry(a), s2 = gf8_xtime(s);
+    t0[a] = (s2 << 24) | (s << 16) | (s << 8) | (s2 ^ s);
+  }
+  __syncthreads();
+  // word i of the area: table 2 (i >> 14) + (i >> 5 & 1), row i >> 6 & 255, copy i & 31
+  uint32_t* area = reinterpret_cast<uint32_t*>(aes_wide_smem);
+  for (uint32_t i = threadIdx.x; i < kAesWideBytes / 4; i += blockDim.x)
+    area[i] = ror32(t0[(i >> 6) & 255u], 8u * (2u * (i >> 14) + ((i >> 5) & 1u)));
+  __syncthreads();
+  const uint32_t l = 4u * (threadIdx.x & 31u);
+  return AesWide{l | (l + 128u) << 8};
 }
 
 // State of one FIPS-197 Cipher (Nk = 4, Nr = 10) between rounds: the round key k and the
@@ -100,54 +156,58 @@ __device__ __forceinline__ AesState aes_begin(const uint32_t key[4], const uint3
 }
 
 // Round r (1..10) with round constant rcon = x^(r-1).
-__device__ __forceinline__ void aes_round(const AesCtx& c, AesState& a, int r, uint32_t rcon) {
+template <class C>
+__device__ __forceinline__ void aes_round(const C& c, AesState& a, int r, uint32_t rcon) {
   // round key r from round key r-1: SubWord(RotWord(w3)) ^ Rcon into w0, then the chain
-  // (RotWord moves byte 2 of w3 to the top, so SubWord(RotWord(w3)) = S(w3 bytes 2,1,0,3))
-  const uint32_t sub = aes_sub4(c, a.k3 << 8, a.k3 << 8, a.k3 << 8, a.k3 >> 24);
-  a.k0 ^= sub ^ (rcon << 24);
+  a.k0 ^= c.sub_rot(a.k3) ^ (rcon << 24);
   a.k1 ^= a.k0;
   a.k2 ^= a.k1;
   a.k3 ^= a.k2;
   uint32_t t0, t1, t2, t3;
   if (r < 10) {
-    t0 = c.T<3>(a.s0) ^ ror32(c.T<2>(a.s1), 8) ^ ror32(c.T<1>(a.s2), 16) ^ ror32(c.T<0>(a.s3), 24) ^ a.k0;
-    t1 = c.T<3>(a.s1) ^ ror32(c.T<2>(a.s2), 8) ^ ror32(c.T<1>(a.s3), 16) ^ ror32(c.T<0>(a.s0), 24) ^ a.k1;
-    t2 = c.T<3>(a.s2) ^ ror32(c.T<2>(a.s3), 8) ^ ror32(c.T<1>(a.s0), 16) ^ ror32(c.T<0>(a.s1), 24) ^ a.k2;
-    t3 = c.T<3>(a.s3) ^ ror32(c.T<2>(a.s0), 8) ^ ror32(c.T<1>(a.s1), 16) ^ ror32(c.T<0>(a.s2), 24) ^ a.k3;
+    t0 = c.column(a.s0, a.s1, a.s2, a.s3) ^ a.k0;
+    t1 = c.column(a.s1, a.s2, a.s3, a.s0) ^ a.k1;
+    t2 = c.column(a.s2, a.s3, a.s0, a.s1) ^ a.k2;
+    t3 = c.column(a.s3, a.s0, a.s1, a.s2) ^ a.k3;
   } else {   // last round: no MixColumns
-    t0 = aes_sub4(c, a.s0, a.s1, a.s2, a.s3) ^ a.k0;
-    t1 = aes_sub4(c, a.s1, a.s2, a.s3, a.s0) ^ a.k1;
-    t2 = aes_sub4(c, a.s2, a.s3, a.s0, a.s1) ^ a.k2;
-    t3 = aes_sub4(c, a.s3, a.s0, a.s1, a.s2) ^ a.k3;
+    t0 = c.sub4(a.s0, a.s1, a.s2, a.s3) ^ a.k0;
+    t1 = c.sub4(a.s1, a.s2, a.s3, a.s0) ^ a.k1;
+    t2 = c.sub4(a.s2, a.s3, a.s0, a.s1) ^ a.k2;
+    t3 = c.sub4(a.s3, a.s0, a.s1, a.s2) ^ a.k3;
   }
   a.s0 = t0; a.s1 = t1; a.s2 = t2; a.s3 = t3;
 }
 
 // E_key(in): FIPS-197 Cipher with Nk = 4, Nr = 10.
-__device__ __forceinline__ void aes128_encrypt(const AesCtx& c, const uint32_t key[4], const uint32_t in[4],
+template <class C>
+__device__ __forceinline__ void aes128_encrypt(const C& c, const uint32_t key[4], const uint32_t in[4],
                                                uint32_t out[4]) {
   AesState a = aes_begin(key, in);
   uint32_t rcon = 0x01u;
 #pragma unroll 1
-  for (int r = 1; r <= 10; ++r) {
+  for (int r = 1; r < 10; ++r) {
     aes_round(c, a, r, rcon);
     rcon = gf8_xtime(rcon);
   }
+  aes_round(c, a, 10, rcon);
   out[0] = a.s0; out[1] = a.s1; out[2] = a.s2; out[3] = a.s3;
 }
 
 // E_keyA(in) and E_keyB(in) with their rounds interleaved: two independent chains in one
 // loop, so each one's table reads and XORs fill the other's dependency gaps.
-__device__ __forceinline__ void aes128_encrypt2(const AesCtx& c, const uint32_t keyA[4], const uint32_t keyB[4],
+template <class C>
+__device__ __forceinline__ void aes128_encrypt2(const C& c, const uint32_t keyA[4], const uint32_t keyB[4],
                                                 const uint32_t in[4], uint32_t outA[4], uint32_t outB[4]) {
   AesState a = aes_begin(keyA, in), b = aes_begin(keyB, in);
   uint32_t rcon = 0x01u;
 #pragma unroll 1
-  for (int r = 1; r <= 10; ++r) {
+  for (int r = 1; r < 10; ++r) {
     aes_round(c, a, r, rcon);
     aes_round(c, b, r, rcon);
     rcon = gf8_xtime(rcon);
   }
+  aes_round(c, a, 10, rcon);
+  aes_round(c, b, 10, rcon);
   outA[0] = a.s0; outA[1] = a.s1; outA[2] = a.s2; outA[3] = a.s3;
   outB[0] = b.s0; outB[1] = b.s1; outB[2] = b.s2; outB[3] = b.s3;
 }
@@ -157,7 +217,8 @@ __device__ __forceinline__ void aes128_encrypt2(const AesCtx& c, const uint32_t 
 constexpr uint32_t kIvA = 0x52525252u, kIvB = 0x25252525u;
 
 // One MMO step: h <- E_h(m) ^ m.
-__device__ __forceinline__ void mmo_step(const AesCtx& c, uint32_t h[4], const uint32_t m[4]) {
+template <class C>
+__device__ __forceinline__ void mmo_step(const C& c, uint32_t h[4], const uint32_t m[4]) {
   uint32_t o[4];
   aes128_encrypt(c, h, m, o);
 #pragma unroll
@@ -166,7 +227,8 @@ __device__ __forceinline__ void mmo_step(const AesCtx& c, uint32_t h[4], const u
 
 // PRF_bit(z) with kappa = 127: the seed's first 127 bits and the bit fill one block, one
 // AES call; the output keeps 127 bits (bit 0 of byte 15 cleared).
-__device__ __forceinline__ void prf_node_aes(const AesCtx& c, const uint32_t z[4], uint32_t bit, uint32_t out[4]) {
+template <class C>
+__device__ __forceinline__ void prf_node_aes(const C& c, const uint32_t z[4], uint32_t bit, uint32_t out[4]) {
   const uint32_t m[4] = {z[0], z[1], z[2], (z[3] & ~1u) | bit};
   uint32_t h[4] = {kIvA, kIvA, kIvA, kIvA};
   mmo_step(c, h, m);
@@ -175,7 +237,8 @@ __device__ __forceinline__ void prf_node_aes(const AesCtx& c, const uint32_t z[4
 
 // x_i^j = PRF_0(x_0[i] || j): MMO over seed (PRF bit 0) || le32(j), 20 bytes padded with
 // 0x80 and zeros to two blocks; truncated to 127 bits.
-__device__ __forceinline__ void prf_entry_aes(const AesCtx& c, const uint32_t x0[4], uint32_t j, uint32_t out[4]) {
+template <class C>
+__device__ __forceinline__ void prf_entry_aes(const C& c, const uint32_t x0[4], uint32_t j, uint32_t out[4]) {
   const uint32_t m1[4] = {x0[0], x0[1], x0[2], x0[3] & ~1u};
   const uint32_t m2[4] = {__byte_perm(j, 0, 0x0123), 0x80000000u, 0u, 0u};
   uint32_t h[4] = {kIvA, kIvA, kIvA, kIvA};
@@ -186,7 +249,8 @@ __device__ __forceinline__ void prf_entry_aes(const AesCtx& c, const uint32_t x0
 
 // One MDC-2 step on block m: both chains take an MMO step, then exchange their right
 // halves (words 2 and 3).
-__device__ __forceinline__ void mdc2_step(const AesCtx& c, uint32_t h[4], uint32_t g[4], const uint32_t m[4]) {
+template <class C>
+__device__ __forceinline__ void mdc2_step(const C& c, uint32_t h[4], uint32_t g[4], const uint32_t m[4]) {
   uint32_t a[4], b[4];
   aes128_encrypt2(c, h, g, m, a, b);
 #pragma unroll

@@ -66,7 +66,8 @@ struct HashArgs {
   uint32_t* z_out;             // optional (weighted): n*4 words of z_t
   const uint32_t* z_in;        // optional (weighted): z_t already computed (k_weights); read, not hashed
   uint8_t* sbad_out;           // optional: n bytes, 1 = s_t is not canonical
-  unsigned long long* partial; // per block: 13 u64 limb sums of e, 13 of s, 1 bad count (27 u64)
+  uint32_t ngroups;            // groups of kHashThreads threads, one partial each (set by launch_hash)
+  unsigned long long* partial; // per group: 13 u64 limb sums of e, 13 of s, 1 bad count (27 u64)
   uint32_t* status;            // device status word (kErrInput for decreasing offsets)
   // multi-device batches (n_seg > 0): entry t belongs to the device d with
   // seg_start[d] <= t < seg_start[d+1]; its index in that signer's log is
@@ -183,14 +184,14 @@ __device__ __forceinline__ void hash_entry(const uint8_t* m, uint32_t L, const u
 // ----------------------------------------------------------------------------------------
 enum : int { kInstSha = 0, kInstAes = 1 };
 
-template <int INST>
-__device__ __forceinline__ void prf_node_i(const AesCtx& c, const uint32_t z[4], uint32_t bit, uint32_t out[4]) {
+template <int INST, class C>
+__device__ __forceinline__ void prf_node_i(const C& c, const uint32_t z[4], uint32_t bit, uint32_t out[4]) {
   if constexpr (INST == kInstAes) prf_node_aes(c, z, bit, out);
   else prf_node(z, bit, out);
 }
 
-template <int INST>
-__device__ __forceinline__ void prf_entry_i(const AesCtx& c, const uint32_t x0[4], uint32_t j, uint32_t out[4]) {
+template <int INST, class C>
+__device__ __forceinline__ void prf_entry_i(const C& c, const uint32_t x0[4], uint32_t j, uint32_t out[4]) {
   if constexpr (INST == kInstAes) prf_entry_aes(c, x0, j, out);
   else prf_entry(x0, j, out);
 }
@@ -198,7 +199,8 @@ __device__ __forceinline__ void prf_entry_i(const AesCtx& c, const uint32_t x0[4
 // MDC-2-AES-128 over the padded stream: (L + 16 + 16) / 16 blocks (the 0x80 byte always
 // fits, a whole-block input gains a block).  dig = the 32-byte digest as 8 little-endian
 // words (the integer H(m || x) before reduction mod q).
-__device__ __forceinline__ void mdc2_stream(const AesCtx& c, const EntryStream& es, uint32_t dig[8]) {
+template <class C>
+__device__ __forceinline__ void mdc2_stream(const C& c, const EntryStream& es, uint32_t dig[8]) {
   uint32_t h[4] = {kIvA, kIvA, kIvA, kIvA}, g[4] = {kIvB, kIvB, kIvB, kIvB};
   const uint32_t nb = (es.L + 32) >> 4;
 #pragma unroll 1
@@ -219,8 +221,8 @@ __device__ __forceinline__ void mdc2_stream(const AesCtx& c, const EntryStream& 
 }
 
 // H(m || x) as 8 little-endian digest words for the instantiation.
-template <int INST>
-__device__ __forceinline__ void entry_digest(const AesCtx& c, const uint8_t* m, uint32_t L, const uint32_t x[4],
+template <int INST, class C>
+__device__ __forceinline__ void entry_digest(const C& c, const uint8_t* m, uint32_t L, const uint32_t x[4],
                                              uint32_t dig[8]) {
   if constexpr (INST == kInstAes) {
     mdc2_stream(c, entry_stream(m, L, x), dig);
@@ -688,7 +690,12 @@ void launch_epoch_seeds(int inst, unsigned grid, unsigned block, cudaStream_t st
 // registers a thread), so that three decoding blocks and one hashing block share an SM and
 // the hashing (ALU pipe) runs during the decoding (IMAD pipe) instead of after it.
 constexpr int kCoresidentMinBlocks = 4;
-void launch_hash(int inst, unsigned grid, cudaStream_t st, const HashArgs& a, bool coresident = false);
+// What shares the SMs with a hashing launch: nothing of its size; the decoding of one point per
+// entry; the same, both compiled for 128 registers a thread (multi-device batches).
+enum HashPlace { kHashAlone, kHashBeside, kHashCoresident };
+unsigned hash_groups(int inst, int sm_count, uint64_t n);
+cudaError_t hash_kernels_init();   // once per device, before the first POSLO+ launch
+void launch_hash(int inst, unsigned groups, cudaStream_t st, HashArgs a, HashPlace place);
 void launch_points(unsigned grid, cudaStream_t st, const PointArgs& a, bool coresident = false);
 struct ZPre { uint32_t w[10]; };   // BE words of "POSLO-Z" || verifier_seed || (byte 39 = 0)
 __global__ void k_weights(const ZPre zp, uint64_t n, uint64_t first, uint32_t* z_out);

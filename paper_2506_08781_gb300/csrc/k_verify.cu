@@ -45,13 +45,23 @@ __global__ void k_epoch_seeds(const DsNode* __restrict__ ds, int nds, uint64_t e
   *o = make_uint4(x[0], x[1], x[2], x[3]);
 }
 
-// Entries are processed in tiles of kHashTile; inside a tile they are reordered by the
-// number of SHA-256 blocks of m_t || x_t (a counting sort in shared memory), so the lanes of
-// a warp run the same number of compressions.  Per entry, one loop drives every
-// compression (the PRF block, the message blocks, and the weight block in weighted mode)
-// through a single inlined copy of the compression function.
+// Entries are processed in tiles of kHashTile by groups of kHashThreads threads; inside a tile
+// they are reordered by their number of compressions (a counting sort in shared memory), so
+// the lanes of a warp run the same number.  A thread's second entry comes from the other end of
+// the order, so that the warps of a group carry like amounts of work.  Per entry, one loop
+// drives every SHA-256 compression (the PRF block, the message blocks, and the weight block in
+// weighted mode) through a single inlined copy of the compression function.
 constexpr int kHashTile = 256;
-constexpr int kHashClasses = 8;
+constexpr int kHashClasses = 32;   // one per lane: the prefix sums are a warp scan
+constexpr int kHashPer = kHashTile / kHashThreads;
+static_assert(kHashPer == 2, "a thread takes one entry from each end of the order");
+
+// Barrier of one group of kHashThreads threads (the whole block when it is one group).
+template <int GROUPS>
+__device__ __forceinline__ void group_sync(int g) {
+  if constexpr (GROUPS == 1) __syncthreads();
+  else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(kHashThreads) : "memory");
+}
 
 // z_t = SHA-256("POSLO-Z" || verifier_seed || le64(t)): the single padded block.
 __device__ __forceinline__ void weight_block(const uint32_t zpre[10], uint64_t zi, uint32_t w[16]) {
@@ -81,61 +91,66 @@ __global__ void k_weights(const ZPre zp, uint64_t n, uint64_t first, uint32_t* z
   }
 }
 
-// MINB: resident blocks per SM the kernel is compiled for -- POSLO_HASH_MIN_BLOCKS when it runs
-// on its own, kCoresidentMinBlocks (128 registers) when it is to share the SMs with the
-// decoding of a multi-device batch.
-template <int INST, int MINB>
-__global__ void __launch_bounds__(kHashThreads, MINB) k_hash(const HashArgs a) {
-  AesCtx c{};
-  if constexpr (INST == kInstAes) {
-    __shared__ AesShared sh;
-    aes_tables_init(sh);
-    c = aes_ctx(&sh);
-  }
+// MINB: resident blocks per SM the kernel is compiled for.  GROUPS: groups per block, each with
+// its own tiles and partial; more than one where the block's tables fill most of an SM's shared
+// memory (POSLO+), so that the groups share them.
+template <int INST, int MINB, int GROUPS>
+__global__ void __launch_bounds__(kHashThreads * GROUPS, MINB) k_hash(const HashArgs a) {
+  AesWide c{};
+  if constexpr (INST == kInstAes) c = aes_wide_init();
   acc13 acc_e, acc_s;
   acc_zero(acc_e);
   acc_zero(acc_s);
   uint32_t bad = 0;
-  __shared__ uint16_t s_order[kHashTile];
-  __shared__ uint32_t s_cnt[kHashClasses], s_off[kHashClasses];
-  constexpr int kPer = kHashTile / kHashThreads;
+  __shared__ uint16_t s_order_[GROUPS][kHashTile];
+  __shared__ uint32_t s_cnt_[GROUPS][kHashClasses], s_off_[GROUPS][kHashClasses];
+  const int g = GROUPS == 1 ? 0 : (int)(threadIdx.x / kHashThreads);
+  const uint32_t tid = threadIdx.x % kHashThreads;
+  const uint32_t group = blockIdx.x * GROUPS + g;
+  uint16_t* s_order = s_order_[g];
+  uint32_t *s_cnt = s_cnt_[g], *s_off = s_off_[g];
   const uint64_t ntiles = (a.n + kHashTile - 1) / kHashTile;
-  for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  for (uint64_t tile = group; tile < ntiles && group < a.ngroups; tile += a.ngroups) {
     const uint64_t base = tile * kHashTile;
     const uint64_t rem = a.n - base;
     const uint32_t m = rem < (uint64_t)kHashTile ? (uint32_t)rem : (uint32_t)kHashTile;
-    if (threadIdx.x < kHashClasses) s_cnt[threadIdx.x] = 0;
-    __syncthreads();
-    uint32_t cls[kPer], pos[kPer];
+    if (tid < kHashClasses) s_cnt[tid] = 0;
+    group_sync<GROUPS>(g);
+    uint32_t cls[kHashPer], pos[kHashPer];
 #pragma unroll
-    for (int r = 0; r < kPer; ++r) {
-      const uint32_t k = threadIdx.x + r * kHashThreads;
+    for (int r = 0; r < kHashPer; ++r) {
+      const uint32_t k = tid + r * kHashThreads;
       if (k < m) {
         const uint64_t lo = a.offs[base + k], hi = a.offs[base + k + 1];
         if (hi < lo || lo < a.base_off || hi - lo > 0xffffffffull) atomicOr(a.status, kErrInput);
         const uint64_t L = hi >= lo ? hi - lo : 0;
-        const uint64_t c = (L + 88) >> 6;
-        cls[r] = c < (uint64_t)(kHashClasses - 1) ? (uint32_t)c : (uint32_t)(kHashClasses - 1);
+        const uint64_t nblk = INST == kInstAes ? (L + 32) >> 4 : (L + 88) >> 6;
+        cls[r] = nblk < (uint64_t)(kHashClasses - 1) ? (uint32_t)nblk : (uint32_t)(kHashClasses - 1);
         pos[r] = atomicAdd(&s_cnt[cls[r]], 1u);
       }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t acc = 0;
-      for (int c = 0; c < kHashClasses; ++c) { s_off[c] = acc; acc += s_cnt[c]; }
-    }
-    __syncthreads();
+    group_sync<GROUPS>(g);
+    if (tid < kHashClasses) {   // one warp: exclusive prefix sums of the class counts
+      const uint32_t own = s_cnt[tid];
+      uint32_t incl = own;
 #pragma unroll
-    for (int r = 0; r < kPer; ++r) {
-      const uint32_t k = threadIdx.x + r * kHashThreads;
+      for (int o = 1; o < kHashClasses; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if ((int)tid >= o) incl += v;
+      }
+      s_off[tid] = incl - own;
+    }
+    group_sync<GROUPS>(g);
+#pragma unroll
+    for (int r = 0; r < kHashPer; ++r) {
+      const uint32_t k = tid + r * kHashThreads;
       if (k < m) s_order[s_off[cls[r]] + pos[r]] = (uint16_t)k;
     }
-    __syncthreads();
+    group_sync<GROUPS>(g);
 #pragma unroll 1
-    for (int r = 0; r < kPer; ++r) {
-      const uint32_t k = threadIdx.x + r * kHashThreads;
-      if (k >= m) continue;
-      const uint64_t t = base + s_order[k];
+    for (int r = 0; r < kHashPer; ++r) {
+      if (tid + r * kHashThreads >= m) continue;
+      const uint64_t t = base + s_order[r == 0 ? tid : m - 1 - tid];
       uint64_t gi, i, j, seed_idx, zi;
       if (a.n_seg) {
         const uint32_t d = segment_of(a.seg_start, a.n_seg, t);
@@ -272,22 +287,23 @@ __global__ void __launch_bounds__(kHashThreads, MINB) k_hash(const HashArgs a) {
         if (a.s) acc_add<8>(acc_s, s);
       }
     }
-    __syncthreads();
+    group_sync<GROUPS>(g);
   }
-  // block reduction of the limb values as 64-bit sums
-  __shared__ unsigned long long red[kHashThreads / 32][kPartialWords];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // reduction of the group's limb values as 64-bit sums
+  __shared__ unsigned long long red_[GROUPS][kHashThreads / 32][kPartialWords];
+  unsigned long long (*red)[kPartialWords] = red_[g];
+  const int lane = threadIdx.x & 31, warp = tid >> 5;
 #pragma unroll
   for (int k = 0; k < kPartialWords; ++k) {
     unsigned long long v = k < 13 ? acc_e.v[k] : (k < 26 ? acc_s.v[k - 13] : bad);
     warp_sum_u64(v);
     if (lane == 0) red[warp][k] = v;
   }
-  __syncthreads();
-  if (threadIdx.x < kPartialWords) {
+  group_sync<GROUPS>(g);
+  if (tid < kPartialWords && group < a.ngroups) {
     unsigned long long v = 0;
-    for (int w = 0; w < kHashThreads / 32; ++w) v += red[w][threadIdx.x];
-    a.partial[(uint64_t)blockIdx.x * kPartialWords + threadIdx.x] = v;
+    for (int w = 0; w < kHashThreads / 32; ++w) v += red[w][tid];
+    a.partial[(uint64_t)group * kPartialWords + tid] = v;
   }
 }
 
@@ -647,13 +663,37 @@ void launch_epoch_seeds(int inst, unsigned grid, unsigned block, cudaStream_t st
   else k_epoch_seeds<kInstSha><<<grid, block, 0, st>>>(ds, nds, e0, ne, x0_out, status);
 }
 
-void launch_hash(int inst, unsigned grid, cudaStream_t st, const HashArgs& a, bool coresident) {
-  if (coresident) {
-    if (inst == kInstAes) k_hash<kInstAes, kCoresidentMinBlocks><<<grid, kHashThreads, 0, st>>>(a);
-    else k_hash<kInstSha, kCoresidentMinBlocks><<<grid, kHashThreads, 0, st>>>(a);
+// POSLO+ blocks hold the 128 KiB of tables, one block per SM: four groups (512 threads, all the
+// registers) when the hashing has the SMs to itself, two beside the decoding.
+constexpr int kAesGroupsAlone = 4, kAesGroupsBeside = 2;
+
+unsigned hash_groups(int inst, int sm_count, uint64_t n) {
+  const uint64_t need = (n + kHashThreads - 1) / kHashThreads;
+  const uint64_t cap = (uint64_t)sm_count * (inst == kInstAes ? kAesGroupsAlone : 8);
+  return (unsigned)(need < 1 ? 1 : need < cap ? need : cap);
+}
+
+cudaError_t hash_kernels_init() {
+  const cudaError_t e = cudaFuncSetAttribute(k_hash<kInstAes, 1, kAesGroupsAlone>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAesWideBytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_hash<kInstAes, 2, kAesGroupsBeside>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)kAesWideBytes);
+}
+
+void launch_hash(int inst, unsigned groups, cudaStream_t st, HashArgs a, HashPlace place) {
+  a.ngroups = groups;
+  if (inst == kInstAes) {
+    if (place == kHashAlone)
+      k_hash<kInstAes, 1, kAesGroupsAlone><<<(groups + kAesGroupsAlone - 1) / kAesGroupsAlone,
+                                             kHashThreads * kAesGroupsAlone, kAesWideBytes, st>>>(a);
+    else
+      k_hash<kInstAes, 2, kAesGroupsBeside><<<(groups + kAesGroupsBeside - 1) / kAesGroupsBeside,
+                                              kHashThreads * kAesGroupsBeside, kAesWideBytes, st>>>(a);
+  } else if (place == kHashCoresident) {
+    k_hash<kInstSha, kCoresidentMinBlocks, 1><<<groups, kHashThreads, 0, st>>>(a);
   } else {
-    if (inst == kInstAes) k_hash<kInstAes, POSLO_HASH_MIN_BLOCKS><<<grid, kHashThreads, 0, st>>>(a);
-    else k_hash<kInstSha, POSLO_HASH_MIN_BLOCKS><<<grid, kHashThreads, 0, st>>>(a);
+    k_hash<kInstSha, POSLO_HASH_MIN_BLOCKS, 1><<<groups, kHashThreads, 0, st>>>(a);
   }
 }
 

@@ -421,7 +421,7 @@ void make_zpre(const uint8_t vseed[32], uint32_t zpre[10]) {
 
 // Hash stage shared by AVer, Distill and the inspection call.
 int run_hash(poslo_ctx* ctx, const poslo_batch* b, const Staged& sb, uint8_t* e_out, bool weighted, bool with_s,
-             uint32_t* z_out, unsigned long long** partial_out, uint32_t* nblocks_out) {
+             uint32_t* z_out, unsigned long long** partial_out, uint32_t* nblocks_out, bool alone) {
   int rc;
   uint64_t e_first = 0, ne = 0;
   if (b->n) {
@@ -430,7 +430,7 @@ int run_hash(poslo_ctx* ctx, const poslo_batch* b, const Staged& sb, uint8_t* e_
   }
   uint32_t* seeds;
   if ((rc = run_epoch_seeds(ctx, b->ds, b->ds_nodes, e_first, ne, &seeds))) return rc;
-  const int blocks = grid_for(ctx, b->n, kHashThreads, 8);
+  const int blocks = (int)hash_groups((int)ctx->inst, ctx->sm_count, b->n);
   unsigned long long* partial;
   if ((rc = ensure_t(ctx, "hash_partial", (size_t)blocks * kPartialWords * 8, &partial))) return rc;
   HashArgs a{};
@@ -452,7 +452,7 @@ int run_hash(poslo_ctx* ctx, const poslo_batch* b, const Staged& sb, uint8_t* e_
   a.status = ctx->status;
   cudaEvent_t tb, te;
   timer_begin(ctx, "hash", ctx->s_main, &tb, &te);
-  launch_hash((int)ctx->inst, (unsigned)blocks, ctx->s_main, a);
+  launch_hash((int)ctx->inst, (unsigned)blocks, ctx->s_main, a, alone ? kHashAlone : kHashBeside);
   ++ctx->launch_count;
   CU(cudaGetLastError());
   timer_end(ctx, "hash", ctx->s_main, tb, te);
@@ -991,6 +991,7 @@ int poslo_create(const poslo_params* params, poslo_ctx** out) {
       cudaEventCreateWithFlags(&ctx->ev_prep, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&ctx->ev_staged, cudaEventDisableTiming) != cudaSuccess)
     return bail(POSLO_EDEVICE);
+  if (hash_kernels_init() != cudaSuccess) return bail(POSLO_EDEVICE);
   if (cudaMalloc(&ctx->status, 4) != cudaSuccess) return bail(POSLO_ENOMEM);
   // page-locked: the status word, then kSmallHostBytes for small results and records
   if (cudaMallocHost(&ctx->h_status, 256 + kSmallHostBytes) != cudaSuccess) return bail(POSLO_ENOMEM);
@@ -1386,7 +1387,7 @@ int poslo_hash_entries(poslo_ctx* ctx, const poslo_batch* batch, uint8_t* e_out)
   if (!batch->on_device && (rc = ensure_t(ctx, "e_out", 32 * batch->n, &d_e))) return rc;
   unsigned long long* partial;
   uint32_t nb;
-  if ((rc = run_hash(ctx, batch, sb, d_e, false, false, nullptr, &partial, &nb))) return rc;
+  if ((rc = run_hash(ctx, batch, sb, d_e, false, false, nullptr, &partial, &nb, true))) return rc;
   if (!batch->on_device && batch->n)
     CU(cudaMemcpyAsync(e_out, d_e, 32 * batch->n, cudaMemcpyDeviceToHost, ctx->s_main));
   return check_status(ctx);
@@ -1433,7 +1434,7 @@ int poslo_aver(poslo_ctx* ctx, const poslo_batch* batch, uint32_t agg_mode, uint
   if (weighted && (rc = ensure_t(ctx, "z", 16 * std::max<uint64_t>(batch->n, 1), &z))) return rc;
   unsigned long long* hpart;
   uint32_t nhb;
-  if ((rc = run_hash(ctx, batch, sb, nullptr, weighted, F, z, &hpart, &nhb))) return rc;
+  if ((rc = run_hash(ctx, batch, sb, nullptr, weighted, F, z, &hpart, &nhb, !F))) return rc;
   if ((rc = run_prep(ctx, hpart, nhb, F ? nullptr : sb.s, tableY, prep, nullptr, 0, nullptr))) return rc;
   if (weighted) {
     MsmState ms;
@@ -1494,7 +1495,7 @@ int poslo_aver_partial(poslo_ctx* ctx, const poslo_batch* batch, uint32_t agg_mo
   if ((rc = ensure_t(ctx, "partial_small", 4 * (65 + (size_t)kShardWords), &small))) return rc;
   uint32_t *unitR = small, *Rw = small + 32, *pbad = small + 64, *rec = small + 65;
   if ((rc = ensure_t(ctx, "seeds", std::max<uint64_t>(1, ne) * 16, &seeds))) return rc;
-  const uint32_t nhb = (uint32_t)grid_for(ctx, n, kHashThreads, 8);
+  const uint32_t nhb = hash_groups((int)ctx->inst, ctx->sm_count, n);
   unsigned long long* hpart;
   if ((rc = ensure_t(ctx, "hash_partial", (size_t)nhb * kPartialWords * 8, &hpart))) return rc;
   const bool replayable = batch->on_device != 0 || sb.packed;
@@ -1534,7 +1535,7 @@ int poslo_aver_partial(poslo_ctx* ctx, const poslo_batch* batch, uint32_t agg_mo
     cudaEvent_t tb, te;
     if (!weighted) {
       timer_begin(ctx, "hash", ctx->s_main, &tb, &te);
-      launch_hash((int)ctx->inst, nhb, ctx->s_main, a);
+      launch_hash((int)ctx->inst, nhb, ctx->s_main, a, F ? kHashBeside : kHashAlone);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", ctx->s_main, tb, te);
@@ -1551,7 +1552,7 @@ int poslo_aver_partial(poslo_ctx* ctx, const poslo_batch* batch, uint32_t agg_mo
       MsmState ms;
       if ((rc = run_msm_sort(ctx, ctx->s_main, z, 4, nullptr, n, ms))) return rc;
       timer_begin(ctx, "hash", ctx->s_hash, &tb, &te);
-      launch_hash((int)ctx->inst, nhb, ctx->s_hash, a);
+      launch_hash((int)ctx->inst, nhb, ctx->s_hash, a, kHashBeside);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", ctx->s_hash, tb, te);
@@ -1712,8 +1713,8 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
   uint32_t *pts, *z, *small, *seeds;
   uint8_t *badR, *badS, *d_e, *inv, *d_ccd, *d_acc;
   unsigned long long *hpart, *sp;
-  const int hblocks = grid_for(ctx, n, kHashThreads, 8);
-  const int sblocks = hblocks;
+  const int hblocks = (int)hash_groups((int)ctx->inst, ctx->sm_count, n);
+  const int sblocks = grid_for(ctx, n, kHashThreads, 8);
   if ((rc = ensure_t(ctx, "pts", 4 * kPtsWords * n1, &pts))) return rc;
   if ((rc = ensure_t(ctx, "badR", n1, &badR))) return rc;
   if ((rc = ensure_t(ctx, "badS", n1, &badS))) return rc;
@@ -1800,7 +1801,7 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     {
       cudaEvent_t tb, te;
       timer_begin(ctx, "hash", hs, &tb, &te);
-      launch_hash((int)ctx->inst, (unsigned)hblocks, hs, a);
+      launch_hash((int)ctx->inst, (unsigned)hblocks, hs, a, kHashBeside);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", hs, tb, te);
@@ -2307,7 +2308,7 @@ int ccd_common(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrella, St
   if ((rc = ensure_t(ctx, "ccd_esum", 32 * n1, esum))) return rc;
   unsigned long long* hpart;
   uint32_t nhb;
-  if ((rc = run_hash(ctx, batch, sb, d_e, false, false, nullptr, &hpart, &nhb))) return rc;
+  if ((rc = run_hash(ctx, batch, sb, d_e, false, false, nullptr, &hpart, &nhb, true))) return rc;
   k_scalar_group_sums<<<(unsigned)n1, kCcdThreads, 0, ctx->s_main>>>(d_e, batch->n2, batch->n, nullptr,
                                                                       reinterpret_cast<uint32_t*>(*esum));
   ++ctx->launch_count;
@@ -2905,7 +2906,7 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
     CU(cudaEventRecord(ctx->ev_main, ctx->s_main));
     CU(cudaStreamWaitEvent(ctx->s_hash, ctx->ev_main, 0));
     {
-      const int blocks = grid_for(ctx, N, kHashThreads, 8);
+      const int blocks = (int)hash_groups((int)ctx->inst, ctx->sm_count, N);
       unsigned long long* hpart;
       if ((rc = ensure_t(ctx, "hash_partial", (size_t)blocks * kPartialWords * 8, &hpart))) return rc;
       HashArgs a{};
@@ -2932,7 +2933,7 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
       a.seg_n2 = d_n2;
       cudaEvent_t tb, te;
       timer_begin(ctx, "hash", ctx->s_hash, &tb, &te);
-      launch_hash((int)ctx->inst, (unsigned)blocks, ctx->s_hash, a, true);
+      launch_hash((int)ctx->inst, (unsigned)blocks, ctx->s_hash, a, kHashCoresident);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", ctx->s_hash, tb, te);
