@@ -8,7 +8,7 @@
 //                   aggregates sum e_t, sum s_t (or their weighted forms)
 //   k_points        strict decoding of R_t and the unit aggregate sum R_t
 //   k_table_*       fixed-window tables {d 16^w P : d = 1..8, w = 0..63} for the check
-//   k_finalize      reduce the partial aggregates and evaluate [8](R - eY - sG) = O
+//   k_final_prep, k_final_check  reduce the partial aggregates and evaluate [8](R - eY - sG) = O
 #pragma once
 #include <cstdint>
 
@@ -291,23 +291,6 @@ __device__ __forceinline__ ge table_pick(const uint32_t* table, int w, int d) {
   const ge p = ge_load(table + ((size_t)w * kTableDigits + (abs(d) - 1)) * 32);
   return d < 0 ? ge_neg(p) : p;
 }
-
-// ----------------------------------------------------------------------------------------
-// Combine the partial aggregates and evaluate the cofactored check.
-// ----------------------------------------------------------------------------------------
-struct FinalArgs {
-  const unsigned long long* hash_partial;   // nhash blocks * kPartialWords
-  uint32_t nhash;
-  const uint32_t* point_partial;            // npoint blocks * kPointPartialWords (unit R sum)
-  uint32_t npoint;
-  const uint32_t* R_given;                  // optional: an extended point (32 words) used as R
-  const uint8_t* s_given;                   // optional: aggregate s (C), 32 bytes
-  const uint32_t* tableY;
-  const uint32_t* tableG;
-  uint8_t* accept;                          // 1 byte
-  uint32_t* out_words;                      // optional: e~ (8), s~ (8), R (32) for inspection
-  uint32_t* status;
-};
 
 constexpr int kFinalThreads = 256;
 
@@ -709,7 +692,6 @@ __global__ void __launch_bounds__(128) k_table_chain(const uint32_t* __restrict_
                                                      uint32_t* __restrict__ status, int use_base,
                                                      uint8_t* __restrict__ bad_out);
 __global__ void __launch_bounds__(128) k_table_fill(uint32_t n, uint32_t* __restrict__ tables, uint32_t* const* dst);
-__global__ void __launch_bounds__(kFinalThreads) k_finalize(const FinalArgs a);
 __global__ void __launch_bounds__(128) k_final_prep(const PrepArgs a);
 __global__ void k_final_check(const uint32_t* prep, const uint32_t* R, const uint32_t* point_bad,
                               const uint32_t* status, uint8_t* accept);
@@ -873,8 +855,8 @@ __global__ void k_segment_any(const uint8_t* inv, const uint64_t* seg_start, con
 constexpr int kCcdThreads = 128;
 __global__ void __launch_bounds__(kCcdThreads) k_scalar_group_sums(const uint8_t* x, uint64_t G, uint64_t n,
                                                                    const uint8_t* skip, uint32_t* out);
-__global__ void __launch_bounds__(kCcdThreads) k_point_group_sums(const uint32_t* pts, const uint8_t* bad, uint64_t G,
-                                                                  uint64_t n, const uint8_t* skip, uint8_t* enc);
+void launch_point_group_sums(unsigned groups, cudaStream_t st, const uint32_t* pts, const uint8_t* bad, uint64_t G,
+                             uint64_t n, const uint8_t* skip, uint8_t* enc, uint32_t* partial);
 __global__ void __launch_bounds__(128) k_check_list(const uint32_t* e, const uint8_t* s, const uint32_t* pts,
                                                     const uint8_t* bad, uint32_t n, const uint32_t* tableY,
                                                     const uint32_t* tableG, uint8_t* ok);

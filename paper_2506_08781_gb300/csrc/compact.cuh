@@ -29,51 +29,9 @@ static __device__ __noinline__ ge add(const ge& p, const ge& q) {
   return r;
 }
 
-// Doubling (dbl-2008-hwcd, a = -1), as ge_dbl.
-static __device__ __noinline__ ge dbl(const ge& p) {
-  const fe A = sq(p.X);
-  const fe B = sq(p.Y);
-  const fe Z2 = sq(p.Z);
-  const fe C = fe_add(Z2, Z2);
-  const fe E = fe_sub(fe_sub(sq(fe_add(p.X, p.Y)), A), B);
-  const fe G = fe_sub(B, A);
-  const fe F = fe_sub(G, C);
-  const fe H = fe_neg(fe_add(A, B));
-  ge r;
-  r.X = mul(E, F);
-  r.Y = mul(G, H);
-  r.Z = mul(F, G);
-  r.T = mul(E, H);
-  return r;
-}
-
-static __device__ __forceinline__ ge sub(const ge& p, const ge& q) { return add(p, ge_neg(q)); }
-
-static __device__ __noinline__ fe sqn(fe a, int n) {
-#pragma unroll 1
-  for (int i = 0; i < n; ++i) a = sq(a);
-  return a;
-}
-
-// z^(p-2), Fermat's inverse (0 -> 0), by the addition chain of fe_inv.
-static __device__ __noinline__ fe inv(const fe& z) {
-  const fe z2 = sq(z);
-  const fe z9 = mul(sqn(z2, 2), z);
-  const fe z11 = mul(z9, z2);
-  const fe z_5 = mul(sq(z11), z9);                 // 2^5 - 1
-  const fe z_10 = mul(sqn(z_5, 5), z_5);           // 2^10 - 1
-  const fe z_20 = mul(sqn(z_10, 10), z_10);        // 2^20 - 1
-  const fe z_40 = mul(sqn(z_20, 20), z_20);        // 2^40 - 1
-  const fe z_50 = mul(sqn(z_40, 10), z_10);        // 2^50 - 1
-  const fe z_100 = mul(sqn(z_50, 50), z_50);       // 2^100 - 1
-  const fe z_200 = mul(sqn(z_100, 100), z_100);    // 2^200 - 1
-  const fe z_250 = mul(sqn(z_200, 50), z_50);      // 2^250 - 1
-  return mul(sqn(z_250, 5), z11);
-}
-
 // The compressed encoding (y with the parity of x in bit 255), as ge_encode.
 static __device__ __noinline__ void encode(const ge& p, uint32_t b[8]) {
-  const fe zi = inv(p.Z);
+  const fe zi = fe_inv(p.Z);
   const fe x = canon(mul(p.X, zi));
   const fe y = canon(mul(p.Y, zi));
 #pragma unroll
@@ -81,31 +39,35 @@ static __device__ __noinline__ void encode(const ge& p, uint32_t b[8]) {
   b[7] |= (x.v[0] & 1u) << 31;
 }
 
-static __device__ __forceinline__ ge mul_cofactor(ge p) {
-#pragma unroll 1
-  for (int i = 0; i < 3; ++i) p = dbl(p);
-  return p;
-}
-
-// The sum of the 128 points terms[0..127] (32 words each, in shared memory) by a block of
-// 128 threads: quad q adds terms 4q .. 4q + 3 (quad-cooperative additions), then a tree over
-// the 32 quads' sums in qs; the sum ends in qs[0].  Every thread calls it (full-mask
-// shuffles, barriers inside); the caller has stored the terms and synchronised.
-__device__ __forceinline__ void quad_sum128(uint32_t (*terms)[32], uint32_t (*qs)[32]) {
-  constexpr int kQuads = 32;
-  const int tid = threadIdx.x, quad = tid >> 2;
-  ge acc = ge_identity();
-#pragma unroll 1
-  for (int k = 0; k < 4; ++k) acc = ge_add_quad(acc, ge_load(terms[4 * quad + k]));
-  if ((tid & 3) == 0) ge_store(qs[quad], acc);
+// The sum of the n points sp[0 .. n) (32 words each, shared memory, n >= 1) into sp[0] by the
+// block's quads, one quad-cooperative addition per pair and level: about 2,200 cycles a level
+// where one lane's addition takes 6,000.  Every thread of the block calls it (full-mask
+// shuffles, barriers inside; blockDim.x a multiple of 32); the caller has stored the points.
+static __device__ __noinline__ void quad_tree(uint32_t (*sp)[32], int n) {
+  const int quad = threadIdx.x >> 2, nq = blockDim.x >> 2;
+  const bool writer = (threadIdx.x & 3) == 0;
   __syncthreads();
 #pragma unroll 1
-  for (int h = kQuads / 2; h > 0; h >>= 1) {
-    const ge sum = ge_add_quad(ge_load(qs[quad]), ge_load(qs[(quad + h) % kQuads]));
+  while (n > 1) {
+    const int half = (n + 1) >> 1, pairs = n - half;   // sp[k] += sp[k + half]
+#pragma unroll 1
+    for (int k0 = 0; k0 < pairs; k0 += nq) {
+      const int k = k0 + quad, c = k < pairs ? k : pairs - 1;   // surplus quads repeat the last pair, unwritten
+      const ge sum = ge_add_quad(ge_load(sp[c]), ge_load(sp[c + half]));
+      __syncthreads();
+      if (writer && k < pairs) ge_store(sp[k], sum);
+    }
     __syncthreads();
-    if ((tid & 3) == 0 && quad < h) ge_store(qs[quad], sum);
-    __syncthreads();
+    n = half;
   }
+}
+
+// [8](a - b) = O by the quads of one warp (every lane calls it with the same points).
+static __device__ __noinline__ bool quad_equal(const ge& a, const ge& b) {
+  ge d = ge_add_quad(a, ge_neg(b));
+#pragma unroll 1
+  for (int i = 0; i < 3; ++i) d = ge_dbl_quad(d);
+  return ge_is_identity(d);
 }
 
 }  // namespace compact

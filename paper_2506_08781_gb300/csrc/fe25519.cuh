@@ -408,37 +408,130 @@ __device__ __forceinline__ fe fe_select(const fe& a, const fe& b, bool pick_b) {
   return r;
 }
 
-// z^(2^250 - 1) and z^11 share one addition chain (z^2, z^9, z^11, then runs of squarings
-// building z^(2^k - 1) for k = 5, 10, 20, 40, 50, 100, 200, 250).
-__device__ __forceinline__ fe fe_pow_2_250_1(const fe& z, fe* z11_out) {
-  const fe z2 = fe_sq(z);
-  const fe z8 = fe_sqn(z2, 2);
-  const fe z9 = fe_mul(z8, z);
-  const fe z11 = fe_mul(z9, z2);
-  const fe z22 = fe_sq(z11);
-  const fe z_5 = fe_mul(z22, z9);                 // 2^5 - 1
-  const fe z_10 = fe_mul(fe_sqn(z_5, 5), z_5);     // 2^10 - 1
-  const fe z_20 = fe_mul(fe_sqn(z_10, 10), z_10);  // 2^20 - 1
-  const fe z_40 = fe_mul(fe_sqn(z_20, 20), z_20);  // 2^40 - 1
-  const fe z_50 = fe_mul(fe_sqn(z_40, 10), z_10);  // 2^50 - 1
-  const fe z_100 = fe_mul(fe_sqn(z_50, 50), z_50); // 2^100 - 1
-  const fe z_200 = fe_mul(fe_sqn(z_100, 100), z_100);
-  const fe z_250 = fe_mul(fe_sqn(z_200, 50), z_50);
-  if (z11_out) *z11_out = z11;
-  return z_250;
-}
-
-// z^(p-2) = z^(2^255 - 21) = (z^(2^250-1))^(2^5) * z^11  (Fermat inverse; 0 -> 0).
-__device__ __forceinline__ fe fe_inv(const fe& z) {
-  fe z11;
-  const fe t = fe_pow_2_250_1(z, &z11);
-  return fe_mul(fe_sqn(t, 5), z11);
-}
-
-// z^((p-5)/8) = z^(2^252 - 3) = (z^(2^250-1))^4 * z.
+// z^((p-5)/8) = z^(2^252 - 3) by the chain z^2, z^9, z^11, z^(2^5 - 1), then eight stages of
+// "n squarings, one product": exponents 2^k - 1 for k = 10, 20, 40, 50, 100, 200, 250 and last
+// 2^252 - 3.  A stage multiplies by the value it started from, by z^(2^10 - 1) (to reach 50), by
+// z^(2^50 - 1) (250) or by z (last).  One loop instead of a call per stage: the decoding runs as
+// one copy each of the squaring and the product (a few KB of code instead of 48), which a
+// launch of few points fetches from a cold instruction cache.
 __device__ __forceinline__ fe fe_pow_p58(const fe& z) {
-  const fe t = fe_pow_2_250_1(z, nullptr);
-  return fe_mul(fe_sqn(t, 2), z);
+  const fe z2 = fe_sq(z);
+  const fe z9 = fe_mul(fe_sqn(z2, 2), z);
+  fe cur = fe_mul(fe_sq(fe_mul(z9, z2)), z9);   // 2^5 - 1
+  fe z10 = cur, z50 = cur;
+#pragma unroll 1
+  for (int k = 0; k < 8; ++k) {
+    // squarings of the stages: 5, 10, 20, 10, 50, 100, 50, 2 (one byte each)
+    const int n = (int)(0x023264320a140a05ull >> (8 * k) & 0xff);
+    fe m = fe_select(cur, z10, k == 3);
+    m = fe_select(m, z50, k == 6);
+    m = fe_select(m, z, k == 7);
+    cur = fe_mul(fe_sqn(cur, n), m);
+    z10 = fe_select(z10, cur, k == 0);
+    z50 = fe_select(z50, cur, k == 3);
+  }
+  return cur;
+}
+
+// z^-1 mod p (0 -> 0) by division steps (D. J. Bernstein, B.-Y. Yang, "Fast constant-time gcd
+// computation and modular inversion", TCHES 2019): from (delta, f, g) = (1, p, z), a step is
+//   (1 - delta, g, (g - f) / 2)        if delta > 0 and g is odd,
+//   (1 + delta, f, (g + (g mod 2) f) / 2)  otherwise,
+// and after at most (49 * 255 + 57) / 17 < 741 of them g = 0 and f = +-1.  The steps look only
+// at the low bits, so 30 at a time run on one word each of f and g and are collected in a
+// matrix (u v; q r) of entries at most 2^30, which then moves f, g (exactly) and the
+// coefficients d, e with d z = f, e z = g (mod p): (u d + v e + m p) / 2^30, with m chosen to
+// make the division exact.  Numbers are nine signed limbs of 30 bits; in them p is 2^15 at limb
+// 8 and -19 at limb 0.  |m| <= 2^29, so d and e grow by at most p / 2 a batch.
+// One thread's chain: about 20 batches of some 1,500 cycles, where the 255 squarings and 11
+// products of z^(p-2) took 95,000 cycles.
+static __device__ __noinline__ fe fe_inv(const fe& z) {
+  constexpr int32_t M = (1 << 30) - 1;
+  constexpr uint32_t kInv19 = 678152731u;   // 19^-1 mod 2^30
+  static_assert(((uint64_t)kInv19 * 19u & (uint32_t)M) == 1u, "inverse of 19 mod 2^30");
+  const fe a = fe_canon(z);
+  int32_t f[9], g[9], d[9], e[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    f[k] = M;
+    d[k] = 0;
+    e[k] = 0;
+    // bits 30k .. 30k + 29 of a: word k - 1 or k on, offset 30k mod 32
+    const int w = (30 * k) >> 5, o = (30 * k) & 31;
+    const uint32_t hi = w + 1 < 8 ? a.v[w + 1] : 0u;
+    g[k] = (int32_t)(__funnelshift_r(a.v[w], hi, o) & (uint32_t)M);
+  }
+  f[0] = M + 1 - 19;
+  f[8] = 0x7fff;
+  e[0] = 1;
+  int32_t delta = 1;
+#pragma unroll 1
+  for (int batch = 0; batch < 25; ++batch) {
+    uint32_t any = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) any |= (uint32_t)g[k];
+    if (any == 0) break;
+    uint32_t f0 = (uint32_t)f[0] | (uint32_t)f[1] << 30, g0 = (uint32_t)g[0] | (uint32_t)g[1] << 30;
+    int32_t u = 1, v = 0, q = 0, r = 1;
+#pragma unroll 6
+    for (int i = 0; i < 30; ++i) {
+      const int32_t odd = -(int32_t)(g0 & 1u);
+      const bool swap = odd != 0 && delta > 0;
+      const uint32_t tf = swap ? 0u - f0 : f0;
+      const int32_t tu = swap ? -u : u, tv = swap ? -v : v;
+      f0 = swap ? g0 : f0;
+      u = (swap ? q : u) << 1;
+      v = (swap ? r : v) << 1;
+      g0 = (g0 + (tf & (uint32_t)odd)) >> 1;
+      q += tu & odd;
+      r += tv & odd;
+      delta = (swap ? -delta : delta) + 1;
+    }
+    int64_t cf = (int64_t)u * f[0] + (int64_t)v * g[0], cg = (int64_t)q * f[0] + (int64_t)r * g[0];
+    int64_t cd = (int64_t)u * d[0] + (int64_t)v * e[0], ce = (int64_t)q * d[0] + (int64_t)r * e[0];
+    // m = cd / 19 mod 2^30 as a signed 30-bit number: cd - 19 m = 0 mod 2^30
+    const int32_t md = (int32_t)((uint32_t)cd * kInv19 << 2) >> 2, me = (int32_t)((uint32_t)ce * kInv19 << 2) >> 2;
+    cd -= (int64_t)19 * md;
+    ce -= (int64_t)19 * me;
+    cf >>= 30; cg >>= 30; cd >>= 30; ce >>= 30;
+#pragma unroll
+    for (int k = 1; k < 9; ++k) {
+      cf += (int64_t)u * f[k] + (int64_t)v * g[k];
+      cg += (int64_t)q * f[k] + (int64_t)r * g[k];
+      cd += (int64_t)u * d[k] + (int64_t)v * e[k];
+      ce += (int64_t)q * d[k] + (int64_t)r * e[k];
+      if (k == 8) {
+        cd += (int64_t)md << 15;
+        ce += (int64_t)me << 15;
+      }
+      f[k - 1] = (int32_t)cf & M; g[k - 1] = (int32_t)cg & M;
+      d[k - 1] = (int32_t)cd & M; e[k - 1] = (int32_t)ce & M;
+      cf >>= 30; cg >>= 30; cd >>= 30; ce >>= 30;
+    }
+    f[8] = (int32_t)cf; g[8] = (int32_t)cg; d[8] = (int32_t)cd; e[8] = (int32_t)ce;
+  }
+  // +-d + 16 p (|d| <= 13 p), carried into non-negative limbs below 2^260
+  const bool neg = f[8] < 0;
+  int32_t c = -16 * 19;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    c += (neg ? -d[k] : d[k]) + (k == 8 ? 1 << 19 : 0);
+    d[k] = k < 8 ? c & M : c;
+    c >>= 30;
+  }
+  fe x;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) x.v[k] = (uint32_t)d[k] >> (2 * k) | (uint32_t)d[k + 1] << (30 - 2 * k);
+  // 2^255 = 19 for the bits above
+  uint32_t cc = 19u * ((uint32_t)d[8] >> 15);
+  x.v[7] &= 0x7fffffffu;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const uint64_t t = (uint64_t)x.v[k] + cc;
+    x.v[k] = (uint32_t)t;
+    cc = (uint32_t)(t >> 32);
+  }
+  return x;
 }
 
 __device__ __forceinline__ uint32_t fe_parity(const fe& a) { return fe_canon(a).v[0] & 1u; }

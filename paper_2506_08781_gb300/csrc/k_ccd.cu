@@ -3,6 +3,7 @@
 // and a list of independent cofactored checks [8](R_k - e_k Y - s_k G) = O (the per-epoch
 // C.AVer of Distill and the checks of SeBVer).
 #include "common.cuh"
+#include "compact.cuh"
 
 namespace poslo {
 
@@ -43,30 +44,40 @@ __global__ void __launch_bounds__(kCcdThreads) k_scalar_group_sums(const uint8_t
 }
 
 // enc[g] = encoding of the sum of the decoded points pts[g G .. (g+1) G) that are neither
-// flagged in skip nor undecodable (bad).  One block per group.
-__global__ void __launch_bounds__(kCcdThreads) k_point_group_sums(const uint32_t* pts, const uint8_t* bad, uint64_t G,
-                                                                  uint64_t n, const uint8_t* skip, uint8_t* enc) {
+// flagged in skip nor undecodable (bad), and the sum itself in the decoding's partial format
+// (kPointPartialWords, bad count 0), so that the sum over all groups needs no second pass over
+// the points.  One block of T threads per group: latency-bound, G / T additions of a lane, a
+// tree by quads and one inversion (64 groups of 64 points: 74 -> 35 us; all 4,096 points in one
+// block before: 177 us).
+template <int T>
+__global__ void __launch_bounds__(T) k_point_group_sums(const uint32_t* pts, const uint8_t* bad, uint64_t G,
+                                                        uint64_t n, const uint8_t* skip, uint8_t* enc,
+                                                        uint32_t* partial) {
   const uint64_t g = blockIdx.x;
   ge acc = ge_identity();
   const uint64_t lo = g * G, hi = min(lo + G, n);
-  for (uint64_t t = lo + threadIdx.x; t < hi; t += blockDim.x) {
+  for (uint64_t t = lo + threadIdx.x; t < hi; t += T) {
     if ((skip && skip[t]) || (bad && bad[t])) continue;
     fe x, y, t2d;
     pts_load(pts + (size_t)kPtsWords * t, x, y, t2d);
     acc = ge_madd(acc, x, y, t2d);
   }
-  __shared__ uint32_t sp[kCcdThreads][32];
+  __shared__ uint32_t sp[T][32];
   ge_store(sp[threadIdx.x], acc);
-  __syncthreads();
-  for (int h = kCcdThreads / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) ge_store(sp[threadIdx.x], ge_add(ge_load(sp[threadIdx.x]), ge_load(sp[threadIdx.x + h])));
-    __syncthreads();
-  }
+  compact::quad_tree(sp, G < T ? (int)G : T);
+  if (threadIdx.x < 32) partial[kPointPartialWords * g + threadIdx.x] = sp[0][threadIdx.x];
   if (threadIdx.x == 0) {
+    partial[kPointPartialWords * g + 32] = 0;
     uint32_t b[8];
-    ge_encode(ge_load(sp[0]), b);
+    compact::encode(ge_load(sp[0]), b);
     for (int k = 0; k < 8; ++k) reinterpret_cast<uint32_t*>(enc + 32 * g)[k] = b[k];
   }
+}
+
+void launch_point_group_sums(unsigned groups, cudaStream_t st, const uint32_t* pts, const uint8_t* bad, uint64_t G,
+                             uint64_t n, const uint8_t* skip, uint8_t* enc, uint32_t* partial) {
+  if (G > 128) k_point_group_sums<256><<<groups, 256, 0, st>>>(pts, bad, G, n, skip, enc, partial);
+  else k_point_group_sums<128><<<groups, 128, 0, st>>>(pts, bad, G, n, skip, enc, partial);
 }
 
 // ok[k] = s_k canonical, R_k decodable (not bad), and [8](R_k - e_k Y - s_k G) = O, for n

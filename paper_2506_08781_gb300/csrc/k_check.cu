@@ -89,25 +89,26 @@ __global__ void k_sum_encode(const uint32_t* partial, uint32_t nparts, uint32_t*
                              uint32_t* bad_out) {
   __shared__ uint32_t sp[kFinalThreads][32];
   __shared__ uint32_t sbad;
-  const int tid = threadIdx.x;
+  const uint32_t tid = threadIdx.x;
   if (tid == 0) sbad = 0;
   __syncthreads();
-  // once per call: compact (out-of-line) point operations, the code being fetched cold
+  // once per call: compact (out-of-line) point operations, the code being fetched cold; the
+  // partials summed by quads (2^20 entries, 456 partials and the encoding: 124 -> 45 us, one
+  // partial without an encoding: 47 -> 4 us)
   ge acc = ge_identity();
   uint32_t bad = 0;
+  if (tid < nparts) {
+    acc = ge_load(partial + (size_t)tid * kPointPartialWords);
+    bad = partial[(size_t)tid * kPointPartialWords + 32];
+  }
 #pragma unroll 1
-  for (uint32_t b = tid; b < nparts; b += kFinalThreads) {
+  for (uint32_t b = tid + kFinalThreads; b < nparts; b += kFinalThreads) {
     acc = compact::add(acc, ge_load(partial + (size_t)b * kPointPartialWords));
     bad += partial[(size_t)b * kPointPartialWords + 32];
   }
   ge_store(sp[tid], acc);
-  atomicAdd(&sbad, bad);
-  __syncthreads();
-#pragma unroll 1
-  for (int h = kFinalThreads / 2; h > 0; h >>= 1) {
-    if (tid < h) ge_store(sp[tid], compact::add(ge_load(sp[tid]), ge_load(sp[tid + h])));
-    __syncthreads();
-  }
+  if (bad) atomicAdd(&sbad, bad);
+  compact::quad_tree(sp, nparts < 1 ? 1 : nparts < kFinalThreads ? (int)nparts : kFinalThreads);
   if (tid == 0) {
     const ge r = ge_load(sp[0]);
     if (point_out) ge_store(point_out, r);

@@ -4,6 +4,7 @@
 // stage is one launch for all devices, and one random linear combination checks them all
 // at once: sum_t z_t R_t - sum_d (sum_{t in d} z_t e_t) Y_d - (sum_t z_t s_t) G = O.
 #include "common.cuh"
+#include "compact.cuh"
 
 namespace poslo {
 
@@ -70,17 +71,6 @@ namespace {
 
 __device__ __forceinline__ uint64_t seg_pieces(uint64_t n) { return n == 0 ? 1 : (n + kSegPiece - 1) / kSegPiece; }
 
-// The shared-memory tree over the block's points (one per thread of kThreads); the sum ends
-// in sp_[0].
-template <int kThreads = kSegThreads>
-__device__ __forceinline__ void seg_point_tree(uint32_t (*sp_)[32]) {
-  __syncthreads();
-  for (int h = kThreads / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) ge_store(sp_[threadIdx.x], ge_add(ge_load(sp_[threadIdx.x]), ge_load(sp_[threadIdx.x + h])));
-    __syncthreads();
-  }
-}
-
 // Device d's results from its exact limb sums (four 13-limb sums, then the bad count) and
 // its point sum R (32 words): the scalars reduced mod q.  kPart selects what is written.
 template <int kPart>
@@ -130,7 +120,7 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) k_segment_sums(const
       acc = ge_madd(acc, x, y, t2d);
     }
     ge_store(sp_[threadIdx.x], acc);
-    seg_point_tree<kThreads>(sp_);
+    compact::quad_tree(sp_, hi - lo < kThreads ? max((int)(hi - lo), 1) : kThreads);
     if (!whole) {
       if (threadIdx.x < 32) piece_R[32 * (size_t)blockIdx.x + threadIdx.x] = sp_[0][threadIdx.x];
       return;
@@ -219,7 +209,7 @@ __global__ void __launch_bounds__(kSegThreads) k_segment_combine(const uint64_t*
   for (uint64_t j = threadIdx.x; j < np; j += blockDim.x) acc = ge_add(acc, ge_load(piece_R + 32 * (p0 + j)));
   __shared__ uint32_t sp_[kSegThreads][32];
   ge_store(sp_[threadIdx.x], acc);
-  seg_point_tree(sp_);
+  compact::quad_tree(sp_, np < kSegThreads ? (int)np : kSegThreads);
   seg_write<kSegScalars | kSegPoints>(tot, sp_[0], d, out);
 }
 
@@ -304,16 +294,12 @@ __global__ void __launch_bounds__(kFinalThreads) k_multi_window_check(const uint
   __syncthreads();
   ge term = threadIdx.x < kTableWindows ? table_pick(tableG, threadIdx.x, dig[threadIdx.x]) : ge_identity();
   ge_store(pts_[threadIdx.x], term);
-  __syncthreads();
-  for (int h = kTableWindows / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) ge_store(pts_[threadIdx.x], ge_add(ge_load(pts_[threadIdx.x]), ge_load(pts_[threadIdx.x + h])));
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
+  compact::quad_tree(pts_, kTableWindows);
+  if (threadIdx.x < 32) {
     ge p1 = ge_load(W + 32 * (size_t)w);
-    if (Wsub) p1 = ge_sub(p1, ge_load(Wsub + 32 * (size_t)w));
-    const ge diff = ge_sub(ge_sub(p1, ge_load(P2w + 32 * (size_t)w)), ge_load(pts_[0]));
-    if (!ge_is_identity(ge_mul_cofactor(diff))) accept[0] = 0;
+    if (Wsub) p1 = ge_add_quad(p1, ge_neg(ge_load(Wsub + 32 * (size_t)w)));
+    const bool ok = compact::quad_equal(ge_add_quad(p1, ge_neg(ge_load(P2w + 32 * (size_t)w))), ge_load(pts_[0]));
+    if (threadIdx.x == 0 && !ok) accept[0] = 0;
   }
 }
 
@@ -339,11 +325,7 @@ __global__ void __launch_bounds__(kPointThreads) k_table_msm_windows(const uint3
   }
   __shared__ uint32_t sp[kPointThreads][32];
   ge_store(sp[threadIdx.x], acc);
-  __syncthreads();
-  for (int h = kPointThreads / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) ge_store(sp[threadIdx.x], ge_add(ge_load(sp[threadIdx.x]), ge_load(sp[threadIdx.x + h])));
-    __syncthreads();
-  }
+  compact::quad_tree(sp, kPointThreads);
   const size_t o = ((size_t)win * gridDim.x + blockIdx.x) * kPointPartialWords;
   if (threadIdx.x < 32) partial[o + threadIdx.x] = sp[0][threadIdx.x];
   if (threadIdx.x == 0) partial[o + 32] = 0;
@@ -358,11 +340,7 @@ __global__ void __launch_bounds__(kPointThreads) k_window_point_sums(const uint3
     acc = ge_add(acc, ge_load(partial + ((size_t)w * nblocks + b) * kPointPartialWords));
   __shared__ uint32_t sp[kPointThreads][32];
   ge_store(sp[threadIdx.x], acc);
-  __syncthreads();
-  for (int h = kPointThreads / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) ge_store(sp[threadIdx.x], ge_add(ge_load(sp[threadIdx.x]), ge_load(sp[threadIdx.x + h])));
-    __syncthreads();
-  }
+  compact::quad_tree(sp, kPointThreads);
   if (threadIdx.x < 32) out[32 * (size_t)w + threadIdx.x] = sp[0][threadIdx.x];
 }
 
@@ -401,16 +379,12 @@ __global__ void __launch_bounds__(kFinalThreads) k_multi_check(const uint32_t* P
   __syncthreads();
   ge term = threadIdx.x < kTableWindows ? table_pick(tableG, threadIdx.x, dig[threadIdx.x]) : ge_identity();
   ge_store(pts_[threadIdx.x], term);
-  __syncthreads();
-  for (int h = kTableWindows / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) ge_store(pts_[threadIdx.x], ge_add(ge_load(pts_[threadIdx.x]), ge_load(pts_[threadIdx.x + h])));
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
+  compact::quad_tree(pts_, kTableWindows);
+  if (threadIdx.x < 32) {
     ge p1 = ge_load(P1);
-    if (P1sub) p1 = ge_sub(p1, ge_load(P1sub));
-    const ge diff = ge_sub(ge_sub(p1, ge_load(P2)), ge_load(pts_[0]));
-    accept[0] = ge_is_identity(ge_mul_cofactor(diff)) ? 1 : 0;
+    if (P1sub) p1 = ge_add_quad(p1, ge_neg(ge_load(P1sub)));
+    const bool ok = compact::quad_equal(ge_add_quad(p1, ge_neg(ge_load(P2))), ge_load(pts_[0]));
+    if (threadIdx.x == 0) accept[0] = ok ? 1 : 0;
   }
 }
 
@@ -455,11 +429,7 @@ __global__ void __launch_bounds__(kPointThreads) k_table_msm(const uint32_t* con
   }
   __shared__ uint32_t sp[kPointThreads][32];
   ge_store(sp[threadIdx.x], acc);
-  __syncthreads();
-  for (int h = kPointThreads / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) ge_store(sp[threadIdx.x], ge_add(ge_load(sp[threadIdx.x]), ge_load(sp[threadIdx.x + h])));
-    __syncthreads();
-  }
+  compact::quad_tree(sp, kPointThreads);
   if (threadIdx.x < 32) partial[(uint64_t)blockIdx.x * kPointPartialWords + threadIdx.x] = sp[0][threadIdx.x];
   if (threadIdx.x == 0) partial[(uint64_t)blockIdx.x * kPointPartialWords + 32] = 0;
 }

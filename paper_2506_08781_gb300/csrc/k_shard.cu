@@ -164,17 +164,13 @@ __global__ void __launch_bounds__(kShardThreads) k_combine_check(const uint32_t*
   __syncthreads();
   const ge term = tid < 64 ? table_pick(tableY, tid, dig_e[tid]) : table_pick(tableG, tid - 64, dig_s[tid - 64]);
   ge_store(pts_[tid], term);
-  __syncthreads();
   // e~Y + s~G: the 128 terms summed by quads
   static_assert(kShardThreads == 128, "one term per thread");
-  __shared__ uint32_t qs_[32][32];
-  compact::quad_sum128(pts_, qs_);
+  compact::quad_tree(pts_, 128);
   // [8](R~ - e~Y - s~G) by the first warp's quads (all of them compute it)
   if (tid < 32) {
-    ge d = ge_add_quad(ge_load(sR), ge_neg(ge_load(qs_[0])));
-#pragma unroll 1
-    for (int i = 0; i < 3; ++i) d = ge_dbl_quad(d);
-    if (tid == 0) accept[0] = (ge_is_identity(d) && well_formed && (*status & kErrKey) == 0) ? 1 : 0;
+    const bool eq = compact::quad_equal(ge_load(sR), ge_load(pts_[0]));
+    if (tid == 0) accept[0] = (eq && well_formed && (*status & kErrKey) == 0) ? 1 : 0;
   }
 }
 

@@ -359,23 +359,17 @@ __global__ void __launch_bounds__(kPointThreads, MINB) k_points(const PointArgs 
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < a.count; t += stride)
     decode_one(a, t, acc, bad);
 #endif
-  // tree reduction in shared memory
+  // the block's sum by quads (a few us less at the end of a small launch than one lane per
+  // addition), over as many points as the block can hold
   __shared__ uint32_t sp[kPointThreads][32];
-  __shared__ uint32_t sbad[kPointThreads];
-  ge_store(sp[threadIdx.x], acc);
-  sbad[threadIdx.x] = bad;
+  __shared__ uint32_t sbad;
+  if (threadIdx.x == 0) sbad = 0;
   __syncthreads();
-  for (int h = kPointThreads / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) {
-      const ge o = ge_load(sp[threadIdx.x + h]);
-      const ge m = ge_load(sp[threadIdx.x]);
-      ge_store(sp[threadIdx.x], ge_add(m, o));
-      sbad[threadIdx.x] += sbad[threadIdx.x + h];
-    }
-    __syncthreads();
-  }
+  ge_store(sp[threadIdx.x], acc);
+  if (bad) atomicAdd(&sbad, bad);
+  compact::quad_tree(sp, a.count < 1 ? 1 : a.count < kPointThreads ? (int)a.count : kPointThreads);
   if (threadIdx.x < 32) a.partial[(uint64_t)blockIdx.x * kPointPartialWords + threadIdx.x] = sp[0][threadIdx.x];
-  if (threadIdx.x == 0) a.partial[(uint64_t)blockIdx.x * kPointPartialWords + 32] = sbad[0];
+  if (threadIdx.x == 0) a.partial[(uint64_t)blockIdx.x * kPointPartialWords + 32] = sbad;
 }
 
 // Fixed-window tables table[w][d-1] = d 16^w P (w = 0..63, d = 1..8) of n keys, in two
@@ -438,91 +432,7 @@ __global__ void __launch_bounds__(128) k_table_fill(uint32_t n, uint32_t* __rest
   }
 }
 
-// Runs once per call: its point operations are the compact (out-of-line) ones, its code being
-// fetched cold on every launch.
-__global__ void __launch_bounds__(kFinalThreads) k_finalize(const FinalArgs a) {
-  __shared__ unsigned long long sums[kPartialWords];
-  __shared__ uint32_t pts[kFinalThreads][32];
-  __shared__ uint32_t pbad;
-  __shared__ int8_t dig_e[64], dig_s[64];
-  __shared__ uint32_t sh_e[8], sh_s[8];
-  __shared__ uint32_t bad_flag;
-  const int tid = threadIdx.x;
-  if (tid < kPartialWords) sums[tid] = 0;
-  if (tid == 0) { pbad = 0; bad_flag = 0; }
-  __syncthreads();
-  // scalar partial sums: word w of every block's partial, the blocks split over
-  // kFinalThreads / kPartialWords threads per word (a chain of dependent loads per word was the
-  // kernel's longest part)
-  constexpr int kLanesPerWord = kFinalThreads / kPartialWords;
-  if (tid < kLanesPerWord * kPartialWords) {
-    const int w = tid % kPartialWords, lane = tid / kPartialWords;
-    unsigned long long v = 0;
-    for (uint32_t b = lane; b < a.nhash; b += kLanesPerWord) v += a.hash_partial[(size_t)b * kPartialWords + w];
-    atomicAdd(&sums[w], v);
-  }
-  // point partials
-  ge acc = ge_identity();
-  uint32_t bad = 0;
-  for (uint32_t b = tid; b < a.npoint; b += kFinalThreads) {
-    acc = compact::add(acc, ge_load(a.point_partial + (size_t)b * kPointPartialWords));
-    bad += a.point_partial[(size_t)b * kPointPartialWords + 32];
-  }
-  ge_store(pts[tid], acc);
-  atomicAdd(&pbad, bad);
-  __syncthreads();
-  for (int h = kFinalThreads / 2; h > 0; h >>= 1) {
-    if (tid < h) ge_store(pts[tid], compact::add(ge_load(pts[tid]), ge_load(pts[tid + h])));
-    __syncthreads();
-  }
-  if (tid == 0) {
-    const sc e = limb_sums_to_scalar(sums);
-    sc s;
-    uint32_t bf = (sums[26] != 0 || pbad != 0) ? 1u : 0u;
-    if (a.s_given) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        s.v[k] = a.s_given[4 * k] | (a.s_given[4 * k + 1] << 8) | (a.s_given[4 * k + 2] << 16) |
-                 ((uint32_t)a.s_given[4 * k + 3] << 24);
-      if (!sc_is_canonical(s.v)) bf = 1;
-    } else {
-      s = limb_sums_to_scalar(sums + 13);
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) { sh_e[k] = e.v[k]; sh_s[k] = s.v[k]; }
-    recode4(e.v, dig_e);
-    recode4(s.v, dig_s);
-    bad_flag = bf;
-  }
-  __syncthreads();
-  // R is the reduced point sum unless given
-  ge R = a.R_given ? ge_load(a.R_given) : ge_load(pts[0]);
-  __syncthreads();
-  // window terms: thread w adds dig_e[w] 16^w Y + dig_s[w] 16^w G
-  ge term = ge_identity();
-  if (tid < kTableWindows) {
-    term = compact::add(table_pick(a.tableY, tid, dig_e[tid]), table_pick(a.tableG, tid, dig_s[tid]));
-  }
-  ge_store(pts[tid], term);
-  __syncthreads();
-  for (int h = kTableWindows / 2; h > 0; h >>= 1) {
-    if (tid < h) ge_store(pts[tid], compact::add(ge_load(pts[tid]), ge_load(pts[tid + h])));
-    __syncthreads();
-  }
-  if (tid == 0) {
-    const ge eYsG = ge_load(pts[0]);
-    const ge diff = compact::sub(R, eYsG);
-    const bool ok = ge_is_identity(compact::mul_cofactor(diff)) && !bad_flag;
-    const bool key_bad = (*a.status & kErrKey) != 0;
-    a.accept[0] = (ok && !key_bad) ? 1 : 0;
-    if (a.out_words) {
-      for (int k = 0; k < 8; ++k) { a.out_words[k] = sh_e[k]; a.out_words[8 + k] = sh_s[k]; }
-      ge_store(a.out_words + 16, R);
-    }
-  }
-}
-
-// The final check split in two so that its expensive half overlaps the MSM:
+// The final check in two halves, so that the expensive one overlaps the MSM:
 // k_final_prep (side stream, after hashing and the window table of Y) reduces the scalar
 // partials to e and s and evaluates [e]Y + [s]G from the two window tables (128 terms
 // summed by a shared-memory tree); k_final_check (after the MSM) only forms
@@ -564,11 +474,9 @@ __global__ void __launch_bounds__(128) k_final_prep(const PrepArgs a) {
   __syncthreads();
   const ge term = tid < 64 ? table_pick(a.tableY, tid, dig_e[tid]) : table_pick(a.tableG, tid - 64, dig_s[tid - 64]);
   ge_store(pts_[tid], term);
-  __syncthreads();
-  static_assert(kPrepThreads == 128 && kWindowThreads == 128, "quad_sum128 takes one term per thread of 128");
-  __shared__ uint32_t qs_[32][32];
-  compact::quad_sum128(pts_, qs_);
-  if (tid < 32) a.prep[tid] = qs_[0][tid];
+  static_assert(kPrepThreads == 128 && kWindowThreads == 128, "one table term per thread");
+  compact::quad_tree(pts_, 128);
+  if (tid < 32) a.prep[tid] = pts_[0][tid];
   if (tid == 0) a.prep[32] = bad_flag;
 }
 
@@ -638,21 +546,16 @@ __global__ void __launch_bounds__(kWindowThreads) k_window_prep(const unsigned l
   __syncthreads();
   const ge term = tid < 64 ? table_pick(tableY, tid, dig_e[tid]) : table_pick(tableG, tid - 64, dig_s[tid - 64]);
   ge_store(pts_[tid], term);
-  __syncthreads();
-  static_assert(kPrepThreads == 128 && kWindowThreads == 128, "quad_sum128 takes one term per thread of 128");
-  __shared__ uint32_t qs_[32][32];
-  compact::quad_sum128(pts_, qs_);
-  if (tid < 32) Pw[32 * w + tid] = qs_[0][tid];
+  compact::quad_tree(pts_, 128);
+  if (tid < 32) Pw[32 * w + tid] = pts_[0][tid];
 }
 
 // One warp (quad operations: every lane takes part).
 __global__ void k_final_check(const uint32_t* prep, const uint32_t* R, const uint32_t* point_bad,
                               const uint32_t* status, uint8_t* accept) {
   if (blockIdx.x != 0) return;
-  ge d = ge_add_quad(ge_load(R), ge_neg(ge_load(prep)));
-#pragma unroll 1
-  for (int i = 0; i < 3; ++i) d = ge_dbl_quad(d);
-  const bool ok = ge_is_identity(d) && prep[32] == 0 && !(point_bad && *point_bad) && (*status & kErrKey) == 0;
+  const bool eq = compact::quad_equal(ge_load(R), ge_load(prep));
+  const bool ok = eq && prep[32] == 0 && !(point_bad && *point_bad) && (*status & kErrKey) == 0;
   if (threadIdx.x == 0) accept[0] = ok ? 1 : 0;
 }
 

@@ -798,30 +798,6 @@ int run_msm(poslo_ctx* ctx, cudaStream_t st, const uint32_t* pts, const uint32_t
   return POSLO_OK;
 }
 
-int run_finalize(poslo_ctx* ctx, const unsigned long long* hpart, uint32_t nhb, const uint32_t* ppart, uint32_t npb,
-                 const uint32_t* R_given, const uint8_t* s_given, const uint32_t* tableY, uint8_t* d_acc,
-                 uint32_t* out_words) {
-  FinalArgs f{};
-  f.hash_partial = hpart;
-  f.nhash = nhb;
-  f.point_partial = ppart;
-  f.npoint = npb;
-  f.R_given = R_given;
-  f.s_given = s_given;
-  f.tableY = tableY;
-  f.tableG = ctx->tableG;
-  f.accept = d_acc;
-  f.out_words = out_words;
-  f.status = ctx->status;
-  cudaEvent_t tb, te;
-  timer_begin(ctx, "finalize", ctx->s_main, &tb, &te);
-  k_finalize<<<1, kFinalThreads, 0, ctx->s_main>>>(f);
-  ++ctx->launch_count;
-  CU(cudaGetLastError());
-  timer_end(ctx, "finalize", ctx->s_main, tb, te);
-  return POSLO_OK;
-}
-
 // Ordered list of flagged entries (first_index + t, ascending) into out (room for cap);
 // the full count goes to *d_count (device).
 int run_compact(poslo_ctx* ctx, const uint8_t* flags, uint64_t n, uint64_t first_index, uint64_t* out, uint64_t cap,
@@ -1947,6 +1923,9 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     if ((rc = ensure_t(ctx, "w_partial", (size_t)wblocks * kPartialWords * 8, &wpart))) return rc;
     k_weighted_sums<<<wblocks, kHashThreads, 0, ctx->s_main>>>(d_e, sb.s, z, inv, nullptr, n, wpart);
     ++ctx->launch_count;
+    uint32_t* prep;   // [e]Y + [s]G of the weighted sums, on the table stream beside the points' side
+    if ((rc = ensure_t(ctx, "confirm_prep", 4 * 33, &prep))) return rc;
+    if ((rc = run_prep(ctx, wpart, (uint32_t)wblocks, nullptr, tableY, prep, nullptr, 0, nullptr))) return rc;
     // sum over the unflagged entries of [z_t]R_t = the whole batch's sum (Horner over the window
     // sums the first weighted check left behind; undecodable points are not in it) minus the
     // flagged entries' with decodable points (an MSM over the flagged entries alone)
@@ -1976,7 +1955,12 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
       CU(cudaGetLastError());
       timer_end(ctx, "confirm", ctx->s_main, tb, te);
     }
-    if ((rc = run_finalize(ctx, wpart, wblocks, nullptr, 0, Rw, nullptr, tableY, d_acc, nullptr))) return rc;
+    // (not run_check: its wait on the points stream's event is for a decoding launched in the
+    // same way, and this one may have run inside a replayed graph)
+    CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_prep, 0));
+    k_final_check<<<1, 32, 0, ctx->s_main>>>(prep, Rw, nullptr, ctx->status, d_acc);
+    ++ctx->launch_count;
+    CU(cudaGetLastError());
     uint8_t conf = 0;
     CU(cudaMemcpyAsync(&conf, d_acc, 1, cudaMemcpyDeviceToHost, ctx->s_main));
     if ((rc = check_status(ctx))) return rc;
@@ -2333,7 +2317,7 @@ int poslo_distill_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrell
   KeyForget kforget{ctx, batch ? batch->Y : nullptr, &kmiss, false};
   if ((rc = ccd_common(ctx, batch, n_umbrella, sb, n1, &tableY, &esum, kmiss, kforget))) return rc;
   const uint64_t g = n1 / n_umbrella;
-  uint32_t *pts, *ppart, npb, *words;
+  uint32_t *pts, *ppart, npb, *words, *usums;
   uint8_t *badR, *ok, *inv, *encs;
   uint64_t* d_idx;
   if ((rc = ensure_t(ctx, "ccd_pts", 4 * kPtsWords * n1, &pts))) return rc;
@@ -2342,20 +2326,22 @@ int poslo_distill_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrell
   inv = ok + n1;
   if ((rc = ensure_t(ctx, "ccd_words", 32 * (1 + (size_t)n_umbrella), &words))) return rc;
   if ((rc = ensure_t(ctx, "ccd_encs", 32 * (1 + (size_t)n_umbrella), &encs))) return rc;
+  if ((rc = ensure_t(ctx, "ccd_usums", 4 * kPointPartialWords * (size_t)n_umbrella, &usums))) return rc;
   const uint64_t capn = std::max<uint64_t>(std::min<uint64_t>(ccd->cap, n1), 1);
   if ((rc = ensure_t(ctx, "ccd_idx", 8 * capn + 8, &d_idx))) return rc;
   uint64_t* d_cnt = d_idx + capn;
   if ((rc = run_points(ctx, sb.R, n1, pts, badR, &ppart, &npb, ctx->ev_staged))) return rc;
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_points, 0));
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_table, 0));
-  // b_i for every epoch, then ccd^v (group 0) and the umbrellas (groups 1..n^u)
+  // b_i for every epoch, then the umbrellas (groups 1..n^u) and from their sums ccd^v (group 0)
   k_check_list<<<(unsigned)((4 * n1 + 127) / 128), 128, 0, ctx->s_main>>>(
       reinterpret_cast<const uint32_t*>(esum), sb.s, pts, badR, (uint32_t)n1, tableY, ctx->tableG, ok);
   k_flip<<<(unsigned)((n1 + 255) / 256), 256, 0, ctx->s_main>>>(ok, n1, inv);
-  k_scalar_group_sums<<<1, kCcdThreads, 0, ctx->s_main>>>(sb.s, n1, n1, inv, words);
-  k_point_group_sums<<<1, kCcdThreads, 0, ctx->s_main>>>(pts, badR, n1, n1, inv, encs);
   k_scalar_group_sums<<<n_umbrella, kCcdThreads, 0, ctx->s_main>>>(sb.s, g, n1, inv, words + 8);
-  k_point_group_sums<<<n_umbrella, kCcdThreads, 0, ctx->s_main>>>(pts, badR, g, n1, inv, encs + 32);
+  launch_point_group_sums(n_umbrella, ctx->s_main, pts, badR, g, n1, inv, encs + 32, usums);
+  k_scalar_group_sums<<<1, kCcdThreads, 0, ctx->s_main>>>(reinterpret_cast<const uint8_t*>(words + 8), n_umbrella,
+                                                          n_umbrella, nullptr, words);
+  k_sum_encode<<<1, kFinalThreads, 0, ctx->s_main>>>(usums, n_umbrella, nullptr, encs, nullptr);
   ctx->launch_count += 6;
   CU(cudaGetLastError());
   const uint64_t first_epoch = batch->first_index / batch->n2;
