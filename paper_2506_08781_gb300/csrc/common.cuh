@@ -315,10 +315,9 @@ __device__ __forceinline__ sc limb_sums_to_scalar(const unsigned long long* sums
 //                  [e]Y + [s]G taken from the two fixed-window tables (128 additions)
 
 
-//   k_entry_check_group  the same check, eight lanes per entry (two quads summing the Y and
-//                  the G terms side by side with quad-cooperative additions), on the decoded
-//                  points and malformed flags of the first stage: the direct localisation of
-//                  small batches, where the latency of one entry is the latency of the launch
+//   k_entry_check_lanes  the same check, 8 to 32 lanes per entry (check_lanes), on the decoded
+//                  points and malformed flags: the direct localisation of small batches, where
+//                  the latency of one entry is the latency of the launch
 struct DirectCheckArgs {
   const uint8_t* e;          // n*32 (from k_hash)
   const uint8_t* s;          // n*32
@@ -330,7 +329,7 @@ struct DirectCheckArgs {
   const uint32_t* tableG;
   uint8_t* invalid;          // n bytes: 1 = entry fails its own check
 };
-__global__ void __launch_bounds__(128) k_entry_check_group(const DirectCheckArgs a);
+void launch_entry_check(cudaStream_t st, const DirectCheckArgs& a);
 
 
 __device__ __forceinline__ ge double_scalar_tables(const uint32_t e[8], const uint32_t s[8],
@@ -595,43 +594,100 @@ __device__ __forceinline__ void pts_load(const uint32_t* src, fe& x, fe& y, fe& 
   t2d = fe_const(v[4].x, v[4].y, v[4].z, v[4].w, v[5].x, v[5].y, v[5].z, v[5].w);
 }
 
-// [8](R_t - e_t Y - s_t G) = O for entry t by the eight lanes of a group (lanes 8g .. 8g+7 of
-// the warp): the first quad sums the 64 terms of [e]Y from Y's window table, the second the
-// 64 of [s]G from G's, each fetching the next window's entry during the current addition;
-// the two sums meet by shuffles and every lane returns the verdict.  Every lane of the warp
-// must call it (full-mask shuffles).
-__device__ __forceinline__ bool entry_check8(const uint8_t* e32, const uint8_t* s32, const uint32_t* pts_t,
-                                             bool malformed, const uint32_t* tableY, const uint32_t* tableG) {
-  const bool g_half = (threadIdx.x & 4) != 0;
+// A point of 32 words at a 16-byte aligned address (the window tables' entries).
+__device__ __forceinline__ ge ge_load4(const uint32_t* src) {
+  const uint4* p = reinterpret_cast<const uint4*>(src);
+  uint4 v[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __ldg(p + i);
+  ge r;
+  r.X = fe_const(v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w);
+  r.Y = fe_const(v[2].x, v[2].y, v[2].z, v[2].w, v[3].x, v[3].y, v[3].z, v[3].w);
+  r.Z = fe_const(v[4].x, v[4].y, v[4].z, v[4].w, v[5].x, v[5].y, v[5].z, v[5].w);
+  r.T = fe_const(v[6].x, v[6].y, v[6].z, v[6].w, v[7].x, v[7].y, v[7].z, v[7].w);
+  return r;
+}
+
+// [8](R - e Y - s G) = O by LANES (8, 16 or 32) consecutive lanes of a warp, which all hold the
+// same R and scalars: the 64 terms of [e]Y and the 64 of [s]G from the two window tables are
+// cut into one run per quad (64, 32 or 16 terms), each quad adds its run with quad-cooperative
+// additions (the next entry fetched during the current addition), a shuffle tree joins the
+// quads, and every lane returns the verdict.  More lanes shorten the chain of one check (LANES =
+// 32: 15 + 3 additions), fewer save the additions of the tree and the last check, which all
+// quads compute.  Every lane of the warp must call it (full-mask shuffles).
+//
+// Digits: with k' = k + sum_i 8 16^i, nibble i of k' is digit i of the signed recoding of
+// sc_digit4 plus 8 (the recoding carries exactly where adding 8 to the nibble does), so a quad
+// starts in the middle of the scalar without walking the windows below.
+template <int LANES>
+__device__ __forceinline__ bool check_lanes(const uint8_t* e32, const uint8_t* s32, const ge& R,
+                                            const uint32_t* tableY, const uint32_t* tableG) {
+  constexpr int kTerms = 512 / LANES, kWords = kTerms / 8;
+  const int lane = threadIdx.x & 31;
+  const int t0 = ((lane & (LANES - 1)) >> 2) * kTerms;   // first term; 64 and up are G's
+  const bool g_half = t0 >= 64;
+  const int w0 = t0 & 63;
   const uint4* kp = reinterpret_cast<const uint4*>(g_half ? s32 : e32);
   const uint4 k0 = __ldg(kp), k1 = __ldg(kp + 1);
-  const uint32_t k[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
-  const uint32_t* tab = g_half ? tableG : tableY;
-  ge acc = ge_identity();
-  int carry = 0;
-  ge next = table_pick(tab, 0, sc_digit4(k, 0, carry));
-  for (int w = 0; w < kTableWindows; ++w) {
+  uint32_t k[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+  const uint32_t eights[8] = {0x88888888u, 0x88888888u, 0x88888888u, 0x88888888u,
+                              0x88888888u, 0x88888888u, 0x88888888u, 0x88888888u};
+  add8(k, k, eights);
+  uint32_t dig[kWords];
+#pragma unroll
+  for (int j = 0; j < kWords; ++j) {   // words w0 / 8 + j (no dynamic register index)
+    dig[j] = k[j];
+#pragma unroll
+    for (int i = kWords; i + j < 8; i += kWords) dig[j] = (w0 >> 3) == i ? k[i + j] : dig[j];
+  }
+  const uint32_t* row = (g_half ? tableG : tableY) + (size_t)w0 * kTableDigits * 32;
+  auto pick = [&](int i) {   // term i of the run; consumes one nibble
+    const int d = (int)(dig[0] & 15u) - 8;
+    dig[0] >>= 4;
+    if ((i & 7) == 7) {
+#pragma unroll
+      for (int j = 0; j + 1 < kWords; ++j) dig[j] = dig[j + 1];
+    }
+    if (d == 0) return ge_identity();
+    const ge p = ge_load4(row + ((size_t)i * kTableDigits + (abs(d) - 1)) * 32);
+    return d < 0 ? ge_neg(p) : p;
+  };
+  ge acc = pick(0);
+  ge next = pick(1);
+#pragma unroll 1
+  for (int i = 1; i < kTerms; ++i) {
     const ge cur = next;
-    if (w + 1 < kTableWindows) next = table_pick(tab, w + 1, sc_digit4(k, w + 1, carry));
+    if (i + 1 < kTerms) next = pick(i + 1);
     acc = ge_add_quad(acc, cur);
   }
-  ge other;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    other.X.v[i] = __shfl_xor_sync(0xffffffffu, acc.X.v[i], 4);
-    other.Y.v[i] = __shfl_xor_sync(0xffffffffu, acc.Y.v[i], 4);
-    other.Z.v[i] = __shfl_xor_sync(0xffffffffu, acc.Z.v[i], 4);
-    other.T.v[i] = __shfl_xor_sync(0xffffffffu, acc.T.v[i], 4);
+#pragma unroll 1
+  for (int o = 4; o < LANES; o <<= 1) {
+    ge other;
+    other.X = fe_shfl(acc.X, lane ^ o); other.Y = fe_shfl(acc.Y, lane ^ o);
+    other.Z = fe_shfl(acc.Z, lane ^ o); other.T = fe_shfl(acc.T, lane ^ o);
+    acc = ge_add_quad(acc, other);
   }
-  acc = ge_add_quad(acc, other);
+  ge d = ge_add_quad(R, ge_neg(acc));
+#pragma unroll 1
+  for (int i = 0; i < 3; ++i) d = ge_dbl_quad(d);
+  return ge_is_identity(d);
+}
+
+// The same for a decoded point (kPtsWords words).
+template <int LANES>
+__device__ __forceinline__ bool entry_check_lanes(const uint8_t* e32, const uint8_t* s32, const uint32_t* pts_t,
+                                                  bool malformed, const uint32_t* tableY, const uint32_t* tableG) {
   ge R;
   fe t2d;
   pts_load(pts_t, R.X, R.Y, t2d);
   R.Z = fe_one();
   R.T = fe_mul(R.X, R.Y);
-  const ge d = ge_sub(R, acc);
-  return !malformed && ge_is_identity(ge_dbl_quad(ge_dbl_quad(ge_dbl_quad(d))));
+  return check_lanes<LANES>(e32, s32, R, tableY, tableG) && !malformed;
 }
+
+// Lanes per check for n checks in one launch (measured on GB300, us per launch at
+// LANES = 8 / 16 / 32: see k_entry_check_lanes).
+constexpr uint64_t kLanes32Max = 2048, kLanes16Max = 4096;
 
 // ---- Distill segment tree (k_distill.cu) ----
 struct TreeArgs {
@@ -771,6 +827,22 @@ __global__ void k_gather_flagged(const uint32_t* pts, const uint32_t* z, const u
 __global__ void k_point_diff(const uint32_t* a, const uint32_t* b, uint32_t* out);
 __global__ void __launch_bounds__(256) k_ccd_points(const uint32_t* pts, const uint8_t* badR, const uint64_t* idx,
                                                     const uint64_t* nf_dev, const uint32_t* unit, uint8_t* enc_out);
+struct DirectFinishArgs {
+  const uint8_t* inv;        // n flags
+  uint64_t n;                // at most kDirectFirstMax
+  uint64_t first_index;
+  const uint8_t* s;          // n*32
+  const uint32_t* pts;       // n*kPtsWords
+  const uint8_t* badR;
+  const uint32_t* unit;      // unit sum of the decodable points (32 words) and its encoding
+  const uint8_t* unit_enc;
+  uint32_t* list;            // scratch: n local indices
+  uint8_t* out;              // ccd^v (s, R: 64 bytes), the count (8 bytes), 8 unused, then the
+  uint64_t cap;              // first cap indices (8 bytes each, ascending)
+};
+constexpr int kDirectFinishThreads = 256;
+constexpr size_t kDirectOutHeader = 80;
+__global__ void __launch_bounds__(kDirectFinishThreads) k_direct_finish(const DirectFinishArgs a);
 __global__ void __launch_bounds__(kHashThreads) k_weighted_sums(const uint8_t* e, const uint8_t* s, const uint32_t* z, const uint8_t* skip1,
                                 const uint8_t* skip2, uint64_t n, unsigned long long* partial);
 __global__ void k_flags_or(const uint8_t* a, const uint8_t* b, const uint8_t* c, uint64_t n, uint8_t* out);
@@ -829,8 +901,8 @@ __global__ void __launch_bounds__(kPointThreads) k_table_msm_windows(const uint3
                                                                      uint32_t* partial);
 __global__ void __launch_bounds__(kPointThreads) k_window_point_sums(const uint32_t* partial, uint32_t nblocks,
                                                                      uint32_t* out);
-__global__ void __launch_bounds__(128) k_device_unit_check(const uint32_t* const* tabs, SegSums ss, uint32_t n_dev,
-                                                           const uint32_t* tableG, uint8_t* dev_flag);
+void launch_device_unit_check(cudaStream_t st, const uint32_t* const* tabs, SegSums ss, uint32_t n_dev,
+                              const uint32_t* tableG, uint8_t* dev_flag);
 struct MultiCheckArgs {
   const uint32_t* pts;        // decoded R_t of the whole batch (kPtsWords each)
   const uint8_t* e;           // e_t, 32 bytes each
@@ -838,7 +910,7 @@ struct MultiCheckArgs {
   const uint8_t* badR;        // 1 = R_t does not decode
   const uint8_t* badS;        // 1 = s_t is not canonical
   const uint64_t* seg_start;  // n_dev + 1 entry offsets of the devices
-  const uint32_t* fl;         // the flagged devices, nfl of them
+  const uint32_t* fl;         // the devices checked, nfl of them (null: all, fstart = seg_start)
   const uint64_t* fstart;     // nfl + 1: prefix sums of their entry counts
   uint32_t nfl;
   const uint32_t* const* tabs;   // window table of each device's key (kTableWords words each)
@@ -846,10 +918,11 @@ struct MultiCheckArgs {
   uint8_t* inv;               // out: 1 = entry invalid (written for the flagged devices' entries)
 };
 __global__ void __launch_bounds__(128) k_multi_entry_check(const MultiCheckArgs a);
-// The same checks with eight lanes per entry (as k_entry_check_group): for few flagged
-// entries, where one entry's latency is the launch's.
-__global__ void __launch_bounds__(128) k_multi_entry_check_group(const MultiCheckArgs a);
-constexpr uint64_t kMultiGroupCheckMax = 16384;   // flagged entries up to which the group form runs
+// The same checks with 8 to 32 lanes per entry (check_lanes), for few entries, where one
+// entry's latency is the launch's: total entries of the devices checked, at most
+// kMultiGroupCheckMax.
+void launch_multi_entry_check_lanes(cudaStream_t st, const MultiCheckArgs& a, uint64_t total);
+constexpr uint64_t kMultiGroupCheckMax = 16384;
 __global__ void k_segment_any(const uint8_t* inv, const uint64_t* seg_start, const uint32_t* fl, uint8_t* out);
 // ---- POSLO-C distillation and SeBVer (k_ccd.cu) ----
 constexpr int kCcdThreads = 128;
@@ -857,11 +930,9 @@ __global__ void __launch_bounds__(kCcdThreads) k_scalar_group_sums(const uint8_t
                                                                    const uint8_t* skip, uint32_t* out);
 void launch_point_group_sums(unsigned groups, cudaStream_t st, const uint32_t* pts, const uint8_t* bad, uint64_t G,
                              uint64_t n, const uint8_t* skip, uint8_t* enc, uint32_t* partial);
-__global__ void __launch_bounds__(128) k_check_list(const uint32_t* e, const uint8_t* s, const uint32_t* pts,
-                                                    const uint8_t* bad, uint32_t n, const uint32_t* tableY,
-                                                    const uint32_t* tableG, uint8_t* ok);
 __global__ void k_gather32(const uint8_t* src, const uint64_t* idx, uint64_t n, uint8_t* dst);
-__global__ void k_flip(const uint8_t* ok, uint64_t n, uint8_t* flag);
+__global__ void k_flip(const uint8_t* flag, uint64_t n, uint8_t* ok);
+__global__ void k_noncanonical(const uint8_t* s, uint64_t n, uint8_t* bad);
 __global__ void k_offs_sub(uint64_t* offs, uint64_t n, uint64_t base);
 __global__ void k_device_to_entries(const uint8_t* dev_flag, const uint64_t* start, const uint8_t* badR,
                                     uint8_t* skip, int keep_flagged);

@@ -1,7 +1,7 @@
 // POSLO-C distillation and selective batch verification (Fig. 3b): per-epoch sums of e,
-// grouped sums of scalars and points (ccd^v, the umbrellas ccd^u, SeBVer's V and U sums),
-// and a list of independent cofactored checks [8](R_k - e_k Y - s_k G) = O (the per-epoch
-// C.AVer of Distill and the checks of SeBVer).
+// grouped sums of scalars and points (ccd^v, the umbrellas ccd^u, SeBVer's V and U sums).  The
+// independent cofactored checks [8](R_k - e_k Y - s_k G) = O (the per-epoch C.AVer of Distill
+// and the checks of SeBVer) are the entry checks of k_check.cu.
 #include "common.cuh"
 #include "compact.cuh"
 
@@ -80,35 +80,14 @@ void launch_point_group_sums(unsigned groups, cudaStream_t st, const uint32_t* p
   else k_point_group_sums<128><<<groups, 128, 0, st>>>(pts, bad, G, n, skip, enc, partial);
 }
 
-// ok[k] = s_k canonical, R_k decodable (not bad), and [8](R_k - e_k Y - s_k G) = O, for n
-// independent checks; one quad of lanes per check (quad-cooperative table additions), the
-// surplus quads repeating the last check without writing.
-__global__ void __launch_bounds__(128) k_check_list(const uint32_t* e, const uint8_t* s, const uint32_t* pts,
-                                                    const uint8_t* bad, uint32_t n, const uint32_t* tableY,
-                                                    const uint32_t* tableG, uint8_t* ok) {
-  const uint32_t quad = ((uint32_t)blockIdx.x * blockDim.x + threadIdx.x) >> 2;
-  const uint32_t k = quad < n ? quad : n - 1;
-  uint32_t ek[8], sk[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) ek[i] = e[8 * (size_t)k + i];
-  const uint4* sp = reinterpret_cast<const uint4*>(s + 32 * (size_t)k);
+// bad[k] = 1 when s_k is not canonical (the checks' other malformed input).
+__global__ void k_noncanonical(const uint8_t* s, uint64_t n, uint8_t* bad) {
+  const uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= n) return;
+  const uint4* sp = reinterpret_cast<const uint4*>(s + 32 * k);
   const uint4 s0 = sp[0], s1 = sp[1];
-  sk[0] = s0.x; sk[1] = s0.y; sk[2] = s0.z; sk[3] = s0.w; sk[4] = s1.x; sk[5] = s1.y; sk[6] = s1.z; sk[7] = s1.w;
-  const bool canon = sc_is_canonical(sk);
-  // every lane runs every quad operation (full-mask shuffles)
-  ge acc = ge_identity();
-  int ce = 0, cs = 0;
-  for (int w = 0; w < 64; ++w) {
-    acc = ge_add_quad(acc, table_pick(tableY, w, sc_digit4(ek, w, ce)));
-    acc = ge_add_quad(acc, table_pick(tableG, w, sc_digit4(sk, w, cs)));
-  }
-  ge R;
-  fe t2d;
-  pts_load(pts + (size_t)kPtsWords * k, R.X, R.Y, t2d);
-  R.Z = fe_one();
-  R.T = fe_mul(R.X, R.Y);
-  const bool good = canon && !bad[k] && ge_is_identity(ge_mul_cofactor(ge_sub(R, acc)));
-  if ((threadIdx.x & 3) == 0 && quad < n) ok[k] = good ? 1 : 0;
+  const uint32_t v[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+  bad[k] = sc_is_canonical(v) ? 0 : 1;
 }
 
 // dst[k] = src[idx[k]] for 32-byte records.
@@ -119,10 +98,10 @@ __global__ void k_gather32(const uint8_t* src, const uint64_t* idx, uint64_t n, 
   reinterpret_cast<uint4*>(dst + 32 * k)[half] = reinterpret_cast<const uint4*>(src + 32 * idx[k])[half];
 }
 
-// flag[k] = 1 - ok[k] (the invalid epochs of Distill, for the compaction and as skip mask).
-__global__ void k_flip(const uint8_t* ok, uint64_t n, uint8_t* flag) {
+// ok[k] = 1 - flag[k]: the bits b_i from the invalid flags.
+__global__ void k_flip(const uint8_t* flag, uint64_t n, uint8_t* ok) {
   const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n) flag[t] = ok[t] ? 0 : 1;
+  if (t < n) ok[t] = flag[t] ? 0 : 1;
 }
 
 }  // namespace poslo

@@ -25,14 +25,108 @@ __global__ void __launch_bounds__(128) k_entry_check(const CheckArgs a) {
   }
 }
 
-// Eight lanes per entry (entry_check8); surplus groups repeat the last entry and do not write.
-__global__ void __launch_bounds__(128) k_entry_check_group(const DirectCheckArgs a) {
-  const uint64_t grp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+// LANES lanes per entry (check_lanes); surplus groups repeat the last entry and do not write.
+template <int LANES>
+__global__ void __launch_bounds__(128) k_entry_check_lanes(const DirectCheckArgs a) {
+  const uint64_t grp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
   if (a.n == 0) return;   // grid-uniform
   const uint64_t t = grp < a.n ? grp : a.n - 1;
-  const bool ok = entry_check8(a.e + 32 * t, a.s + 32 * t, a.pts + (size_t)kPtsWords * t, a.badR[t] || a.badS[t],
-                               a.tableY, a.tableG);
-  if ((threadIdx.x & 7) == 0 && grp < a.n) a.invalid[t] = ok ? 0 : 1;
+  const bool ok = entry_check_lanes<LANES>(a.e + 32 * t, a.s + 32 * t, a.pts + (size_t)kPtsWords * t,
+                                           a.badR[t] || a.badS[t], a.tableY, a.tableG);
+  if ((threadIdx.x & (LANES - 1)) == 0 && grp < a.n) a.invalid[t] = ok ? 0 : 1;
+}
+
+void launch_entry_check(cudaStream_t st, const DirectCheckArgs& a) {
+  const int lanes = a.n <= kLanes32Max ? 32 : a.n <= kLanes16Max ? 16 : 8;
+  const unsigned grid = (unsigned)(((uint64_t)lanes * a.n + 127) / 128);
+  if (lanes == 32) k_entry_check_lanes<32><<<grid, 128, 0, st>>>(a);
+  else if (lanes == 16) k_entry_check_lanes<16><<<grid, 128, 0, st>>>(a);
+  else k_entry_check_lanes<8><<<grid, 128, 0, st>>>(a);
+}
+
+// The rest of Distill of a small batch after every entry's own check, in one block: the ordered
+// list of the flagged entries, ccd^v's scalar (the sum of the others' s_t) and its point (the
+// unit sum minus the flagged entries' decodable points, encoded; the unit sum's own encoding
+// when nothing is flagged).  Eight launches of the general path in one.
+__global__ void __launch_bounds__(kDirectFinishThreads) k_direct_finish(const DirectFinishArgs a) {
+  __shared__ uint32_t wsum[kDirectFinishThreads / 32];
+  __shared__ unsigned long long red[kDirectFinishThreads / 32][13];
+  __shared__ uint32_t sp[kDirectFinishThreads][32];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // thread tid owns the flags of a contiguous run
+  const uint64_t per = (a.n + kDirectFinishThreads - 1) / kDirectFinishThreads;
+  const uint64_t lo = min((uint64_t)tid * per, a.n), hi = min(lo + per, a.n);
+  uint32_t own = 0;
+  for (uint64_t t = lo; t < hi; ++t) own += a.inv[t] ? 1u : 0u;
+  uint32_t incl = own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+    if ((int)lane >= o) incl += v;
+  }
+  if (lane == 31) wsum[warp] = incl;
+  acc13 acc;
+  acc_zero(acc);
+  for (uint64_t t = tid; t < a.n; t += kDirectFinishThreads) {
+    if (a.inv[t]) continue;
+    const uint4* q = reinterpret_cast<const uint4*>(a.s + 32 * t);
+    const uint4 s0 = __ldg(q), s1 = __ldg(q + 1);
+    const uint32_t v[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+    acc_add<8>(acc, v);
+  }
+#pragma unroll
+  for (int k = 0; k < 13; ++k) {
+    unsigned long long v = acc.v[k];
+    warp_sum_u64(v);
+    if (lane == 0) red[warp][k] = v;
+  }
+  __syncthreads();
+  uint32_t base = incl - own, nf = 0;
+  for (uint32_t w = 0; w < kDirectFinishThreads / 32; ++w) {
+    base += w < warp ? wsum[w] : 0u;
+    nf += wsum[w];
+  }
+  uint64_t* idx = reinterpret_cast<uint64_t*>(a.out + kDirectOutHeader);
+  for (uint64_t t = lo; t < hi; ++t) {
+    if (!a.inv[t]) continue;
+    a.list[base] = (uint32_t)t;
+    if (base < a.cap) idx[base] = a.first_index + t;
+    ++base;
+  }
+  __syncthreads();   // the list is read by the whole block
+  if (tid == 32) {
+    unsigned long long sums[13];
+    for (int k = 0; k < 13; ++k) {
+      unsigned long long v = 0;
+      for (int w = 0; w < kDirectFinishThreads / 32; ++w) v += red[w][k];
+      sums[k] = v;
+    }
+    const sc r = limb_sums_to_scalar(sums);
+    for (int k = 0; k < 8; ++k) reinterpret_cast<uint32_t*>(a.out)[k] = r.v[k];
+  }
+  if (tid == 64) *reinterpret_cast<uint64_t*>(a.out + 64) = nf;
+  if (nf == 0) {   // block-uniform
+    if (tid < 8) reinterpret_cast<uint32_t*>(a.out + 32)[tid] = reinterpret_cast<const uint32_t*>(a.unit_enc)[tid];
+    return;
+  }
+  ge sum = ge_identity();
+  for (uint32_t i = tid; i < nf; i += kDirectFinishThreads) {
+    const uint32_t t = a.list[i];
+    if (a.badR[t]) continue;
+    fe x, y, t2d;
+    pts_load(a.pts + (size_t)kPtsWords * t, x, y, t2d);
+    sum = ge_madd(sum, x, y, t2d);
+  }
+  ge_store(sp[tid], sum);
+  compact::quad_tree(sp, nf < kDirectFinishThreads ? (int)nf : kDirectFinishThreads);
+  if (tid < 32) {
+    const ge v = ge_add_quad(ge_load(a.unit), ge_neg(ge_load(sp[0])));
+    if (tid == 0) {
+      uint32_t w[8];
+      compact::encode(v, w);
+      for (int k = 0; k < 8; ++k) reinterpret_cast<uint32_t*>(a.out + 32)[k] = w[k];
+    }
+  }
 }
 
 __global__ void __launch_bounds__(kHashThreads) k_sum_scalars(const uint8_t* s, uint64_t n, const uint8_t* skip,

@@ -388,26 +388,25 @@ __global__ void __launch_bounds__(kFinalThreads) k_multi_check(const uint32_t* P
   }
 }
 
-// Per-device unit check [8](Ru - Eu Y_d - Su G) = O, one quad of lanes per device: 64 + 64
-// quad-cooperative additions of entries of the window tables of Y_d and of G.  Devices that
-// fail, or hold malformed entries, are flagged.
+// Per-device unit check [8](Ru - Eu Y_d - Su G) = O, LANES lanes per device (check_lanes).
+// Devices that fail, or hold malformed entries, are flagged.
+template <int LANES>
 __global__ void __launch_bounds__(128) k_device_unit_check(const uint32_t* const* tabs, SegSums ss, uint32_t n_dev,
                                                            const uint32_t* tableG, uint8_t* dev_flag) {
-  const uint32_t quad = ((uint32_t)blockIdx.x * blockDim.x + threadIdx.x) >> 2;
-  const uint32_t d = quad < n_dev ? quad : n_dev - 1;   // surplus quads repeat the last device
-  const uint32_t* tY = tabs[d];
-  const uint32_t* eu = ss.Eu + 8 * (size_t)d;
-  const uint32_t* su = ss.Su + 8 * (size_t)d;
-  // every lane runs every quad operation (full-mask shuffles)
-  ge acc = ge_identity();
-  int ce = 0, cs = 0;
-  for (int w = 0; w < 64; ++w) {
-    acc = ge_add_quad(acc, table_pick(tY, w, sc_digit4(eu, w, ce)));
-    acc = ge_add_quad(acc, table_pick(tableG, w, sc_digit4(su, w, cs)));
-  }
-  const ge diff = ge_sub(ge_load(ss.Ru + 32 * (size_t)d), acc);
-  const bool ok = ge_is_identity(ge_mul_cofactor(diff)) && ss.bad[d] == 0;
-  if ((threadIdx.x & 3) == 0 && quad < n_dev) dev_flag[d] = ok ? 0 : 1;
+  const uint32_t grp = ((uint32_t)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
+  const uint32_t d = grp < n_dev ? grp : n_dev - 1;   // surplus groups repeat the last device
+  const bool ok = check_lanes<LANES>(reinterpret_cast<const uint8_t*>(ss.Eu + 8 * (size_t)d),
+                                     reinterpret_cast<const uint8_t*>(ss.Su + 8 * (size_t)d),
+                                     ge_load(ss.Ru + 32 * (size_t)d), tabs[d], tableG) && ss.bad[d] == 0;
+  if ((threadIdx.x & (LANES - 1)) == 0 && grp < n_dev) dev_flag[d] = ok ? 0 : 1;
+}
+
+void launch_device_unit_check(cudaStream_t st, const uint32_t* const* tabs, SegSums ss, uint32_t n_dev,
+                              const uint32_t* tableG, uint8_t* dev_flag) {
+  if (n_dev <= kLanes32Max)
+    k_device_unit_check<32><<<(unsigned)((32ull * n_dev + 127) / 128), 128, 0, st>>>(tabs, ss, n_dev, tableG, dev_flag);
+  else
+    k_device_unit_check<8><<<(unsigned)((8ull * n_dev + 127) / 128), 128, 0, st>>>(tabs, ss, n_dev, tableG, dev_flag);
 }
 
 // sum_d [k_d] Y_d over the keys not skipped, from their window tables: one (key, window)
@@ -476,27 +475,33 @@ __global__ void __launch_bounds__(128) k_multi_entry_check(const MultiCheckArgs 
   }
 }
 
-// k_multi_entry_check with eight lanes per entry; surplus groups repeat the last entry and
-// do not write.
-__global__ void __launch_bounds__(128) k_multi_entry_check_group(const MultiCheckArgs a) {
+// k_multi_entry_check with LANES lanes per entry (check_lanes); surplus groups repeat the last
+// entry and do not write.
+template <int LANES>
+__global__ void __launch_bounds__(128) k_multi_entry_check_lanes(const MultiCheckArgs a) {
   const uint64_t total = a.fstart[a.nfl];
   if (total == 0) return;   // grid-uniform
-  const uint64_t grp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+  const uint64_t grp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
   const uint64_t t = grp < total ? grp : total - 1;
-  uint32_t lo = 0, hi = a.nfl;   // fstart[lo] <= t < fstart[hi]
-  while (hi - lo > 1) {
-    const uint32_t mid = (lo + hi) >> 1;
-    if (a.fstart[mid] <= t) lo = mid; else hi = mid;
-  }
-  const uint64_t g = a.seg_start[a.fl[lo]] + (t - a.fstart[lo]);
-  const bool ok = entry_check8(a.e + 32 * g, a.s + 32 * g, a.pts + (size_t)kPtsWords * g, a.badR[g] || a.badS[g],
-                               a.tabs[a.fl[lo]], a.tableG);
-  if ((threadIdx.x & 7) == 0 && grp < total) a.inv[g] = ok ? 0 : 1;
+  const uint32_t k = segment_of(a.fstart, a.nfl, t);
+  const uint32_t d = a.fl ? a.fl[k] : k;
+  const uint64_t g = a.seg_start[d] + (t - a.fstart[k]);
+  const bool ok = entry_check_lanes<LANES>(a.e + 32 * g, a.s + 32 * g, a.pts + (size_t)kPtsWords * g,
+                                           a.badR[g] || a.badS[g], a.tabs[d], a.tableG);
+  if ((threadIdx.x & (LANES - 1)) == 0 && grp < total) a.inv[g] = ok ? 0 : 1;
 }
 
-// Per flagged device k: 1 if any of its entries is flagged in inv.
+void launch_multi_entry_check_lanes(cudaStream_t st, const MultiCheckArgs& a, uint64_t total) {
+  const int lanes = total <= kLanes32Max ? 32 : total <= kLanes16Max ? 16 : 8;
+  const unsigned grid = (unsigned)(((uint64_t)lanes * total + 127) / 128);
+  if (lanes == 32) k_multi_entry_check_lanes<32><<<grid, 128, 0, st>>>(a);
+  else if (lanes == 16) k_multi_entry_check_lanes<16><<<grid, 128, 0, st>>>(a);
+  else k_multi_entry_check_lanes<8><<<grid, 128, 0, st>>>(a);
+}
+
+// Per flagged device k (fl null: per device): 1 if any of its entries is flagged in inv.
 __global__ void k_segment_any(const uint8_t* inv, const uint64_t* seg_start, const uint32_t* fl, uint8_t* out) {
-  const uint32_t d = fl[blockIdx.x];
+  const uint32_t d = fl ? fl[blockIdx.x] : blockIdx.x;
   int any = 0;
   for (uint64_t t = seg_start[d] + threadIdx.x; t < seg_start[d + 1]; t += blockDim.x) any |= inv[t];
   any = __syncthreads_or(any);

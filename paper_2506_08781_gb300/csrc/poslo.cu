@@ -338,6 +338,17 @@ constexpr uint64_t kMaxCallEntries = (1ull << 32) - 1;
 // tree, descent and confirmation; the two meet near 32,768.
 constexpr uint64_t kDirectCheckMax = 16384;
 
+// Batches of at most this many entries are checked entry by entry at once, without the weighted
+// check of the batch before it (no weights, no MSM): the definition itself, in one launch whose
+// latency at this size is below that of the MSM's chain of short kernels, and the same work
+// whether the batch is valid or not.  Measured on GB300 (weighted check first / direct, us):
+// Distill of a valid batch 300 / 186 at 1,024 entries, 297 / 254 at 4,096, 305 / 304 at 6,000,
+// 308 / 374 at 8,192, with flips 510 / 199 at 1,024, 568 / 287 at 4,096; many signers with one
+// flipped entry 1,252 / 209 at 300 entries, 1,344 / 382 at 5,000, 1,418 / 512 at 8,000.
+constexpr uint64_t kDirectFirstMax = 4096;        // Distill
+constexpr uint64_t kMultiDirectFirstMax = 8192;   // many signers
+static_assert(kDirectFirstMax <= kDirectCheckMax && kMultiDirectFirstMax <= kMultiGroupCheckMax, "sizes of the checks");
+
 // Host inputs are copied R_t first: ev_staged marks their arrival, so the decoding (the
 // longest stage) starts while the messages are still on their way.
 int stage_batch(poslo_ctx* ctx, const poslo_batch* b, Staged& sb, size_t s_bytes_override = 0) {
@@ -1707,25 +1718,141 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
   uint32_t* Pw;   // per-window [E_w]Y + [S_w]G (32 words each), then the malformed-s flag
   if ((rc = ensure_t(ctx, "win_P", 4 * (32 * (size_t)kMsmMaxWindows + 1), &Pw))) return rc;
   uint32_t* Pw_bad = Pw + 32 * kMsmMaxWindows;
+  // window table of Y (table stream), unless cached
+  auto launch_key_table = [&]() -> int {
+    if (!kbuild) {
+      CU(cudaEventRecord(ctx->ev_table, ctx->s_main));
+      return POSLO_OK;
+    }
+    int rc;
+    CU(cudaEventRecord(ctx->ev_main, ctx->s_main));
+    CU(cudaStreamWaitEvent(ctx->s_table, ctx->ev_main, 0));
+    cudaEvent_t tb, te;
+    timer_begin(ctx, "table", ctx->s_table, &tb, &te);
+    if ((rc = launch_tables(ctx, ctx->s_table, d_Y, nullptr, nullptr, 1, kcached ? nullptr : tableY, 0, nullptr,
+                            kcached ? d_ydst : nullptr)))
+      return rc;
+    timer_end(ctx, "table", ctx->s_table, tb, te);
+    CU(cudaEventRecord(ctx->ev_table, ctx->s_table));
+    return POSLO_OK;
+  };
+  auto launch_seeds = [&]() -> int {
+    if (!ne) return POSLO_OK;
+    cudaEvent_t b, e;
+    timer_begin(ctx, "seeds", ctx->s_main, &b, &e);
+    launch_epoch_seeds((int)ctx->inst, (unsigned)((ne + 127) / 128), 128, ctx->s_main, d_ds, (int)ds_nodes.size(),
+                       e_first, ne, seeds, ctx->status);
+    ++ctx->launch_count;
+    CU(cudaGetLastError());
+    timer_end(ctx, "seeds", ctx->s_main, b, e);
+    return POSLO_OK;
+  };
+  HashArgs ha{};
+  ha.msgs = sb.msgs;
+  ha.offs = sb.offs;
+  ha.base_off = sb.base_off;
+  ha.n = n;
+  ha.first_index = batch->first_index;
+  ha.e0 = e_first;
+  ha.n2 = batch->n2;
+  ha.n2_log2 = log2_exact(batch->n2);
+  ha.seeds = seeds;
+  ha.e_out = d_e;
+  ha.s = sb.s;
+  ha.sbad_out = badS;
+  ha.partial = hpart;
+  ha.status = ctx->status;
+  DirectCheckArgs dc{};
+  dc.e = d_e;
+  dc.s = sb.s;
+  dc.pts = pts;
+  dc.badR = badR;
+  dc.badS = badS;
+  dc.n = n;
+  dc.tableY = tableY;
+  dc.tableG = ctx->tableG;
+  dc.invalid = inv;
+  const bool replayable = batch->on_device != 0 || sb.packed;
+  std::vector<uint64_t> sig = {n, batch->n2, batch->first_index, reinterpret_cast<uint64_t>(sb.msgs),
+                               reinterpret_cast<uint64_t>(sb.offs), reinterpret_cast<uint64_t>(sb.s),
+                               reinterpret_cast<uint64_t>(sb.R), sb.base_off, ds_nodes.size(), ctx->inst,
+                               reinterpret_cast<uint64_t>(tableY), kbuild ? 1u : 0u};
+  if (n && n <= kDirectFirstMax) {
+    // ---- a small batch: decoding beside seeds and hashing, every entry's own check, then list
+    // and ccd^v in one block; one round trip
+    const uint64_t capd = std::min(cap, n);
+    uint8_t* d_out;
+    uint32_t* list;
+    if ((rc = ensure_t(ctx, "direct_out", kDirectOutHeader + 8 * n, &d_out))) return rc;
+    if ((rc = ensure_t(ctx, "direct_list", 4 * n, &list))) return rc;
+    auto launch = [&]() -> int {
+      int rc;
+      if ((rc = launch_key_table())) return rc;
+      uint32_t *ppart, npb;
+      if ((rc = run_points(ctx, sb.R, n, pts, badR, &ppart, &npb, replayable ? nullptr : ctx->ev_staged))) return rc;
+      if ((rc = run_unit_sum(ctx, ppart, npb, unitR, d_ccd + 32, pbad))) return rc;
+      if ((rc = launch_seeds())) return rc;
+      cudaEvent_t tb, te;
+      timer_begin(ctx, "hash", ctx->s_main, &tb, &te);
+      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->s_main, ha, kHashBeside);
+      ++ctx->launch_count;
+      CU(cudaGetLastError());
+      timer_end(ctx, "hash", ctx->s_main, tb, te);
+      CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_table, 0));
+      CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_decoded, 0));
+      timer_begin(ctx, "direct", ctx->s_main, &tb, &te);
+      launch_entry_check(ctx->s_main, dc);
+      ++ctx->launch_count;
+      CU(cudaGetLastError());
+      timer_end(ctx, "direct", ctx->s_main, tb, te);
+      CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_points, 0));
+      DirectFinishArgs fa{};
+      fa.inv = inv;
+      fa.n = n;
+      fa.first_index = batch->first_index;
+      fa.s = sb.s;
+      fa.pts = pts;
+      fa.badR = badR;
+      fa.unit = unitR;
+      fa.unit_enc = d_ccd + 32;
+      fa.list = list;
+      fa.out = d_out;
+      fa.cap = capd;
+      k_direct_finish<<<1, kDirectFinishThreads, 0, ctx->s_main>>>(fa);
+      ++ctx->launch_count;
+      CU(cudaGetLastError());
+      return POSLO_OK;
+    };
+    sig.push_back(1);
+    sig.push_back(capd);
+    sig.push_back(reinterpret_cast<uint64_t>(d_out));
+    if ((rc = replayable ? run_replayable(ctx, ctx->g_distill, sig, launch) : launch())) return rc;
+    // the header and the first indices in one copy (page-locked)
+    const uint64_t first = std::min<uint64_t>(capd, (kSmallHostBytes - kDirectOutHeader) / 8);
+    CU(cudaMemcpyAsync(ctx->h_small, d_out, kDirectOutHeader + 8 * first, cudaMemcpyDeviceToHost, ctx->s_main));
+    if ((rc = check_status(ctx))) return rc;
+    kforget.armed = false;   // the key decoded: its table is sound
+    uint64_t cnt;
+    memcpy(&cnt, ctx->h_small + 64, 8);
+    const uint64_t got = std::min(cnt, capd);
+    if (invalid_idx) {
+      memcpy(invalid_idx, ctx->h_small + kDirectOutHeader, 8 * std::min(got, first));
+      if (got > first)
+        CU(cudaMemcpy(invalid_idx + first, d_out + kDirectOutHeader + 8 * first, 8 * (got - first),
+                      cudaMemcpyDeviceToHost));
+    }
+    *n_invalid = cnt;
+    if (ccd_s) memcpy(ccd_s, ctx->h_small, 32);
+    if (ccd_R) memcpy(ccd_R, ctx->h_small + 32, 32);
+    if (cnt > cap) return fail(ctx, POSLO_EBUFSMALL, "%llu invalid entries, room for %llu", (unsigned long long)cnt,
+                               (unsigned long long)cap);
+    return POSLO_OK;
+  }
   // ---- up to the weighted check of the whole batch; a device-resident batch of the previous
   // call's shape replays it from a CUDA graph
-  const bool replayable = batch->on_device != 0 || sb.packed;
   auto stage1 = [&]() -> int {
     int rc;
-    // window table of Y (table stream), unless cached
-    if (kbuild) {
-      CU(cudaEventRecord(ctx->ev_main, ctx->s_main));
-      CU(cudaStreamWaitEvent(ctx->s_table, ctx->ev_main, 0));
-      cudaEvent_t tb, te;
-      timer_begin(ctx, "table", ctx->s_table, &tb, &te);
-      if ((rc = launch_tables(ctx, ctx->s_table, d_Y, nullptr, nullptr, 1, kcached ? nullptr : tableY, 0, nullptr,
-                              kcached ? d_ydst : nullptr)))
-        return rc;
-      timer_end(ctx, "table", ctx->s_table, tb, te);
-      CU(cudaEventRecord(ctx->ev_table, ctx->s_table));
-    } else {
-      CU(cudaEventRecord(ctx->ev_table, ctx->s_main));
-    }
+    if ((rc = launch_key_table())) return rc;
     // decoding (points stream), from the moment the R_t have landed; then the speculative
     // ccd^v of the all-valid case (its R part)
     uint32_t *ppart, npb;
@@ -1734,15 +1861,7 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     // epoch seeds, then the weights z_t alone (they do not depend on the messages) so the
     // MSM's counting sort starts at once; the message hashing (with the per-entry outputs
     // Distill needs) runs on its own stream
-    if (ne) {
-      cudaEvent_t b, e;
-      timer_begin(ctx, "seeds", ctx->s_main, &b, &e);
-      launch_epoch_seeds((int)ctx->inst, (unsigned)((ne + 127) / 128), 128, ctx->s_main, d_ds, (int)ds_nodes.size(),
-                         e_first, ne, seeds, ctx->status);
-      ++ctx->launch_count;
-      CU(cudaGetLastError());
-      timer_end(ctx, "seeds", ctx->s_main, b, e);
-    }
+    if ((rc = launch_seeds())) return rc;
     ZPre zp;
     make_zpre(ctx->vseed, zp.w);
     if (n) {
@@ -1754,24 +1873,10 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     // (measured: hashing beside the decoding, 4.78 ms per 2^20-entry step, beats hashing on the
     // main stream before the sort, 4.88 ms, and beside the bucket accumulation, 4.95 ms)
     cudaStream_t hs = ctx->s_hash;
-    HashArgs a{};
-    a.msgs = sb.msgs;
-    a.offs = sb.offs;
-    a.base_off = sb.base_off;
-    a.n = n;
-    a.first_index = batch->first_index;
-    a.e0 = e_first;
-    a.n2 = batch->n2;
-    a.n2_log2 = log2_exact(batch->n2);
-    a.seeds = seeds;
-    a.e_out = d_e;
-    a.s = sb.s;
+    HashArgs a = ha;
     a.weighted = 1;
     for (int q = 0; q < 10; ++q) a.zpre[q] = zp.w[q];
     a.z_in = z;
-    a.sbad_out = badS;
-    a.partial = hpart;
-    a.status = ctx->status;
     MsmState ms;
     if ((rc = run_msm_sort(ctx, ctx->s_main, z, 4, nullptr, n, ms))) return rc;
     {
@@ -1799,11 +1904,9 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
   };
   if (replayable) {
     const MsmPlan plan = msm_plan(ctx, n, 4);
-    const std::vector<uint64_t> sig = {n, batch->n2, batch->first_index, reinterpret_cast<uint64_t>(sb.msgs),
-                                       reinterpret_cast<uint64_t>(sb.offs), reinterpret_cast<uint64_t>(sb.s),
-                                       reinterpret_cast<uint64_t>(sb.R), sb.base_off, ds_nodes.size(),
-                                       (uint64_t)plan.c, (uint64_t)plan.seg_log2, ctx->inst,
-                                       reinterpret_cast<uint64_t>(tableY), kbuild ? 1u : 0u};
+    sig.push_back(0);
+    sig.push_back((uint64_t)plan.c);
+    sig.push_back((uint64_t)plan.seg_log2);
     rc = run_replayable(ctx, ctx->g_distill, sig, stage1);
   } else {
     rc = stage1();
@@ -1838,19 +1941,9 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     // ---- a small batch: every entry's own check (Fig. 4 with |m| = 1) in one launch, the
     // definition itself, instead of the tree, the descent and the confirmation, whose fixed
     // latencies cost more at this size
-    DirectCheckArgs a{};
-    a.e = d_e;
-    a.s = sb.s;
-    a.pts = pts;
-    a.badR = badR;
-    a.badS = badS;
-    a.n = n;
-    a.tableY = tableY;
-    a.tableG = ctx->tableG;
-    a.invalid = inv;
     cudaEvent_t tb, te;
     timer_begin(ctx, "direct", ctx->s_main, &tb, &te);
-    k_entry_check_group<<<(unsigned)((8 * n + 127) / 128), 128, 0, ctx->s_main>>>(a);
+    launch_entry_check(ctx->s_main, dc);
     ++ctx->launch_count;
     CU(cudaGetLastError());
     timer_end(ctx, "direct", ctx->s_main, tb, te);
@@ -2265,6 +2358,26 @@ void store_le_words(const uint32_t* w, uint8_t* out) {
 // limbs little-endian) in *esum.
 // The key's window table comes from the key cache; a table this call builds into a new cache
 // slot is forgotten again (kforget) unless the caller disarms it once the key has decoded.
+// Main stream: ok[k] = s_k canonical, R_k decodable (badR) and [8](R_k - e_k Y - s_k G) = O for n
+// independent checks; inv[k] = 1 - ok[k], badS scratch of n bytes.
+void launch_check_list(poslo_ctx* ctx, const uint8_t* e, const uint8_t* s, const uint32_t* pts, const uint8_t* badR,
+                       uint8_t* badS, uint64_t n, const uint32_t* tableY, uint8_t* inv, uint8_t* ok) {
+  k_noncanonical<<<(unsigned)((n + 255) / 256), 256, 0, ctx->s_main>>>(s, n, badS);
+  DirectCheckArgs a{};
+  a.e = e;
+  a.s = s;
+  a.pts = pts;
+  a.badR = badR;
+  a.badS = badS;
+  a.n = n;
+  a.tableY = tableY;
+  a.tableG = ctx->tableG;
+  a.invalid = inv;
+  launch_entry_check(ctx->s_main, a);
+  k_flip<<<(unsigned)((n + 255) / 256), 256, 0, ctx->s_main>>>(inv, n, ok);
+  ctx->launch_count += 3;
+}
+
 int ccd_common(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrella, Staged& sb, uint64_t& n1,
                uint32_t** tableY, uint8_t** esum, std::vector<uint32_t>& kmiss, KeyForget& kforget) {
   int rc;
@@ -2321,7 +2434,8 @@ int poslo_distill_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrell
   uint8_t *badR, *ok, *inv, *encs;
   uint64_t* d_idx;
   if ((rc = ensure_t(ctx, "ccd_pts", 4 * kPtsWords * n1, &pts))) return rc;
-  if ((rc = ensure_t(ctx, "ccd_badR", n1, &badR))) return rc;
+  if ((rc = ensure_t(ctx, "ccd_badR", 2 * n1, &badR))) return rc;
+  uint8_t* badS = badR + n1;
   if ((rc = ensure_t(ctx, "ccd_ok", 2 * n1, &ok))) return rc;
   inv = ok + n1;
   if ((rc = ensure_t(ctx, "ccd_words", 32 * (1 + (size_t)n_umbrella), &words))) return rc;
@@ -2334,15 +2448,13 @@ int poslo_distill_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrell
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_points, 0));
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_table, 0));
   // b_i for every epoch, then the umbrellas (groups 1..n^u) and from their sums ccd^v (group 0)
-  k_check_list<<<(unsigned)((4 * n1 + 127) / 128), 128, 0, ctx->s_main>>>(
-      reinterpret_cast<const uint32_t*>(esum), sb.s, pts, badR, (uint32_t)n1, tableY, ctx->tableG, ok);
-  k_flip<<<(unsigned)((n1 + 255) / 256), 256, 0, ctx->s_main>>>(ok, n1, inv);
+  launch_check_list(ctx, esum, sb.s, pts, badR, badS, n1, tableY, inv, ok);
   k_scalar_group_sums<<<n_umbrella, kCcdThreads, 0, ctx->s_main>>>(sb.s, g, n1, inv, words + 8);
   launch_point_group_sums(n_umbrella, ctx->s_main, pts, badR, g, n1, inv, encs + 32, usums);
   k_scalar_group_sums<<<1, kCcdThreads, 0, ctx->s_main>>>(reinterpret_cast<const uint8_t*>(words + 8), n_umbrella,
                                                           n_umbrella, nullptr, words);
   k_sum_encode<<<1, kFinalThreads, 0, ctx->s_main>>>(usums, n_umbrella, nullptr, encs, nullptr);
-  ctx->launch_count += 6;
+  ctx->launch_count += 4;
   CU(cudaGetLastError());
   const uint64_t first_epoch = batch->first_index / batch->n2;
   if ((rc = run_compact(ctx, inv, n1, first_epoch, d_idx, std::min<uint64_t>(ccd->cap, n1), d_cnt))) return rc;
@@ -2410,7 +2522,7 @@ int poslo_sebver_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrella
   if ((rc = ensure_t(ctx, "seb_s", 32 * nchk, &s_chk))) return rc;
   if ((rc = ensure_t(ctx, "seb_R", 32 * nchk, &R_chk))) return rc;
   if ((rc = ensure_t(ctx, "seb_pts", 4 * kPtsWords * nchk, &pts))) return rc;
-  if ((rc = ensure_t(ctx, "seb_bad", 2 * nchk, &bad))) return rc;
+  if ((rc = ensure_t(ctx, "seb_bad", 4 * nchk, &bad))) return rc;
   d_bits = bad + nchk;
   CU(cudaMemcpyAsync(d_mask, mask.data(), n1, cudaMemcpyHostToDevice, ctx->s_main));
   if (mode == POSLO_SEBVER_V) {
@@ -2442,9 +2554,8 @@ int poslo_sebver_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrella
   if ((rc = run_points(ctx, R_chk, nchk, pts, bad, &ppart, &npb))) return rc;
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_points, 0));
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_table, 0));
-  k_check_list<<<(unsigned)((4 * nchk + 127) / 128), 128, 0, ctx->s_main>>>(e_chk, s_chk, pts, bad, (uint32_t)nchk,
-                                                                             tableY, ctx->tableG, d_bits);
-  ++ctx->launch_count;
+  launch_check_list(ctx, reinterpret_cast<const uint8_t*>(e_chk), s_chk, pts, bad, bad + 2 * nchk, nchk, tableY,
+                    bad + 3 * nchk, d_bits);
   CU(cudaGetLastError());
   CU(cudaMemcpyAsync(bits, d_bits, nchk, cudaMemcpyDeviceToHost, ctx->s_main));
   if ((rc = check_status(ctx))) return rc;
@@ -2846,7 +2957,8 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
   sig.insert(sig.end(), mb->first_index, mb->first_index + nd);
   sig.insert(sig.end(), mb->n2, mb->n2 + nd);
   sig.insert(sig.end(), mb->ds_off, mb->ds_off + nd + 1);
-  auto stage1 = [&]() -> int {
+  // window tables of the keys that need building (table stream) and the epoch seeds of every device
+  auto launch_tables_seeds = [&]() -> int {
     int rc;
     if (key_tables || (kcached && nbuild == 0)) {
       CU(cudaMemsetAsync(badY, 0, nd, ctx->s_main));
@@ -2872,12 +2984,132 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
       timer_end(ctx, "table", ctx->s_table, tb, te);
       CU(cudaEventRecord(ctx->ev_table, ctx->s_table));
     }
-    // epoch seeds of every device
     if (seed_off[nd]) {
       launch_epoch_seeds_multi((int)ctx->inst, (unsigned)((seed_off[nd] + 127) / 128), 128, ctx->s_main, d_nodes,
                                d_dsoff, seg_seed_off, seg_e0, nd, seeds, ctx->status);
       ++ctx->launch_count;
     }
+    return POSLO_OK;
+  };
+  HashArgs ha{};
+  ha.msgs = sb.msgs;
+  ha.offs = sb.offs;
+  ha.base_off = sb.base_off;
+  ha.n = N;
+  ha.n2 = 1;
+  ha.n2_log2 = 0xffffffffu;
+  ha.seeds = seeds;
+  ha.e_out = d_e;
+  ha.s = sb.s;
+  ha.sbad_out = badS;
+  ha.status = ctx->status;
+  ha.n_seg = nd;
+  ha.seg_start = seg_start;
+  ha.seg_first = seg_first;
+  ha.seg_seed_off = seg_seed_off;
+  ha.seg_e0 = seg_e0;
+  ha.seg_n2 = d_n2;
+  const int hblocks = (int)hash_groups((int)ctx->inst, ctx->sm_count, N);
+  unsigned long long* hpart;
+  if ((rc = ensure_t(ctx, "hash_partial", (size_t)hblocks * kPartialWords * 8, &hpart))) return rc;
+  ha.partial = hpart;
+  MultiCheckArgs ca{};
+  ca.pts = pts;
+  ca.e = d_e;
+  ca.s = sb.s;
+  ca.badR = badR;
+  ca.badS = badS;
+  ca.seg_start = seg_start;
+  ca.tabs = d_tabs;
+  ca.tableG = ctx->tableG;
+  // host side of a result: the pairs of the flagged batch positions g[0 .. got), ascending
+  auto write_pairs = [&](const uint64_t* g, uint64_t got) {
+    uint32_t d = 0;   // positions ascend, and so do devices: one walk of the device table
+    for (uint64_t q = 0; q < got; ++q) {
+      while (mb->dev_start[d + 1] <= g[q]) ++d;
+      invalid_pairs[2 * q] = d;
+      invalid_pairs[2 * q + 1] = mb->first_index[d] + (g[q] - mb->dev_start[d]);
+    }
+  };
+  // host side of the first round trip: a key that does not decode fails the call
+  std::vector<uint8_t> hbadY(nd), hmbad(nbuild);
+  auto read_bad_keys = [&]() -> int {
+    CU(cudaMemcpyAsync(hbadY.data(), badY, nd, cudaMemcpyDeviceToHost, ctx->s_main));
+    if (nbuild) CU(cudaMemcpyAsync(hmbad.data(), d_mbad, nbuild, cudaMemcpyDeviceToHost, ctx->s_main));
+    return POSLO_OK;
+  };
+  auto check_keys = [&]() -> int {
+    for (uint32_t k = 0; k < nbuild; ++k)
+      if (hmbad[k]) hbadY[kmiss[k]] = 1;
+    for (uint32_t d = 0; d < nd; ++d)
+      if (hbadY[d]) return fail(ctx, POSLO_EINVAL, "public key of device %u does not decode", d);
+    forget.armed = false;   // the built tables are sound
+    return POSLO_OK;
+  };
+  if (N && N <= kMultiDirectFirstMax && !per_window) {
+    // ---- a small batch: every entry of every device by its own check at once (see
+    // kMultiDirectFirstMax), instead of the combined check, the unit checks of the devices, their
+    // confirmation and the localisation after it
+    uint64_t* d_idx;
+    uint8_t *minv, *d_any;
+    const uint64_t capn = std::max<uint64_t>(std::min(cap, N), 1);
+    if ((rc = ensure_t(ctx, "m_inv", N1, &minv))) return rc;
+    if ((rc = ensure_t(ctx, "m_any", nd, &d_any))) return rc;
+    if ((rc = ensure_t(ctx, "m_idx", 8 * capn + 8, &d_idx))) return rc;
+    ca.fstart = seg_start;
+    ca.nfl = nd;
+    ca.inv = minv;
+    auto launch = [&]() -> int {
+      int rc;
+      if ((rc = launch_tables_seeds())) return rc;
+      uint32_t *ppart, npb;
+      if ((rc = run_points(ctx, sb.R, N, pts, badR, &ppart, &npb))) return rc;
+      cudaEvent_t tb, te;
+      timer_begin(ctx, "hash", ctx->s_main, &tb, &te);
+      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->s_main, ha, kHashBeside);
+      ++ctx->launch_count;
+      CU(cudaGetLastError());
+      timer_end(ctx, "hash", ctx->s_main, tb, te);
+      CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_table, 0));
+      CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_points, 0));
+      timer_begin(ctx, "localise", ctx->s_main, &tb, &te);
+      launch_multi_entry_check_lanes(ctx->s_main, ca, N);
+      k_segment_any<<<nd, 256, 0, ctx->s_main>>>(minv, seg_start, nullptr, d_any);
+      ctx->launch_count += 2;
+      CU(cudaGetLastError());
+      if ((rc = run_compact(ctx, minv, N, 0, d_idx + 1, std::min(cap, N), d_idx))) return rc;
+      timer_end(ctx, "localise", ctx->s_main, tb, te);
+      return POSLO_OK;
+    };
+    sig.push_back(1);
+    sig.push_back(std::min(cap, N));
+    if ((rc = run_replayable(ctx, ctx->g_multi, sig, launch))) return rc;
+    std::vector<uint8_t> any(nd);
+    if ((rc = read_bad_keys())) return rc;
+    CU(cudaMemcpyAsync(any.data(), d_any, nd, cudaMemcpyDeviceToHost, ctx->s_main));
+    const uint64_t first = std::min<uint64_t>(std::min(cap, N), kSmallHostBytes / 8 - 1);
+    CU(cudaMemcpyAsync(ctx->h_small, d_idx, 8 * (1 + first), cudaMemcpyDeviceToHost, ctx->s_main));
+    if ((rc = check_status(ctx))) return rc;
+    if ((rc = check_keys())) return rc;
+    if (settled) (*settled)(any.data());
+    for (uint32_t d = 0; d < nd; ++d) accept[d] = any[d] ? 0 : 1;
+    uint64_t cnt;
+    memcpy(&cnt, ctx->h_small, 8);
+    const uint64_t got = std::min(cnt, cap);
+    if (got && invalid_pairs) {
+      std::vector<uint64_t> g(got);
+      memcpy(g.data(), ctx->h_small + 8, 8 * std::min(got, first));
+      if (got > first) CU(cudaMemcpy(g.data() + first, d_idx + 1 + first, 8 * (got - first), cudaMemcpyDeviceToHost));
+      write_pairs(g.data(), got);
+    }
+    *n_invalid = cnt;
+    if (cnt > cap) return fail(ctx, POSLO_EBUFSMALL, "%llu invalid entries, room for %llu", (unsigned long long)cnt,
+                               (unsigned long long)cap);
+    return POSLO_OK;
+  }
+  auto stage1 = [&]() -> int {
+    int rc;
+    if ((rc = launch_tables_seeds())) return rc;
     // (side stream) decode every R_t, compiled to share the SMs with the hashing
     uint32_t *ppart, npb;
     if ((rc = run_points(ctx, sb.R, N, pts, badR, &ppart, &npb, nullptr, true))) return rc;
@@ -2892,34 +3124,13 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
     CU(cudaEventRecord(ctx->ev_main, ctx->s_main));
     CU(cudaStreamWaitEvent(ctx->s_hash, ctx->ev_main, 0));
     {
-      const int blocks = (int)hash_groups((int)ctx->inst, ctx->sm_count, N);
-      unsigned long long* hpart;
-      if ((rc = ensure_t(ctx, "hash_partial", (size_t)blocks * kPartialWords * 8, &hpart))) return rc;
-      HashArgs a{};
-      a.msgs = sb.msgs;
-      a.offs = sb.offs;
-      a.base_off = sb.base_off;
-      a.n = N;
-      a.n2 = 1;
-      a.n2_log2 = 0xffffffffu;
-      a.seeds = seeds;
-      a.e_out = d_e;
-      a.s = sb.s;
+      HashArgs a = ha;
       a.weighted = 1;
       for (int q = 0; q < 10; ++q) a.zpre[q] = zp.w[q];
       a.z_in = z;
-      a.sbad_out = badS;
-      a.partial = hpart;
-      a.status = ctx->status;
-      a.n_seg = nd;
-      a.seg_start = seg_start;
-      a.seg_first = seg_first;
-      a.seg_seed_off = seg_seed_off;
-      a.seg_e0 = seg_e0;
-      a.seg_n2 = d_n2;
       cudaEvent_t tb, te;
       timer_begin(ctx, "hash", ctx->s_hash, &tb, &te);
-      launch_hash((int)ctx->inst, (unsigned)blocks, ctx->s_hash, a, kHashCoresident);
+      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->s_hash, a, kHashCoresident);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", ctx->s_hash, tb, te);
@@ -2977,25 +3188,17 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
   if ((rc = run_replayable(ctx, ctx->g_multi, sig, stage1))) return rc;
   uint8_t all_ok = 0;
   std::vector<uint32_t> bad(nd);
-  std::vector<uint8_t> hbadY(nd);
   CU(cudaMemcpyAsync(&all_ok, d_acc, 1, cudaMemcpyDeviceToHost, ctx->s_main));
   CU(cudaMemcpyAsync(bad.data(), ss.bad, 4 * (size_t)nd, cudaMemcpyDeviceToHost, ctx->s_main));
-  CU(cudaMemcpyAsync(hbadY.data(), badY, nd, cudaMemcpyDeviceToHost, ctx->s_main));
-  std::vector<uint8_t> hmbad(nbuild);
-  if (nbuild) CU(cudaMemcpyAsync(hmbad.data(), d_mbad, nbuild, cudaMemcpyDeviceToHost, ctx->s_main));
+  if ((rc = read_bad_keys())) return rc;
   if ((rc = check_status(ctx))) return rc;
-  for (uint32_t k = 0; k < nbuild; ++k)
-    if (hmbad[k]) hbadY[kmiss[k]] = 1;
-  for (uint32_t d = 0; d < nd; ++d)
-    if (hbadY[d]) return fail(ctx, POSLO_EINVAL, "public key of device %u does not decode", d);
-  forget.armed = false;   // the built tables are sound
+  if ((rc = check_keys())) return rc;
   uint64_t total_bad = 0;
   for (uint32_t d = 0; d < nd; ++d) total_bad += bad[d];
   std::vector<uint8_t> flag(nd, 0);
   if (!(all_ok && total_bad == 0)) {
     // ---- localisation across devices: unit check per device, then confirm the rest together
-    k_device_unit_check<<<(unsigned)((4ull * nd + 127) / 128), 128, 0, ctx->s_main>>>(d_tabs, ss, nd, ctx->tableG,
-                                                                                     dev_flag);
+    launch_device_unit_check(ctx->s_main, d_tabs, ss, nd, ctx->tableG, dev_flag);
     // the weighted sum over the devices not flagged = P1 minus the flagged devices' part,
     // an MSM over their entries only
     k_device_to_entries<<<nd, 256, 0, ctx->s_main>>>(dev_flag, seg_start, badR, eskip, 1);
@@ -3057,21 +3260,12 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
     CU(cudaMemsetAsync(inv, 0, N1, ctx->s_main));
     cudaEvent_t tb, te;
     timer_begin(ctx, "localise", ctx->s_main, &tb, &te);
-    MultiCheckArgs ca{};
-    ca.pts = pts;
-    ca.e = d_e;
-    ca.s = sb.s;
-    ca.badR = badR;
-    ca.badS = badS;
-    ca.seg_start = seg_start;
     ca.fl = d_fl;
     ca.fstart = d_fst;
     ca.nfl = nfl;
-    ca.tabs = d_tabs;
-    ca.tableG = ctx->tableG;
     ca.inv = inv;
     if (fst[nfl] && fst[nfl] <= kMultiGroupCheckMax)
-      k_multi_entry_check_group<<<(unsigned)((8 * fst[nfl] + 127) / 128), 128, 0, ctx->s_main>>>(ca);
+      launch_multi_entry_check_lanes(ctx->s_main, ca, fst[nfl]);
     else if (fst[nfl])
       k_multi_entry_check<<<grid_for(ctx, fst[nfl], 128, 8), 128, 0, ctx->s_main>>>(ca);
     k_segment_any<<<nfl, 256, 0, ctx->s_main>>>(inv, seg_start, d_fl, d_any);
@@ -3089,13 +3283,7 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
     if (got && invalid_pairs) {
       std::vector<uint64_t> g(got);
       CU(cudaMemcpy(g.data(), d_idx, 8 * got, cudaMemcpyDeviceToHost));
-      // global positions ascend, and so do devices: walk the device table once
-      uint32_t d = 0;
-      for (uint64_t q = 0; q < got; ++q) {
-        while (mb->dev_start[d + 1] <= g[q]) ++d;
-        invalid_pairs[2 * q] = d;
-        invalid_pairs[2 * q + 1] = mb->first_index[d] + (g[q] - mb->dev_start[d]);
-      }
+      write_pairs(g.data(), got);
     }
   }
   *n_invalid = cnt;
