@@ -793,11 +793,13 @@ __global__ void __launch_bounds__(32) k_msm_final(const uint32_t* groups, MsmPla
 __global__ void __launch_bounds__(32) k_msm_windows(const uint32_t* groups, MsmPlan pl, uint32_t* W);
 __global__ void __launch_bounds__(32) k_msm_window_check(const uint32_t* groups, MsmPlan pl, const uint32_t* Pw,
                                                          const uint32_t* bad, const uint32_t* point_bad,
-                                                         const uint32_t* status, uint8_t* accept);
+                                                         const uint32_t* status, uint32_t* W, uint8_t* accept);
 constexpr int kWindowThreads = 128;
 __global__ void __launch_bounds__(kWindowThreads) k_window_sums(const uint8_t* e, const uint8_t* s, const uint32_t* z,
-                                                                uint64_t n, MsmPlan pl, unsigned long long* partial);
+                                                                const uint64_t* idx, uint64_t n, MsmPlan pl,
+                                                                unsigned long long* partial);
 __global__ void __launch_bounds__(kWindowThreads) k_window_prep(const unsigned long long* partial, uint32_t nblocks,
+                                                                const unsigned long long* less, uint32_t nless,
                                                                 const unsigned long long* hash_partial, uint32_t nhash,
                                                                 const uint32_t* tableY, const uint32_t* tableG,
                                                                 uint32_t* Pw, uint32_t* bad);
@@ -815,13 +817,23 @@ struct BisectState {
 // Resident blocks per SM the descent is compiled for (its checks are latency-bound chains of
 // point additions: more warps per SM hide more of it, at the cost of registers).
 #ifndef POSLO_BISECT_MINB
-#define POSLO_BISECT_MINB 2
+#define POSLO_BISECT_MINB 3
 #endif
-#ifndef POSLO_BISECT_WAVES
-#define POSLO_BISECT_WAVES 1   // the descent's grid: this many waves of resident blocks
-#endif
+// Levels a step descends from F failing nodes at level l: as many as keep the checks within
+// slots, at least one (and at most l).
+__host__ __device__ inline int bisect_depth(uint64_t F, int l, uint64_t slots) {
+  int j = 1;
+  while (j < l && (F << (j + 1)) <= slots) ++j;
+  return j;
+}
 __global__ void __launch_bounds__(128, POSLO_BISECT_MINB) k_bisect_step(const TreeArgs a, BisectState st, int step,
-                                                     const uint32_t* tY, const uint32_t* tG, uint8_t* invalid);
+                                                     uint64_t slots, const uint32_t* tY, const uint32_t* tG,
+                                                     uint8_t* invalid);
+__global__ void __launch_bounds__(128) k_flagged_windows(const uint32_t* pts, const uint32_t* z, const uint8_t* badR,
+                                                         const uint64_t* idx, uint64_t cnt, MsmPlan pl,
+                                                         uint32_t* partial);
+__global__ void __launch_bounds__(32) k_confirm_windows(const uint32_t* W, const uint32_t* F, const uint32_t* Pw,
+                                                        int windows, uint8_t* accept);
 __global__ void k_gather_flagged(const uint32_t* pts, const uint32_t* z, const uint8_t* badR, const uint64_t* idx,
                                  uint64_t cnt, uint32_t* gp, uint32_t* gz, uint8_t* gs);
 __global__ void k_point_diff(const uint32_t* a, const uint32_t* b, uint32_t* out);
@@ -936,6 +948,9 @@ __global__ void k_noncanonical(const uint8_t* s, uint64_t n, uint8_t* bad);
 __global__ void k_offs_sub(uint64_t* offs, uint64_t n, uint64_t base);
 __global__ void k_device_to_entries(const uint8_t* dev_flag, const uint64_t* start, const uint8_t* badR,
                                     uint8_t* skip, int keep_flagged);
+// out[i] = first_index + list[i] for the first min(*count, cap) entries of a list.
+__global__ void k_shift_list(const uint64_t* list, const uint64_t* count, uint64_t cap, uint64_t first_index,
+                             uint64_t* out);
 constexpr uint32_t kFlagChunk = 8192;
 __global__ void __launch_bounds__(1024) k_flag_count(const uint8_t* flags, uint64_t n, uint32_t* blockcnt);
 __global__ void __launch_bounds__(1024) k_flag_scan(const uint32_t* blockcnt, uint32_t nblocks, uint64_t* blockoff,

@@ -85,6 +85,7 @@ struct poslo_ctx {
   cudaEvent_t ev_table = nullptr, ev_points = nullptr, ev_main = nullptr, ev_hash = nullptr, ev_prep = nullptr;
   cudaEvent_t ev_decoded = nullptr;   // points stream, right after the decoding (before its sums)
   cudaEvent_t ev_staged = nullptr;   // main stream, right after a batch's R_t have been staged
+  cudaEvent_t ev_result = nullptr;   // the list of flagged entries and ccd^v are complete
   std::map<std::string, poslo_host::DevBuf> bufs;
   uint32_t* tableG = nullptr;     // fixed-window table of G (64 KiB)
   uint32_t* status = nullptr;     // device status word

@@ -229,6 +229,12 @@ __global__ void k_encode_ext(const uint32_t* point, uint8_t* out) {
   }
 }
 
+__global__ void k_shift_list(const uint64_t* list, const uint64_t* count, uint64_t cap, uint64_t first_index,
+                             uint64_t* out) {
+  const uint64_t n = min(*count, cap), stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) out[i] = first_index + list[i];
+}
+
 // Ordered compaction across many blocks: block b owns flags [b*kFlagChunk, (b+1)*kFlagChunk).
 // Pass 1 counts, pass 2 scans the counts (one block), pass 3 writes first_index + t of
 // every flagged t in ascending order.

@@ -77,130 +77,70 @@ __global__ void __launch_bounds__(128) k_tree_level(const TreeArgs a, uint64_t i
   sc_store(a.tree_s + 32 * o, sc_add(sc_load(a.tree_s + 32 * c0), sc_load(a.tree_s + 32 * c1)));
 }
 
-// Lane l's two signed 4-bit digits (windows 2l and 2l+1) of the recoding of sc_digit4, with
-// the carries of the lower windows from a warp scan instead of a walk over them: a window
-// generates a carry when its nibble is 8 or more and propagates the incoming one when it is
-// 7, so the carry into lane l is the scan of (generate, propagate) over lanes 0 .. l-1.
-__device__ __forceinline__ void lane_digits(const uint32_t k[8], int lane, int& d0, int& d1) {
-  uint32_t word = 0;                                         // windows 2l, 2l+1 = byte (l & 3) of word l / 4
-#pragma unroll
-  for (int i = 0; i < 8; ++i) word = i == (lane >> 2) ? k[i] : word;   // (no dynamic register index)
-  const int n0 = (int)((word >> (8 * (lane & 3))) & 15u), n1 = (int)((word >> (8 * (lane & 3) + 4)) & 15u);
-  uint32_t G = (n1 >= 8) | ((n1 == 7) & (n0 >= 8)), P = (n1 == 7) & (n0 == 7);
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t Gp = __shfl_up_sync(0xffffffffu, G, o), Pp = __shfl_up_sync(0xffffffffu, P, o);
-    if (lane >= o) {
-      G = G | (P & Gp);
-      P = P & Pp;
+// The checks of one pass: w = 0 .. total - 1, LANES lanes each (check_lanes).  Check w is of
+// descendant (w mod 2^j) of failing node fail_in[w >> j], at level tl.  The loop runs the same
+// number of times for all lanes of a warp (the checks shuffle across the warp); a group past
+// the end repeats a node and records nothing.
+template <int LANES>
+__device__ __forceinline__ void bisect_pass(const TreeArgs& a, const uint64_t* fail_in, uint64_t total, int j, int tl,
+                                            const uint32_t* tY, const uint32_t* tG, uint64_t* fail_out,
+                                            unsigned long long* cnt_out, uint8_t* invalid) {
+  constexpr int kPerWarp = 32 / LANES;
+  const uint64_t mask = (1ull << j) - 1;
+  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  const uint32_t grp = (threadIdx.x & 31) / LANES;
+#pragma unroll 1
+  for (uint64_t w0 = kPerWarp * warp; w0 < total; w0 += kPerWarp * nwarps) {
+    const uint64_t w = w0 + grp;
+    bool live = w < total;
+    const uint64_t wc = live ? w : total - 1;
+    const uint64_t k = (fail_in[wc >> j] << j) | (wc & mask);
+    ge P;
+    const uint8_t *e, *s;
+    if (tl > 0) {
+      const uint64_t node = a.M - (a.M >> (tl - 1)) + k;   // levels 1 .. tl-1 hold M/2 + ... + M/2^(tl-1) nodes
+      P = ge_load4(a.tree_pts + 32 * node);
+      e = a.tree_e + 32 * node;
+      s = a.tree_s + 32 * node;
+    } else {
+      // malformed entries are flagged already; padding leaves hold nothing
+      live = live && k < a.n && !flagged(a.skip1, a.skip2, k);
+      const uint64_t t = k < a.n ? k : a.n - 1;
+      fe t2d;
+      pts_load(a.pts + (size_t)kPtsWords * t, P.X, P.Y, t2d);
+      P.Z = fe_one();
+      P.T = fe_mul(P.X, P.Y);
+      e = a.e + 32 * t;
+      s = a.s + 32 * t;
+    }
+    const bool ok = check_lanes<LANES>(e, s, P, tY, tG);
+    if (live && !ok && (threadIdx.x & (LANES - 1)) == 0) {
+      if (tl > 0) fail_out[atomicAdd(cnt_out, 1ull)] = k;
+      else invalid[k] = 1;
     }
   }
-  const uint32_t up = __shfl_up_sync(0xffffffffu, G, 1);
-  int carry = lane ? (int)up : 0;
-  d0 = n0 + carry;
-  carry = d0 >= 8 ? 1 : 0;
-  d0 -= carry << 4;
-  d1 = n1 + carry;
-  d1 -= (d1 >= 8 ? 1 : 0) << 4;
-}
-
-// [8](P - eY - sG) = O evaluated by one warp: lane l adds the table terms of windows 2l and
-// 2l+1, a shuffle tree sums the 32 partial points.  Every lane returns the same answer.
-__device__ __forceinline__ bool warp_check(const ge& P, const sc& e, const sc& s, const uint32_t* tY,
-                                           const uint32_t* tG) {
-  const int lane = threadIdx.x & 31;
-  const int w0 = 2 * lane, w1 = w0 + 1;
-  int de0, de1, ds0, ds1;
-  lane_digits(e.v, lane, de0, de1);
-  lane_digits(s.v, lane, ds0, ds1);
-  ge acc = ge_add(table_pick(tY, w0, de0), table_pick(tY, w1, de1));
-  acc = ge_add(acc, table_pick(tG, w0, ds0));
-  acc = ge_add(acc, table_pick(tG, w1, ds1));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    ge other;
-    other.X = fe_shfl(acc.X, lane ^ o); other.Y = fe_shfl(acc.Y, lane ^ o);
-    other.Z = fe_shfl(acc.Z, lane ^ o); other.T = fe_shfl(acc.T, lane ^ o);
-    acc = ge_add(acc, other);
-  }
-  return ge_is_identity(ge_mul_cofactor(ge_sub(P, acc)));
-}
-
-// [8](P - eY - sG) = O evaluated by a group of 8 lanes (lanes 8g .. 8g+7 of the warp hold the
-// same P, e, s; four groups check four nodes at once).  Lane r of the group takes word r of
-// each scalar, i.e. the 8 windows 8r .. 8r+7: it recodes them into signed 4-bit digits (the
-// carry into its first window from a scan over the group's lower lanes, as in lane_digits),
-// adds their 16 table terms, and a shuffle tree over the group sums the 8 partial points.
-// Fewer lanes per check than warp_check, so fewer instructions per check: each lane's chain is
-// longer (15 additions instead of 3), but the work of the tree and of the final check is shared
-// by 8 lanes instead of 32.  Every lane of the group returns the same answer.
-__device__ __forceinline__ void group8_digits(uint32_t word, int r, int8_t d[8]) {
-  uint32_t G = 0, Pp = 1;   // carry out of this lane's 8 windows with no carry in; all-7 propagate
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const uint32_t n = (word >> (4 * i)) & 15u;
-    G = (n >= 8) | ((n == 7) & G);
-    Pp &= (n == 7);
-  }
-#pragma unroll
-  for (int o = 1; o < 8; o <<= 1) {
-    const uint32_t Gu = __shfl_up_sync(0xffffffffu, G, o, 8), Pu = __shfl_up_sync(0xffffffffu, Pp, o, 8);
-    if (r >= o) {
-      G = G | (Pp & Gu);
-      Pp = Pp & Pu;
-    }
-  }
-  const uint32_t up = __shfl_up_sync(0xffffffffu, G, 1, 8);
-  int carry = r ? (int)up : 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    int v = (int)((word >> (4 * i)) & 15u) + carry;
-    carry = v >= 8 ? 1 : 0;
-    d[i] = (int8_t)(v - (carry << 4));
-  }
-}
-
-__device__ __forceinline__ bool group8_check(const ge& P, const sc& e, const sc& s, const uint32_t* tY,
-                                             const uint32_t* tG) {
-  const int lane = threadIdx.x & 31, r = lane & 7;
-  uint32_t we = 0, ws = 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {   // word r of each scalar (no dynamic register index)
-    we = i == r ? e.v[i] : we;
-    ws = i == r ? s.v[i] : ws;
-  }
-  int8_t dg[16];   // the 8 digits of e, then the 8 of s
-  group8_digits(we, r, dg);
-  group8_digits(ws, r, dg + 8);
-  // loops, not unrolled: one copy of the point addition in the code keeps the kernel inside
-  // the instruction cache (unrolled, the warps stalled mostly on instruction fetch)
-  ge acc = ge_identity();
-#pragma unroll 1
-  for (int i = 0; i < 16; ++i) acc = ge_add(acc, table_pick(i < 8 ? tY : tG, 8 * r + (i & 7), dg[i]));
-#pragma unroll 1
-  for (int o = 4; o > 0; o >>= 1) {
-    ge other;
-    other.X = fe_shfl(acc.X, lane ^ o); other.Y = fe_shfl(acc.Y, lane ^ o);
-    other.Z = fe_shfl(acc.Z, lane ^ o); other.T = fe_shfl(acc.T, lane ^ o);
-    acc = ge_add(acc, other);
-  }
-  return ge_is_identity(ge_mul_cofactor(ge_sub(P, acc)));
 }
 
 // One step of the descent, several levels at a time.  The step reads the failing nodes of
 // level l (state.fail[s % 3], count state.cnt[s % 3], level state.level[s % 2]) and checks
-// their descendants j levels further down, j the largest depth for which all of them fit in
-// one pass of the grid's check slots (4 per warp; at least 1, at most l): with few failing nodes a step jumps
-// many levels, with many it descends one.  Failing descendants go to the next list
+// their descendants j levels further down, j from bisect_depth: with few failing nodes a step
+// jumps many levels, with many it descends one.  Failing descendants go to the next list
 // (state.fail[(s+1) % 3]); at level 0 the descendants are entries, checked on their own, and
 // failing ones are marked invalid.  Each step also clears the counter the step after it will
 // fill, and block 0 publishes the level it reached; a step that starts at level 0 (done)
-// returns at once, so the host issues as many steps as the tree has levels without reading
-// anything back.  Checking the descendants of a failing node directly, instead of its
-// children first, only adds checks of nodes whose ancestors failed: every entry that fails
-// its own check is still found, and entries are flagged only by their own check.
+// returns at once, so the host issues as many steps as there can be without reading anything
+// back.  Checking the descendants of a failing node directly, instead of its children first,
+// only adds checks of nodes whose ancestors failed: every entry that fails its own check is
+// still found, and entries are flagged only by their own check.
+//
+// A step takes 59 us for 640 checks and about 100 us for 2,048 to 3,700 (throughput of the
+// point additions); as many lanes per check as the grid has for their number keep the latency
+// short (one lane's 16 additions in groups of 8 lanes before: 100 to 120 us a step also with 160
+// checks).
 __global__ void __launch_bounds__(128, POSLO_BISECT_MINB) k_bisect_step(const TreeArgs a, BisectState st, int step,
-                                                     const uint32_t* tY, const uint32_t* tG, uint8_t* invalid) {
+                                                     uint64_t slots, const uint32_t* tY, const uint32_t* tG,
+                                                     uint8_t* invalid) {
   const int l = st.level[step & 1];
   const uint64_t* fail_in = st.fail[step % 3];
   uint64_t* fail_out = st.fail[(step + 1) % 3];
@@ -211,41 +151,76 @@ __global__ void __launch_bounds__(128, POSLO_BISECT_MINB) k_bisect_step(const Tr
     return;
   }
   const uint64_t F = st.cnt[step % 3];
-  // four checks per warp (one per group of 8 lanes)
-  const uint64_t slots = ((uint64_t)gridDim.x * blockDim.x) >> 3;
-  int j = 1;
-  while (j < l && (F << (j + 1)) <= slots) ++j;
+  const int j = bisect_depth(F, l, slots);
   const int tl = l - j;
   if (blockIdx.x == 0 && threadIdx.x == 0) st.level[(step + 1) & 1] = tl;
-  const uint64_t total = F << j;
-  const uint64_t mask = (1ull << j) - 1;
-  // the loop runs the same number of times for all lanes of a warp (the check shuffles across
-  // the warp); a group past the end checks the identity and records nothing
-  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  const uint32_t grp = (threadIdx.x & 31) >> 3;
-  for (uint64_t w0 = 4 * warp; w0 < total; w0 += 4 * nwarps) {
-    const uint64_t w = w0 + grp;
-    const bool live = w < total;
-    const uint64_t k = live ? ((fail_in[w >> j] << j) | (w & mask)) : 0;
-    ge P = ge_identity();
-    sc e = sc_zero(), s = sc_zero();
-    if (live) {
-      if (tl > 0) {
-        const uint64_t node = a.M - (a.M >> (tl - 1)) + k;   // levels 1 .. tl-1 hold M/2 + ... + M/2^(tl-1) nodes
-        P = ge_load(a.tree_pts + 32 * node);
-        e = sc_load(a.tree_e + 32 * node);
-        s = sc_load(a.tree_s + 32 * node);
-      } else {
-        leaf(a, k, P, e, s);
-      }
+  const uint64_t total = F << j, threads = (uint64_t)gridDim.x * blockDim.x;
+  if (total == 0) return;
+  if (32 * total <= threads) bisect_pass<32>(a, fail_in, total, j, tl, tY, tG, fail_out, cnt_out, invalid);
+  else if (16 * total <= threads) bisect_pass<16>(a, fail_in, total, j, tl, tY, tG, fail_out, cnt_out, invalid);
+  else bisect_pass<8>(a, fail_in, total, j, tl, tY, tG, fail_out, cnt_out, invalid);
+}
+
+// Confirmation of a few flagged entries, point side: F_w = sum of d_{t,w} R_t over the flagged
+// entries idx[0 .. cnt) whose point decodes, d_{t,w} the MSM's signed digit of window w
+// (blockIdx.y).  One quad per (entry, window): |d| R by double-and-add over c bits (the same
+// steps for every quad), negated for a negative digit; per block a partial sum (decode
+// partial format).  Latency-bound: c doublings and additions, about 30 us, instead of an MSM over
+// the flagged entries whose windows Horner's rule then joins (280 us).
+__global__ void __launch_bounds__(128) k_flagged_windows(const uint32_t* pts, const uint32_t* z, const uint8_t* badR,
+                                                         const uint64_t* idx, uint64_t cnt, MsmPlan pl,
+                                                         uint32_t* partial) {
+  const int w = blockIdx.y;
+  const uint32_t quad = threadIdx.x >> 2, nq = blockDim.x >> 2;
+  ge sum = ge_identity();
+  // block-uniform trip count (quad operations need every lane)
+  for (uint64_t i0 = (uint64_t)blockIdx.x * nq; i0 < cnt; i0 += (uint64_t)gridDim.x * nq) {
+    const uint64_t i = i0 + quad;
+    const uint64_t t = idx[i < cnt ? i : cnt - 1];
+    bool neg;
+    uint32_t d = weight_digit(z, t, w, pl.c, neg);
+    if (i >= cnt || (badR && badR[t])) d = 0;
+    ge P;
+    fe t2d;
+    pts_load(pts + (size_t)kPtsWords * t, P.X, P.Y, t2d);
+    P.Z = fe_one();
+    P.T = fe_mul(P.X, P.Y);
+    if (neg) P = ge_neg(P);
+    ge acc = ge_identity();
+#pragma unroll 1
+    for (int bit = pl.c - 1; bit >= 0; --bit) {
+      acc = ge_dbl_quad(acc);
+      const ge more = ge_add_quad(acc, P);
+      acc = ge_select(acc, more, ((d >> bit) & 1u) != 0);
     }
-    const bool ok = group8_check(P, e, s, tY, tG);
-    if (live && !ok && (threadIdx.x & 7) == 0) {
-      if (tl > 0) fail_out[atomicAdd(cnt_out, 1ull)] = k;
-      else if (k < a.n) invalid[k] = 1;
-    }
+    sum = ge_add_quad(sum, acc);
   }
+  __shared__ uint32_t sp[32][32];
+  if ((threadIdx.x & 3) == 0) ge_store(sp[quad], sum);
+  compact::quad_tree(sp, 32);
+  const size_t o = ((size_t)w * gridDim.x + blockIdx.x) * kPointPartialWords;
+  if (threadIdx.x < 32) partial[o + threadIdx.x] = sp[0][threadIdx.x];
+  if (threadIdx.x == 0) partial[o + 32] = 0;
+}
+
+// Confirmation of a few flagged entries: for every window w
+//   [8](W_w - F_w - P_w) = O
+// with W_w the whole batch's window sum (left by k_msm_window_check), F_w the flagged entries'
+// and P_w = [E'_w] Y + [S'_w] G over the others (k_window_prep).  One warp, a quad per window;
+// the windows together imply the check with the full weights.
+__global__ void __launch_bounds__(32) k_confirm_windows(const uint32_t* W, const uint32_t* F, const uint32_t* Pw,
+                                                        int windows, uint8_t* accept) {
+  const int lane = threadIdx.x & 31, quad = lane >> 2;
+  bool ok = true;
+#pragma unroll 1
+  for (int r0 = 0; r0 < windows; r0 += 8) {
+    const int w = r0 + quad, wc = w < windows ? w : windows - 1;
+    const ge d = ge_add_quad(ge_load(W + 32 * (size_t)wc), ge_neg(ge_load(F + 32 * (size_t)wc)));
+    const bool eq = compact::quad_equal(d, ge_load(Pw + 32 * (size_t)wc));
+    if (w < windows) ok = ok && eq;
+  }
+  const bool all = __all_sync(0xffffffffu, ok);
+  if (lane == 0) *accept = all ? 1 : 0;
 }
 
 // The flagged entries' rows for the MSM of the confirmation: decoded point (kPtsWords words),

@@ -372,17 +372,18 @@ __global__ void __launch_bounds__(32) k_msm_windows(const uint32_t* groups, MsmP
 
 // Per-window weighted check, group side: quad w forms the window sum W_w and tests
 // [8](W_w - P_w) = O against P_w = [E_w] Y + [S_w] G (k_window_prep); windows are processed in
-// rounds of eight quads.  accept = every window holds, no malformed s (*bad), no undecodable
+// rounds of eight quads.  The window sums go to W (a confirmation needs them).  accept = every window holds, no malformed s (*bad), no undecodable
 // R (*point_bad) and a decodable key.  One warp.
 __global__ void __launch_bounds__(32) k_msm_window_check(const uint32_t* groups, MsmPlan pl, const uint32_t* Pw,
                                                          const uint32_t* bad, const uint32_t* point_bad,
-                                                         const uint32_t* status, uint8_t* accept) {
+                                                         const uint32_t* status, uint32_t* W, uint8_t* accept) {
   const int lane = threadIdx.x & 31, quad = lane >> 2;
   bool ok = true;
   for (int r0 = 0; r0 < pl.windows; r0 += 8) {
     const int w = r0 + quad;
     const int wc = w < pl.windows ? w : pl.windows - 1;
     const ge acc = window_sum_quad(groups, pl, wc);
+    if ((lane & 3) == 0 && w < pl.windows) ge_store(W + 32 * (size_t)w, acc);
     ge diff = ge_add_quad(acc, ge_neg(ge_load(Pw + 32 * (size_t)wc)));
     for (int i = 0; i < 3; ++i) diff = ge_dbl_quad(diff);   // cofactor 8
     if (w < pl.windows) ok = ok && ge_is_identity(diff);

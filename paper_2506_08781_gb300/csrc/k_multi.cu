@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(kPointThreads) k_window_point_sums(const uint3
     acc = ge_add(acc, ge_load(partial + ((size_t)w * nblocks + b) * kPointPartialWords));
   __shared__ uint32_t sp[kPointThreads][32];
   ge_store(sp[threadIdx.x], acc);
-  compact::quad_tree(sp, kPointThreads);
+  compact::quad_tree(sp, nblocks < kPointThreads ? (int)nblocks : kPointThreads);
   if (threadIdx.x < 32) out[32 * (size_t)w + threadIdx.x] = sp[0][threadIdx.x];
 }
 

@@ -488,14 +488,15 @@ __global__ void __launch_bounds__(128) k_final_prep(const PrepArgs a) {
 // a negative one, into exact 416-bit accumulators; per block 13 limb sums of E_w and 13 of
 // S_w (26 u64 at partial[(w * gridDim.x + blockIdx.x) * 26]).
 __global__ void __launch_bounds__(kWindowThreads) k_window_sums(const uint8_t* e, const uint8_t* s, const uint32_t* z,
-                                                                uint64_t n, MsmPlan pl,
+                                                                const uint64_t* idx, uint64_t n, MsmPlan pl,
                                                                 unsigned long long* partial) {
   const int w = blockIdx.y;
   acc13 ae, as;
   acc_zero(ae);
   acc_zero(as);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += stride) {
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const uint64_t t = idx ? idx[i] : i;   // all entries, or the n listed ones
     bool neg;
     const uint32_t d = weight_digit(z, t, w, pl.c, neg);
     if (d) add_window_terms(ae, as, e + 32 * t, s + 32 * t, d, neg);
@@ -516,32 +517,43 @@ __global__ void __launch_bounds__(kWindowThreads) k_window_sums(const uint8_t* e
   }
 }
 
-// One block per window: E_w and S_w from the partials of k_window_sums, then
+// One block per window: E_w and S_w from the partials of k_window_sums (minus those of `less`,
+// when given: the sums over a few entries left out), then
 // P_w = [E_w] Y + [S_w] G from the two window tables (128 terms, shared-memory tree) into
 // Pw[w] (32 words).  Block 0 also writes the malformed-s flag of the hashing partials to *bad.
 __global__ void __launch_bounds__(kWindowThreads) k_window_prep(const unsigned long long* partial, uint32_t nblocks,
+                                                                const unsigned long long* less, uint32_t nless,
                                                                 const unsigned long long* hash_partial, uint32_t nhash,
                                                                 const uint32_t* tableY, const uint32_t* tableG,
                                                                 uint32_t* Pw, uint32_t* bad) {
-  __shared__ unsigned long long sums[26];
+  __shared__ unsigned long long sums[2][26];
   __shared__ int8_t dig_e[64], dig_s[64];
   __shared__ uint32_t pts_[kWindowThreads][32];
   const int w = blockIdx.x, tid = threadIdx.x;
-  if (tid < 26) {
-    unsigned long long v = 0;
-    for (uint32_t b = 0; b < nblocks; ++b) v += partial[((size_t)w * nblocks + b) * 26 + tid];
-    sums[tid] = v;
+  if (tid < 52) sums[tid / 26][tid % 26] = 0;
+  __syncthreads();
+  // word k of every block's partial, the blocks split over four lanes per word
+  for (int h = 0; h < 2; ++h) {
+    const unsigned long long* src = h ? less : partial;
+    const uint32_t nb = h ? nless : nblocks;
+    if (src && tid < 4 * 26) {
+      unsigned long long v = 0;
+      for (uint32_t b = tid / 26; b < nb; b += 4) v += src[((size_t)w * nb + b) * 26 + tid % 26];
+      atomicAdd(&sums[h][tid % 26], v);
+    }
   }
-  if (w == 0 && tid == 32) {
+  if (w == 0 && hash_partial && tid >= 32 && tid < 64) {
     unsigned long long v = 0;
-    for (uint32_t b = 0; b < nhash; ++b) v += hash_partial[(size_t)b * kPartialWords + 26];
-    *bad = v != 0 ? 1u : 0u;
+    for (uint32_t b = tid - 32; b < nhash; b += 32) v += hash_partial[(size_t)b * kPartialWords + 26];
+    warp_sum_u64(v);
+    if (tid == 32) *bad = v != 0 ? 1u : 0u;
   }
   __syncthreads();
-  if (tid == 0) {
-    const sc E = limb_sums_to_scalar(sums), S = limb_sums_to_scalar(sums + 13);
-    recode4(E.v, dig_e);
-    recode4(S.v, dig_s);
+  if (tid < 64 && (tid & 31) == 0) {   // E_w by one warp, S_w by another
+    const int o = tid ? 13 : 0;
+    sc x = limb_sums_to_scalar(sums[0] + o);
+    if (less) x = sc_sub(x, limb_sums_to_scalar(sums[1] + o));
+    recode4(x.v, tid ? dig_s : dig_e);
   }
   __syncthreads();
   const ge term = tid < 64 ? table_pick(tableY, tid, dig_e[tid]) : table_pick(tableG, tid - 64, dig_s[tid - 64]);

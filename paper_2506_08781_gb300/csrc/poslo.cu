@@ -345,6 +345,9 @@ constexpr uint64_t kDirectCheckMax = 16384;
 // Distill of a valid batch 300 / 186 at 1,024 entries, 297 / 254 at 4,096, 305 / 304 at 6,000,
 // 308 / 374 at 8,192, with flips 510 / 199 at 1,024, 568 / 287 at 4,096; many signers with one
 // flipped entry 1,252 / 209 at 300 entries, 1,344 / 382 at 5,000, 1,418 / 512 at 8,000.
+// Flagged entries up to which a confirmation subtracts them window by window (one quad per
+// entry and window) instead of by an MSM over them and Horner's rule over the windows.
+constexpr uint64_t kConfirmWindowsMax = 4096;
 constexpr uint64_t kDirectFirstMax = 4096;        // Distill
 constexpr uint64_t kMultiDirectFirstMax = 8192;   // many signers
 static_assert(kDirectFirstMax <= kDirectCheckMax && kMultiDirectFirstMax <= kMultiGroupCheckMax, "sizes of the checks");
@@ -871,7 +874,11 @@ int run_prep(poslo_ctx* ctx, const unsigned long long* hpart, uint32_t nhb, cons
   return POSLO_OK;
 }
 
-// Main stream: [8](R - prep) = O and no malformed input -> accept byte.
+// Blocks per window of k_window_sums.
+unsigned window_sum_blocks(const poslo_ctx* ctx, uint64_t n, const MsmPlan& pl) {
+  return (unsigned)std::max<int>(1, grid_for(ctx, n, kWindowThreads, 4) / pl.windows);
+}
+
 // Table stream, once hashing is done: the per-window scalar sums E_w, S_w of the MSM plan pl
 // and P_w = [E_w] Y + [S_w] G for every window into Pw (32 words each), the malformed-s flag
 // into *bad; optionally the unit sum of all s_t for ccd^v; then ev_prep.
@@ -881,13 +888,13 @@ int run_prep_windows(poslo_ctx* ctx, const unsigned long long* hpart, uint32_t n
   int rc;
   CU(cudaEventRecord(ctx->ev_hash, hash_stream));
   CU(cudaStreamWaitEvent(ctx->s_table, ctx->ev_hash, 0));
-  const unsigned bx = (unsigned)std::max<int>(1, grid_for(ctx, n, kWindowThreads, 4) / pl.windows);
+  const unsigned bx = window_sum_blocks(ctx, n, pl);
   unsigned long long* wpart;
   if ((rc = ensure_t(ctx, "win_partial", (size_t)bx * pl.windows * 26 * 8, &wpart))) return rc;
   cudaEvent_t tb, te;
   timer_begin(ctx, "prep", ctx->s_table, &tb, &te);
-  k_window_sums<<<dim3(bx, (unsigned)pl.windows), kWindowThreads, 0, ctx->s_table>>>(e, s_all, z, n, pl, wpart);
-  k_window_prep<<<(unsigned)pl.windows, kWindowThreads, 0, ctx->s_table>>>(wpart, bx, hpart, nhb, tableY,
+  k_window_sums<<<dim3(bx, (unsigned)pl.windows), kWindowThreads, 0, ctx->s_table>>>(e, s_all, z, nullptr, n, pl, wpart);
+  k_window_prep<<<(unsigned)pl.windows, kWindowThreads, 0, ctx->s_table>>>(wpart, bx, nullptr, 0, hpart, nhb, tableY,
                                                                            ctx->tableG, Pw, bad);
   ctx->launch_count += 2;
   timer_end(ctx, "prep", ctx->s_table, tb, te);
@@ -904,20 +911,21 @@ int run_prep_windows(poslo_ctx* ctx, const unsigned long long* hpart, uint32_t n
   return POSLO_OK;
 }
 
-// Main stream, after the MSM's group sums: the per-window check into d_acc.
+// Main stream, after the MSM's group sums: the per-window check into d_acc, the window sums into W.
 int run_window_check(poslo_ctx* ctx, const uint32_t* groups, const MsmPlan& pl, const uint32_t* Pw,
-                     const uint32_t* bad, const uint32_t* pbad, uint8_t* d_acc) {
+                     const uint32_t* bad, const uint32_t* pbad, uint32_t* W, uint8_t* d_acc) {
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_prep, 0));
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_points, 0));
   cudaEvent_t tb, te;
   timer_begin(ctx, "finalize", ctx->s_main, &tb, &te);
-  k_msm_window_check<<<1, 32, 0, ctx->s_main>>>(groups, pl, Pw, bad, pbad, ctx->status, d_acc);
+  k_msm_window_check<<<1, 32, 0, ctx->s_main>>>(groups, pl, Pw, bad, pbad, ctx->status, W, d_acc);
   ++ctx->launch_count;
   timer_end(ctx, "finalize", ctx->s_main, tb, te);
   CU(cudaGetLastError());
   return POSLO_OK;
 }
 
+// Main stream: [8](R - prep) = O and no malformed input -> accept byte.
 int run_check(poslo_ctx* ctx, const uint32_t* prep, const uint32_t* R, const uint32_t* pbad, uint8_t* d_acc) {
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_prep, 0));
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_points, 0));
@@ -976,7 +984,8 @@ int poslo_create(const poslo_params* params, poslo_ctx** out) {
       cudaEventCreateWithFlags(&ctx->ev_main, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&ctx->ev_hash, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&ctx->ev_prep, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&ctx->ev_staged, cudaEventDisableTiming) != cudaSuccess)
+      cudaEventCreateWithFlags(&ctx->ev_staged, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&ctx->ev_result, cudaEventDisableTiming) != cudaSuccess)
     return bail(POSLO_EDEVICE);
   if (hash_kernels_init() != cudaSuccess) return bail(POSLO_EDEVICE);
   if (cudaMalloc(&ctx->status, 4) != cudaSuccess) return bail(POSLO_ENOMEM);
@@ -1028,6 +1037,7 @@ void poslo_destroy(poslo_ctx* ctx) {
   if (ctx->ev_hash) cudaEventDestroy(ctx->ev_hash);
   if (ctx->ev_prep) cudaEventDestroy(ctx->ev_prep);
   if (ctx->ev_staged) cudaEventDestroy(ctx->ev_staged);
+  if (ctx->ev_result) cudaEventDestroy(ctx->ev_result);
   if (ctx->s_main) cudaStreamDestroy(ctx->s_main);
   if (ctx->s_table) cudaStreamDestroy(ctx->s_table);
   if (ctx->s_points) cudaStreamDestroy(ctx->s_points);
@@ -1718,6 +1728,8 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
   uint32_t* Pw;   // per-window [E_w]Y + [S_w]G (32 words each), then the malformed-s flag
   if ((rc = ensure_t(ctx, "win_P", 4 * (32 * (size_t)kMsmMaxWindows + 1), &Pw))) return rc;
   uint32_t* Pw_bad = Pw + 32 * kMsmMaxWindows;
+  uint32_t* winW;   // the window sums of the first weighted check, for a confirmation
+  if ((rc = ensure_t(ctx, "win_W", 4 * 32 * (size_t)kMsmMaxWindows, &winW))) return rc;
   // window table of Y (table stream), unless cached
   auto launch_key_table = [&]() -> int {
     if (!kbuild) {
@@ -1899,7 +1911,7 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     // the windows)
     uint32_t* groups;
     if ((rc = run_msm_finish(ctx, ctx->s_main, pts, badR, ms, nullptr, &groups))) return rc;
-    if ((rc = run_window_check(ctx, groups, ms.pl, Pw, Pw_bad, pbad, d_acc))) return rc;
+    if ((rc = run_window_check(ctx, groups, ms.pl, Pw, Pw_bad, pbad, winW, d_acc))) return rc;
     return POSLO_OK;
   };
   if (replayable) {
@@ -1931,12 +1943,25 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
   }
   uint64_t* d_idx;
   const uint64_t capn = std::max<uint64_t>(std::min(cap, n), 1);
-  if ((rc = ensure_t(ctx, "invalid_idx", 8 * capn + 8, &d_idx))) return rc;
-  uint64_t* d_cnt = d_idx + capn;
+  if ((rc = ensure_t(ctx, "invalid_idx", 8 * capn, &d_idx))) return rc;
   uint64_t* fidx;   // local indices of the flagged entries (confirmation, ccd^v), count at fidx[n]
   if ((rc = ensure_t(ctx, "confirm_idx", 8 * (n + 1), &fidx))) return rc;
   uint64_t nf = 0;
   bool confirmed = false;
+  // the ordered list of flagged entries and ccd^v over the others from the local list fidx (its
+  // count on the device); ccd^v's point is the batch's unit sum (from the first stage) minus the
+  // flagged entries' points.  On st, then ev_result
+  auto launch_result = [&](cudaStream_t st) -> int {
+    k_shift_list<<<grid_for(ctx, capn, 256, 4), 256, 0, st>>>(fidx, fidx + n, std::min(cap, n), batch->first_index,
+                                                              d_idx);
+    k_sum_scalars<<<sblocks, kHashThreads, 0, st>>>(sb.s, n, inv, sp);
+    k_reduce_scalars<<<1, 256, 0, st>>>(sp, sblocks, d_ccd);
+    k_ccd_points<<<1, 256, 0, st>>>(pts, badR, fidx, fidx + n, unitR, d_ccd + 32);
+    ctx->launch_count += 4;
+    CU(cudaGetLastError());
+    CU(cudaEventRecord(ctx->ev_result, st));
+    return POSLO_OK;
+  };
   if (n <= kDirectCheckMax) {
     // ---- a small batch: every entry's own check (Fig. 4 with |m| = 1) in one launch, the
     // definition itself, instead of the tree, the descent and the confirmation, whose fixed
@@ -1962,11 +1987,18 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     if ((rc = ensure_t(ctx, "tree_pts", 128 * (M - 1), &ta.tree_pts))) return rc;
     if ((rc = ensure_t(ctx, "tree_e", 32 * (M - 1), &ta.tree_e))) return rc;
     if ((rc = ensure_t(ctx, "tree_s", 32 * (M - 1), &ta.tree_s))) return rc;
+    // the descent's grid (one wave of resident blocks), its check slots, and the level its first
+    // step goes to: the tree is built up to there
+    int bres = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bres, k_bisect_step, 128, 0) != cudaSuccess || bres < 1) bres = 1;
+    const int bgrid = ctx->sm_count * bres;
+    const uint64_t slots = (uint64_t)bgrid * 128 / 16;
+    const uint64_t top = L - (uint64_t)bisect_depth(1, (int)L, slots);
     cudaEvent_t tb, te;
     timer_begin(ctx, "tree", ctx->s_main, &tb, &te);
     k_tree_leaves<<<(unsigned)((M / 2 + 127) / 128), 128, 0, ctx->s_main>>>(ta);
     ++ctx->launch_count;
-    for (uint64_t l = 2; l <= L; ++l) {   // level l from level l - 1 (node (l, k) at M - (M >> (l - 1)) + k)
+    for (uint64_t l = 2; l <= top; ++l) {   // level l from level l - 1 (node (l, k) at M - (M >> (l - 1)) + k)
       const uint64_t count = M >> l;
       k_tree_level<<<(unsigned)((count + 127) / 128), 128, 0, ctx->s_main>>>(ta, M - (M >> (l - 2)),
                                                                              M - (M >> (l - 1)), count);
@@ -1998,62 +2030,84 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     // invalid starts as the malformed entries
     k_flags_or<<<grid_for(ctx, n, 256, 4), 256, 0, ctx->s_main>>>(badR, badS, nullptr, n, inv);
     ++ctx->launch_count;
-    // POSLO_BISECT_WAVES waves of resident blocks: a step checks at most as many nodes as the
-    // grid has warps
-    int bres = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bres, k_bisect_step, 128, 0) != cudaSuccess || bres < 1) bres = 1;
-    const int bgrid = ctx->sm_count * bres * POSLO_BISECT_WAVES;
     timer_begin(ctx, "bisect", ctx->s_main, &tb, &te);
-    for (int step = 0; step < (int)L; ++step) {
-      k_bisect_step<<<bgrid, 128, 0, ctx->s_main>>>(ta, bst, step, tableY, ctx->tableG, inv);
+    for (int step = 0; step <= (int)top; ++step) {   // the first step reaches `top`, each other one at least a level
+      k_bisect_step<<<bgrid, 128, 0, ctx->s_main>>>(ta, bst, step, slots, tableY, ctx->tableG, inv);
       ++ctx->launch_count;
     }
     CU(cudaGetLastError());
     timer_end(ctx, "bisect", ctx->s_main, tb, te);
-    // ---- confirmation: weighted check of every entry not flagged ----
-    const int wblocks = grid_for(ctx, n, kHashThreads, 8);
-    unsigned long long* wpart;
-    if ((rc = ensure_t(ctx, "w_partial", (size_t)wblocks * kPartialWords * 8, &wpart))) return rc;
-    k_weighted_sums<<<wblocks, kHashThreads, 0, ctx->s_main>>>(d_e, sb.s, z, inv, nullptr, n, wpart);
-    ++ctx->launch_count;
-    uint32_t* prep;   // [e]Y + [s]G of the weighted sums, on the table stream beside the points' side
-    if ((rc = ensure_t(ctx, "confirm_prep", 4 * 33, &prep))) return rc;
-    if ((rc = run_prep(ctx, wpart, (uint32_t)wblocks, nullptr, tableY, prep, nullptr, 0, nullptr))) return rc;
-    // sum over the unflagged entries of [z_t]R_t = the whole batch's sum (Horner over the window
-    // sums the first weighted check left behind; undecodable points are not in it) minus the
-    // flagged entries' with decodable points (an MSM over the flagged entries alone)
-    {
-      timer_begin(ctx, "confirm", ctx->s_main, &tb, &te);
-      const MsmPlan pl1 = msm_plan(ctx, n, 4);
-      uint32_t *groups1, *Wc;
+    // ---- confirmation: weighted check of every entry not flagged, from the first check's sums
+    // minus the flagged entries' part; beside it (points stream) the result as it is if the
+    // confirmation holds
+    if ((rc = run_compact(ctx, inv, n, 0, fidx, n, fidx + n))) return rc;
+    CU(cudaMemcpyAsync(&nf, fidx + n, 8, cudaMemcpyDeviceToHost, ctx->s_main));
+    CU(cudaStreamSynchronize(ctx->s_main));
+    if ((rc = launch_result(ctx->s_points))) return rc;
+    timer_begin(ctx, "confirm", ctx->s_main, &tb, &te);
+    const MsmPlan pl1 = msm_plan(ctx, n, 4);
+    if (nf == 0) {
+      // nothing flagged: the equation is the one that has just failed
+      CU(cudaMemsetAsync(d_acc, 0, 1, ctx->s_main));
+    } else if (nf <= kConfirmWindowsMax) {
+      // window by window: [8](W_w - F_w - [E_w - e_w]Y - [S_w - s_w]G) = O
+      const unsigned bx = window_sum_blocks(ctx, n, pl1), bl = window_sum_blocks(ctx, nf, pl1);
+      const unsigned bf = (unsigned)std::max<uint64_t>(
+          1, std::min<uint64_t>((nf + 31) / 32, 4 * (uint64_t)ctx->sm_count / (uint64_t)pl1.windows));
+      unsigned long long *wpart, *lpart;
+      uint32_t *fpart, *Fw, *Pc;
+      if ((rc = ensure_t(ctx, "win_partial", (size_t)bx * pl1.windows * 26 * 8, &wpart))) return rc;
+      if ((rc = ensure_t(ctx, "confirm_less", (size_t)bl * pl1.windows * 26 * 8, &lpart))) return rc;
+      if ((rc = ensure_t(ctx, "confirm_fpart", 4 * kPointPartialWords * (size_t)bf * pl1.windows, &fpart))) return rc;
+      if ((rc = ensure_t(ctx, "confirm_F", 4 * 32 * (size_t)kMsmMaxWindows, &Fw))) return rc;
+      if ((rc = ensure_t(ctx, "confirm_P", 4 * 32 * (size_t)kMsmMaxWindows, &Pc))) return rc;
+      k_window_sums<<<dim3(bl, (unsigned)pl1.windows), kWindowThreads, 0, ctx->s_table>>>(d_e, sb.s, z, fidx, nf, pl1,
+                                                                                         lpart);
+      k_window_prep<<<(unsigned)pl1.windows, kWindowThreads, 0, ctx->s_table>>>(wpart, bx, lpart, bl, nullptr, 0, tableY,
+                                                                               ctx->tableG, Pc, nullptr);
+      CU(cudaEventRecord(ctx->ev_prep, ctx->s_table));
+      k_flagged_windows<<<dim3(bf, (unsigned)pl1.windows), 128, 0, ctx->s_main>>>(pts, z, badR, fidx, nf, pl1, fpart);
+      k_window_point_sums<<<(unsigned)pl1.windows, kPointThreads, 0, ctx->s_main>>>(fpart, bf, Fw);
+      CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_prep, 0));
+      k_confirm_windows<<<1, 32, 0, ctx->s_main>>>(winW, Fw, Pc, pl1.windows, d_acc);
+      ctx->launch_count += 5;
+      CU(cudaGetLastError());
+    } else {
+      // many: weighted sums over the others, and the batch's weighted sum (Horner over the
+      // window sums the first weighted check left behind; undecodable points are not in it)
+      // minus the flagged entries' with decodable points (an MSM over them alone)
+      const int wblocks = grid_for(ctx, n, kHashThreads, 8);
+      unsigned long long* wpart;
+      if ((rc = ensure_t(ctx, "w_partial", (size_t)wblocks * kPartialWords * 8, &wpart))) return rc;
+      k_weighted_sums<<<wblocks, kHashThreads, 0, ctx->s_main>>>(d_e, sb.s, z, inv, nullptr, n, wpart);
+      ++ctx->launch_count;
+      uint32_t* prep;   // [e]Y + [s]G of the weighted sums, on the table stream beside the points' side
+      if ((rc = ensure_t(ctx, "confirm_prep", 4 * 33, &prep))) return rc;
+      if ((rc = run_prep(ctx, wpart, (uint32_t)wblocks, nullptr, tableY, prep, nullptr, 0, nullptr))) return rc;
+      uint32_t *groups1, *Wc, *gp, *gz;
+      uint8_t* gs;
       if ((rc = ensure_t(ctx, "msm_groups", 128 * (size_t)pl1.windows * (1 + pl1.jbits), &groups1))) return rc;
       if ((rc = ensure_t(ctx, "confirm_pts", 4 * 96, &Wc))) return rc;
       k_msm_final<<<1, 32, 0, ctx->s_main>>>(groups1, pl1, Wc);
       ++ctx->launch_count;
-      if ((rc = run_compact(ctx, inv, n, 0, fidx, n, fidx + n))) return rc;
-      CU(cudaMemcpyAsync(&nf, fidx + n, 8, cudaMemcpyDeviceToHost, ctx->s_main));
-      CU(cudaStreamSynchronize(ctx->s_main));
-      if (nf) {
-        uint32_t *gp, *gz;
-        uint8_t* gs;
-        if ((rc = ensure_t(ctx, "confirm_gpts", 4 * kPtsWords * nf, &gp))) return rc;
-        if ((rc = ensure_t(ctx, "confirm_gz", 16 * nf, &gz))) return rc;
-        if ((rc = ensure_t(ctx, "confirm_gskip", nf, &gs))) return rc;
-        k_gather_flagged<<<(unsigned)((nf + 127) / 128), 128, 0, ctx->s_main>>>(pts, z, badR, fidx, nf, gp, gz, gs);
-        ++ctx->launch_count;
-        if ((rc = run_msm(ctx, ctx->s_main, gp, gz, 4, gs, nf, Wc + 32))) return rc;
-      }
-      k_point_diff<<<1, 32, 0, ctx->s_main>>>(Wc, nf ? Wc + 32 : nullptr, Rw);
+      if ((rc = ensure_t(ctx, "confirm_gpts", 4 * kPtsWords * nf, &gp))) return rc;
+      if ((rc = ensure_t(ctx, "confirm_gz", 16 * nf, &gz))) return rc;
+      if ((rc = ensure_t(ctx, "confirm_gskip", nf, &gs))) return rc;
+      k_gather_flagged<<<(unsigned)((nf + 127) / 128), 128, 0, ctx->s_main>>>(pts, z, badR, fidx, nf, gp, gz, gs);
+      ++ctx->launch_count;
+      if ((rc = run_msm(ctx, ctx->s_main, gp, gz, 4, gs, nf, Wc + 32))) return rc;
+      k_point_diff<<<1, 32, 0, ctx->s_main>>>(Wc, Wc + 32, Rw);
+      ++ctx->launch_count;
+      // (not run_check: its wait on the points stream's event is for a decoding launched in the
+      // same way, and this one may have run inside a replayed graph)
+      CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_prep, 0));
+      k_final_check<<<1, 32, 0, ctx->s_main>>>(prep, Rw, nullptr, ctx->status, d_acc);
       ++ctx->launch_count;
       CU(cudaGetLastError());
-      timer_end(ctx, "confirm", ctx->s_main, tb, te);
     }
-    // (not run_check: its wait on the points stream's event is for a decoding launched in the
-    // same way, and this one may have run inside a replayed graph)
-    CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_prep, 0));
-    k_final_check<<<1, 32, 0, ctx->s_main>>>(prep, Rw, nullptr, ctx->status, d_acc);
-    ++ctx->launch_count;
-    CU(cudaGetLastError());
+    timer_end(ctx, "confirm", ctx->s_main, tb, te);
+    CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_result, 0));
+    CU(cudaMemcpyAsync(hccd, d_ccd, 64, cudaMemcpyDeviceToHost, ctx->s_main));
     uint8_t conf = 0;
     CU(cudaMemcpyAsync(&conf, d_acc, 1, cudaMemcpyDeviceToHost, ctx->s_main));
     if ((rc = check_status(ctx))) return rc;
@@ -2075,24 +2129,16 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
       timer_end(ctx, "check", ctx->s_main, tb, te);
     }
   }
-  // ordered list of flagged entries and ccd^v over the others; its point is the batch's unit
-  // sum (from the first stage) minus the flagged entries' points
-  {
-    if ((rc = run_compact(ctx, inv, n, batch->first_index, d_idx, std::min(cap, n), d_cnt))) return rc;
-    k_sum_scalars<<<sblocks, kHashThreads, 0, ctx->s_main>>>(sb.s, n, inv, sp);
-    k_reduce_scalars<<<1, 256, 0, ctx->s_main>>>(sp, sblocks, d_ccd);
-    ctx->launch_count += 2;
+  uint64_t cnt = nf;
+  if (!confirmed) {
     // the per-entry checks set the flags (direct localisation, or the fallback after a failed
-    // confirmation): list them again; the count stays on the device for k_ccd_points
-    if (!confirmed && (rc = run_compact(ctx, inv, n, 0, fidx, n, fidx + n))) return rc;
-    k_ccd_points<<<1, 256, 0, ctx->s_main>>>(pts, badR, fidx, fidx + n, unitR, d_ccd + 32);
-    ++ctx->launch_count;
-    CU(cudaGetLastError());
+    // confirmation): list them now
+    if ((rc = run_compact(ctx, inv, n, 0, fidx, n, fidx + n))) return rc;
+    if ((rc = launch_result(ctx->s_main))) return rc;
+    CU(cudaMemcpyAsync(&cnt, fidx + n, 8, cudaMemcpyDeviceToHost, ctx->s_main));
+    CU(cudaMemcpyAsync(hccd, d_ccd, 64, cudaMemcpyDeviceToHost, ctx->s_main));
+    if ((rc = check_status(ctx))) return rc;
   }
-  uint64_t cnt = 0;
-  CU(cudaMemcpyAsync(&cnt, d_cnt, 8, cudaMemcpyDeviceToHost, ctx->s_main));
-  CU(cudaMemcpyAsync(hccd, d_ccd, 64, cudaMemcpyDeviceToHost, ctx->s_main));
-  if ((rc = check_status(ctx))) return rc;
   const uint64_t got = std::min(cnt, cap);
   if (got && invalid_idx) CU(cudaMemcpy(invalid_idx, d_idx, 8 * got, cudaMemcpyDeviceToHost));
   *n_invalid = cnt;
