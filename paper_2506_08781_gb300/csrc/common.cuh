@@ -276,7 +276,8 @@ __device__ __forceinline__ ge ge_load(const uint32_t* src) {
 
 
 // ----------------------------------------------------------------------------------------
-// Fixed-window tables: table[w][d-1] = d * 16^w * P for w = 0..63, d = 1..8 (k_table_*).
+// Fixed-window tables: table[w][d-1] = d * 16^w * P for w = 0..63, d = 1..8 (k_table_*), each
+// entry in cached form (Y-X, Y+X, 2Z, 2dT), 128-byte aligned.
 // ----------------------------------------------------------------------------------------
 
 
@@ -286,10 +287,39 @@ __device__ __forceinline__ void recode4(const uint32_t k[8], int8_t dig[64]) {
   for (int w = 0; w < 64; ++w) dig[w] = (int8_t)sc_digit4(k, w, carry);
 }
 
+// Entry (w, |d|) of a window table in cached form, negated for d < 0 (d != 0).
+__device__ __forceinline__ void table_entry(const uint32_t* table, int w, int d, fe& ymx, fe& ypx, fe& z2, fe& t2d) {
+  const uint4* p = reinterpret_cast<const uint4*>(table + ((size_t)w * kTableDigits + (abs(d) - 1)) * 32);
+  uint4 v[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __ldg(p + i);
+  const fe a = fe_const(v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w);
+  const fe b = fe_const(v[2].x, v[2].y, v[2].z, v[2].w, v[3].x, v[3].y, v[3].z, v[3].w);
+  z2 = fe_const(v[4].x, v[4].y, v[4].z, v[4].w, v[5].x, v[5].y, v[5].z, v[5].w);
+  const fe t = fe_const(v[6].x, v[6].y, v[6].z, v[6].w, v[7].x, v[7].y, v[7].z, v[7].w);
+  ymx = fe_select(a, b, d < 0);
+  ypx = fe_select(b, a, d < 0);
+  t2d = fe_select(t, fe_neg(t), d < 0);
+}
+
+// acc + d 16^w P from P's window table.
+__device__ __forceinline__ ge table_add(const ge& acc, const uint32_t* table, int w, int d) {
+  if (d == 0) return acc;
+  fe ymx, ypx, z2, t2d;
+  table_entry(table, w, d, ymx, ypx, z2, t2d);
+  return ge_add_cached(acc, ymx, ypx, z2, t2d);
+}
+
+// d 16^w P itself.
 __device__ __forceinline__ ge table_pick(const uint32_t* table, int w, int d) {
   if (d == 0) return ge_identity();
-  const ge p = ge_load(table + ((size_t)w * kTableDigits + (abs(d) - 1)) * 32);
-  return d < 0 ? ge_neg(p) : p;
+  fe ymx, ypx, t2d;
+  ge r;
+  table_entry(table, w, d, ymx, ypx, r.Z, t2d);
+  r.X = fe_sub(ypx, ymx);
+  r.Y = fe_add(ypx, ymx);
+  r.T = fe_mul(t2d, fe_dinv());
+  return r;
 }
 
 constexpr int kFinalThreads = 256;
@@ -339,8 +369,8 @@ __device__ __forceinline__ ge double_scalar_tables(const uint32_t e[8], const ui
   recode4(s, ds_);
   ge acc = ge_identity();
   for (int w = 0; w < 64; ++w) {
-    acc = ge_add(acc, table_pick(tableY, w, de[w]));
-    acc = ge_add(acc, table_pick(tableG, w, ds_[w]));
+    acc = table_add(acc, tableY, w, de[w]);
+    acc = table_add(acc, tableG, w, ds_[w]);
   }
   return acc;
 }
@@ -412,7 +442,7 @@ __device__ __forceinline__ ge base_mult_table(const uint32_t k[8], const uint32_
   int8_t dig[64];
   recode4(k, dig);
   ge acc = ge_identity();
-  for (int w = 0; w < 64; ++w) acc = ge_add(acc, table_pick(tableG, w, dig[w]));
+  for (int w = 0; w < 64; ++w) acc = table_add(acc, tableG, w, dig[w]);
   return acc;
 }
 
@@ -594,36 +624,35 @@ __device__ __forceinline__ void pts_load(const uint32_t* src, fe& x, fe& y, fe& 
   t2d = fe_const(v[4].x, v[4].y, v[4].z, v[4].w, v[5].x, v[5].y, v[5].z, v[5].w);
 }
 
-// A point of 32 words at a 16-byte aligned address (the window tables' entries).
-__device__ __forceinline__ ge ge_load4(const uint32_t* src) {
-  const uint4* p = reinterpret_cast<const uint4*>(src);
-  uint4 v[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __ldg(p + i);
-  ge r;
-  r.X = fe_const(v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w);
-  r.Y = fe_const(v[2].x, v[2].y, v[2].z, v[2].w, v[3].x, v[3].y, v[3].z, v[3].w);
-  r.Z = fe_const(v[4].x, v[4].y, v[4].z, v[4].w, v[5].x, v[5].y, v[5].z, v[5].w);
-  r.T = fe_const(v[6].x, v[6].y, v[6].z, v[6].w, v[7].x, v[7].y, v[7].z, v[7].w);
-  return r;
+// -R in cached form, spread over the quad, for a decoded point (kPtsWords words, which hold 2dxy)
+// and for an extended point (32 words, 16-byte aligned).
+__device__ __forceinline__ fe qp_minus_affine(const uint32_t* pts_t) {
+  fe x, y, t2d;
+  pts_load(pts_t, x, y, t2d);
+  const int q = quad_lane();
+  const fe r = fe_addsub(y, x, q == 1);                          // lane 0: y + x, lane 1: y - x
+  return fe_select(fe_select(r, fe_small(2u), q == 2), fe_neg(t2d), q == 3);
 }
 
+__device__ __forceinline__ fe qp_minus_extended(const uint32_t* p) { return qp_neg_cached(qp_cached(qp_load(p))); }
+
 // [8](R - e Y - s G) = O by LANES (8, 16 or 32) consecutive lanes of a warp, which all hold the
-// same R and scalars: the 64 terms of [e]Y and the 64 of [s]G from the two window tables are
-// cut into one run per quad (64, 32 or 16 terms), each quad adds its run with quad-cooperative
-// additions (the next entry fetched during the current addition), a shuffle tree joins the
-// quads, and every lane returns the verdict.  More lanes shorten the chain of one check (LANES =
-// 32: 15 + 3 additions), fewer save the additions of the tree and the last check, which all
-// quads compute.  Every lane of the warp must call it (full-mask shuffles).
+// same scalars and, spread over each quad, the same -R (minus_R, cached form): the 64 terms of
+// [e]Y and the 64 of [s]G from the two window tables are cut into one run per quad (64, 32 or 16
+// terms), each quad adds its run (every lane fetching its quarter of the next entry during the
+// current addition), a shuffle tree joins the quads, and every lane returns the verdict.  More
+// lanes shorten the chain of one check (LANES = 32: 15 + 3 additions), fewer save the additions
+// of the tree and the last check, which all quads compute.  Every lane of the warp must call it
+// (full-mask shuffles).
 //
 // Digits: with k' = k + sum_i 8 16^i, nibble i of k' is digit i of the signed recoding of
 // sc_digit4 plus 8 (the recoding carries exactly where adding 8 to the nibble does), so a quad
 // starts in the middle of the scalar without walking the windows below.
 template <int LANES>
-__device__ __forceinline__ bool check_lanes(const uint8_t* e32, const uint8_t* s32, const ge& R,
+__device__ __forceinline__ bool check_lanes(const uint8_t* e32, const uint8_t* s32, const fe& minus_R,
                                             const uint32_t* tableY, const uint32_t* tableG) {
   constexpr int kTerms = 512 / LANES, kWords = kTerms / 8;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, q = quad_lane();
   const int t0 = ((lane & (LANES - 1)) >> 2) * kTerms;   // first term; 64 and up are G's
   const bool g_half = t0 >= 64;
   const int w0 = t0 & 63;
@@ -641,48 +670,40 @@ __device__ __forceinline__ bool check_lanes(const uint8_t* e32, const uint8_t* s
     for (int i = kWords; i + j < 8; i += kWords) dig[j] = (w0 >> 3) == i ? k[i + j] : dig[j];
   }
   const uint32_t* row = (g_half ? tableG : tableY) + (size_t)w0 * kTableDigits * 32;
-  auto pick = [&](int i) {   // term i of the run; consumes one nibble
+  // term i of the run in cached form, the own quarter of it; consumes one nibble
+  auto pick = [&](int i) {
     const int d = (int)(dig[0] & 15u) - 8;
     dig[0] >>= 4;
     if ((i & 7) == 7) {
 #pragma unroll
       for (int j = 0; j + 1 < kWords; ++j) dig[j] = dig[j + 1];
     }
-    if (d == 0) return ge_identity();
-    const ge p = ge_load4(row + ((size_t)i * kTableDigits + (abs(d) - 1)) * 32);
-    return d < 0 ? ge_neg(p) : p;
+    if (d == 0) return fe_small(q == 3 ? 0u : q == 2 ? 2u : 1u);
+    // -P: the first two quarters exchanged, the last negated
+    const int part = d < 0 && q < 2 ? 1 - q : q;
+    const uint4* p = reinterpret_cast<const uint4*>(row + ((size_t)i * kTableDigits + (abs(d) - 1)) * 32 + 8 * part);
+    const uint4 a = __ldg(p), b = __ldg(p + 1);
+    const fe c = fe_const(a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w);
+    return d < 0 && q == 3 ? fe_neg(c) : c;
   };
-  ge acc = pick(0);
-  ge next = pick(1);
+  fe acc = qp_identity();
+  fe next = pick(0);
 #pragma unroll 1
-  for (int i = 1; i < kTerms; ++i) {
-    const ge cur = next;
+  for (int i = 0; i < kTerms; ++i) {
+    const fe cur = next;
     if (i + 1 < kTerms) next = pick(i + 1);
-    acc = ge_add_quad(acc, cur);
+    acc = qp_add_cached(acc, cur);
   }
 #pragma unroll 1
-  for (int o = 4; o < LANES; o <<= 1) {
-    ge other;
-    other.X = fe_shfl(acc.X, lane ^ o); other.Y = fe_shfl(acc.Y, lane ^ o);
-    other.Z = fe_shfl(acc.Z, lane ^ o); other.T = fe_shfl(acc.T, lane ^ o);
-    acc = ge_add_quad(acc, other);
-  }
-  ge d = ge_add_quad(R, ge_neg(acc));
-#pragma unroll 1
-  for (int i = 0; i < 3; ++i) d = ge_dbl_quad(d);
-  return ge_is_identity(d);
+  for (int o = 4; o < LANES; o <<= 1) acc = qp_add(acc, fe_shfl_xor(acc, o));
+  return qp_is_torsion(qp_add_cached(acc, minus_R));
 }
 
 // The same for a decoded point (kPtsWords words).
 template <int LANES>
 __device__ __forceinline__ bool entry_check_lanes(const uint8_t* e32, const uint8_t* s32, const uint32_t* pts_t,
                                                   bool malformed, const uint32_t* tableY, const uint32_t* tableG) {
-  ge R;
-  fe t2d;
-  pts_load(pts_t, R.X, R.Y, t2d);
-  R.Z = fe_one();
-  R.T = fe_mul(R.X, R.Y);
-  return check_lanes<LANES>(e32, s32, R, tableY, tableG) && !malformed;
+  return check_lanes<LANES>(e32, s32, qp_minus_affine(pts_t), tableY, tableG) && !malformed;
 }
 
 // Lanes per check for n checks in one launch (measured on GB300, us per launch at

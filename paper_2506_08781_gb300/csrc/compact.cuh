@@ -39,13 +39,12 @@ static __device__ __noinline__ void encode(const ge& p, uint32_t b[8]) {
   b[7] |= (x.v[0] & 1u) << 31;
 }
 
-// The sum of the n points sp[0 .. n) (32 words each, shared memory, n >= 1) into sp[0] by the
-// block's quads, one quad-cooperative addition per pair and level: about 2,200 cycles a level
-// where one lane's addition takes 6,000.  Every thread of the block calls it (full-mask
-// shuffles, barriers inside; blockDim.x a multiple of 32); the caller has stored the points.
+// The sum of the n points sp[0 .. n) (32 words each, 16-byte aligned shared memory, n >= 1) into
+// sp[0] by the block's quads, one addition per pair and level: about 2,000 cycles a level where
+// one lane's addition takes 6,000.  Every thread of the block calls it (full-mask shuffles,
+// barriers inside; blockDim.x a multiple of 32); the caller has stored the points.
 static __device__ __noinline__ void quad_tree(uint32_t (*sp)[32], int n) {
   const int quad = threadIdx.x >> 2, nq = blockDim.x >> 2;
-  const bool writer = (threadIdx.x & 3) == 0;
   __syncthreads();
 #pragma unroll 1
   while (n > 1) {
@@ -53,21 +52,18 @@ static __device__ __noinline__ void quad_tree(uint32_t (*sp)[32], int n) {
 #pragma unroll 1
     for (int k0 = 0; k0 < pairs; k0 += nq) {
       const int k = k0 + quad, c = k < pairs ? k : pairs - 1;   // surplus quads repeat the last pair, unwritten
-      const ge sum = ge_add_quad(ge_load(sp[c]), ge_load(sp[c + half]));
+      const fe sum = qp_add(qp_load(sp[c]), qp_load(sp[c + half]));
       __syncthreads();
-      if (writer && k < pairs) ge_store(sp[k], sum);
+      if (k < pairs) qp_store(sp[k], sum);
     }
     __syncthreads();
     n = half;
   }
 }
 
-// [8](a - b) = O by the quads of one warp (every lane calls it with the same points).
-static __device__ __noinline__ bool quad_equal(const ge& a, const ge& b) {
-  ge d = ge_add_quad(a, ge_neg(b));
-#pragma unroll 1
-  for (int i = 0; i < 3; ++i) d = ge_dbl_quad(d);
-  return ge_is_identity(d);
+// [8](a - b) = O for two points of 32 words, by the quads of one warp (every lane calls it).
+static __device__ __noinline__ bool quad_equal(const uint32_t* a, const uint32_t* b) {
+  return qp_is_torsion(qp_add(qp_load(a), qp_neg(qp_load(b))));
 }
 
 }  // namespace compact

@@ -24,6 +24,9 @@ __device__ __forceinline__ fe fe_d() {
 __device__ __forceinline__ fe fe_d2() {
   return fe_const(0x26b2f159u, 0xebd69b94u, 0x8283b156u, 0x00e0149au, 0xeef3d130u, 0x198e80f2u, 0x56dffce7u, 0x2406d9dcu);
 }
+__device__ __forceinline__ fe fe_dinv() {   // 1/d
+  return fe_const(0xcdc9f843u, 0x25e0f276u, 0x4279542eu, 0x0b5dd698u, 0xcdb9cf66u, 0x2b162114u, 0x14d5ce43u, 0x40907ed2u);
+}
 __device__ __forceinline__ fe fe_sqrtm1() {
   return fe_const(0x4a0ea0b0u, 0xc4ee1b27u, 0xad2fe478u, 0x2f431806u, 0x3dfbd7a7u, 0x2b4d0099u, 0x4fc1df0bu, 0x2b832480u);
 }
@@ -96,6 +99,48 @@ __device__ __forceinline__ fe fe_sub(const fe& a, const fe& b) {
         "+r"(r.v[7]), "=r"(bo)
       : "r"(k));
   r.v[0] -= bo & 38u;
+  return r;
+}
+
+// r = a + b, or a - b when neg: a + (b ^ m) + (m & 1) with m = neg ? ~0 : 0, one chain for both.
+// The carry out means "above 2^256" for a sum and "no borrow" for a difference; 38 is added or
+// subtracted accordingly, at most twice (fe_add, fe_sub).
+__device__ __forceinline__ fe fe_addsub(const fe& a, const fe& b, bool neg) {
+  const uint32_t m = neg ? 0xffffffffu : 0u;
+  fe r;
+  uint32_t c;
+  asm("add.cc.u32 %0, %9, %9;\n\t"   // carry in: bit 31 of m
+      "addc.cc.u32 %0, %10, %18;\n\t"
+      "addc.cc.u32 %1, %11, %19;\n\t"
+      "addc.cc.u32 %2, %12, %20;\n\t"
+      "addc.cc.u32 %3, %13, %21;\n\t"
+      "addc.cc.u32 %4, %14, %22;\n\t"
+      "addc.cc.u32 %5, %15, %23;\n\t"
+      "addc.cc.u32 %6, %16, %24;\n\t"
+      "addc.cc.u32 %7, %17, %25;\n\t"
+      "addc.u32 %8, 0, 0;"
+      : "=&r"(r.v[0]), "=&r"(r.v[1]), "=&r"(r.v[2]), "=&r"(r.v[3]), "=&r"(r.v[4]), "=&r"(r.v[5]), "=&r"(r.v[6]),
+        "=&r"(r.v[7]), "=&r"(c)
+      : "r"(m), "r"(a.v[0]), "r"(a.v[1]), "r"(a.v[2]), "r"(a.v[3]), "r"(a.v[4]), "r"(a.v[5]), "r"(a.v[6]),
+        "r"(a.v[7]), "r"(b.v[0] ^ m), "r"(b.v[1] ^ m), "r"(b.v[2] ^ m), "r"(b.v[3] ^ m), "r"(b.v[4] ^ m),
+        "r"(b.v[5] ^ m), "r"(b.v[6] ^ m), "r"(b.v[7] ^ m));
+  // fold: +38 (sum with carry), -38 (difference with borrow) or nothing, as a signed 256-bit word
+  const uint32_t hit = (c ^ m) & 1u;               // 1: a fold is due
+  const uint32_t k = ((38u ^ m) - m) & (0u - hit);  // 38, -38 or 0
+  const uint32_t x = m & (0u - hit);                // its upper words
+  asm("add.cc.u32 %0, %0, %9;\n\t"
+      "addc.cc.u32 %1, %1, %10;\n\t"
+      "addc.cc.u32 %2, %2, %10;\n\t"
+      "addc.cc.u32 %3, %3, %10;\n\t"
+      "addc.cc.u32 %4, %4, %10;\n\t"
+      "addc.cc.u32 %5, %5, %10;\n\t"
+      "addc.cc.u32 %6, %6, %10;\n\t"
+      "addc.cc.u32 %7, %7, %10;\n\t"
+      "addc.u32 %8, 0, 0;"
+      : "+r"(r.v[0]), "+r"(r.v[1]), "+r"(r.v[2]), "+r"(r.v[3]), "+r"(r.v[4]), "+r"(r.v[5]), "+r"(r.v[6]),
+        "+r"(r.v[7]), "=&r"(c)
+      : "r"(k), "r"(x));
+  r.v[0] += ((38u ^ m) - m) & (0u - ((c ^ x) & 1u) & (0u - hit));
   return r;
 }
 

@@ -145,61 +145,142 @@ __device__ __forceinline__ ge ge_madd_signed(const ge& p, const fe& x, const fe&
   return r;
 }
 
-// ---- quad-cooperative point operations ------------------------------------------------
-// Four consecutive lanes of a warp (a quad) hold the same point and split the field
-// multiplications of one group operation between them, then exchange the results by
-// shuffles: a doubling costs the latency of 2 multiplications instead of 8, an addition
-// 3 instead of 9.  Every lane of the warp must take part (full-mask shuffles); each quad
-// works on its own point.
-__device__ __forceinline__ fe fe_shfl(const fe& a, int src) {
-  fe r;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) r.v[i] = __shfl_sync(0xffffffffu, a.v[i], src);
+// P + Q for Q given as (Y-X, Y+X, 2Z, 2dT) ("cached" form, the window tables' entries): 8M.
+__device__ __forceinline__ ge ge_add_cached(const ge& p, const fe& ymx, const fe& ypx, const fe& z2, const fe& t2d) {
+  const fe A = fe_mul(fe_sub(p.Y, p.X), ymx);
+  const fe B = fe_mul(fe_add(p.Y, p.X), ypx);
+  const fe C = fe_mul(p.T, t2d);
+  const fe D = fe_mul(p.Z, z2);
+  const fe E = fe_sub(B, A), F = fe_sub(D, C), G = fe_add(D, C), H = fe_add(B, A);
+  ge r;
+  r.X = fe_mul(E, F); r.Y = fe_mul(G, H); r.Z = fe_mul(F, G); r.T = fe_mul(E, H);
   return r;
 }
 
-__device__ __forceinline__ ge ge_dbl_quad(const ge& p) {
-  const int lane = threadIdx.x & 31, q = lane & 3, base = lane & ~3;
-  fe in = fe_select(p.X, p.Y, q == 1);
-  in = fe_select(in, p.Z, q == 2);
-  in = fe_select(in, fe_add(p.X, p.Y), q == 3);
-  const fe sq = fe_sq(in);
-  const fe A = fe_shfl(sq, base), B = fe_shfl(sq, base + 1), Z2 = fe_shfl(sq, base + 2), S = fe_shfl(sq, base + 3);
-  const fe C = fe_add(Z2, Z2);
-  const fe E = fe_sub(fe_sub(S, A), B);
-  const fe G = fe_sub(B, A);
-  const fe F = fe_sub(G, C);
-  const fe H = fe_neg(fe_add(A, B));
-  // X3 = E F, Y3 = G H, Z3 = F G, T3 = E H
-  fe m1 = fe_select(E, G, q == 1), m2 = fe_select(F, H, q == 1);
-  m1 = fe_select(m1, F, q == 2); m2 = fe_select(m2, G, q == 2);
-  m2 = fe_select(m2, H, q == 3);
-  const fe r = fe_mul(m1, m2);
-  ge o;
-  o.X = fe_shfl(r, base); o.Y = fe_shfl(r, base + 1); o.Z = fe_shfl(r, base + 2); o.T = fe_shfl(r, base + 3);
-  return o;
+// ---- points spread over a quad --------------------------------------------------------
+// Four consecutive lanes of a warp (a quad) hold one point: lane q has coordinate q of
+// (X, Y, Z, T), one field element.  An addition of a cached point is two rounds of one product
+// per lane with three exchanges between them (32 word shuffles, two additions a lane), a
+// doubling a squaring and a product.  Where every lane held the whole point and repeated the
+// additions, an addition took three rounds, 64 shuffles and nine additions a lane (about 760
+// instructions against 450) and four times the registers.  Every lane of the warp must take
+// part (full-mask shuffles); each quad works on its own point.
+__device__ __forceinline__ int quad_lane() { return threadIdx.x & 3; }
+
+// The element held by lane `src` of the own quad.
+__device__ __forceinline__ fe fe_quad(const fe& a, int src) {
+  const int lane = (threadIdx.x & 28) | src;
+  fe r;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) r.v[i] = __shfl_sync(0xffffffffu, a.v[i], lane);
+  return r;
 }
 
-__device__ __forceinline__ ge ge_add_quad(const ge& p, const ge& qq) {
-  const int lane = threadIdx.x & 31, q = lane & 3, base = lane & ~3;
-  // phase 1: A = (Y1-X1)(Y2-X2), B = (Y1+X1)(Y2+X2), TT = T1 T2, ZZ = Z1 Z2
-  fe a = fe_select(fe_sub(p.Y, p.X), fe_add(p.Y, p.X), q == 1);
-  fe b = fe_select(fe_sub(qq.Y, qq.X), fe_add(qq.Y, qq.X), q == 1);
-  a = fe_select(a, p.T, q == 2); b = fe_select(b, qq.T, q == 2);
-  a = fe_select(a, p.Z, q == 3); b = fe_select(b, qq.Z, q == 3);
-  fe r = fe_mul(a, b);
-  // lane 2 turns T1 T2 into C = 2d T1 T2
-  r = fe_select(r, fe_mul(r, fe_d2()), q == 2);
-  const fe A = fe_shfl(r, base), B = fe_shfl(r, base + 1), C = fe_shfl(r, base + 2), ZZ = fe_shfl(r, base + 3);
-  const fe D = fe_add(ZZ, ZZ);
-  const fe E = fe_sub(B, A), F = fe_sub(D, C), G = fe_add(D, C), H = fe_add(B, A);
-  fe m1 = fe_select(E, G, q == 1), m2 = fe_select(F, H, q == 1);
-  m1 = fe_select(m1, F, q == 2); m2 = fe_select(m2, G, q == 2);
-  m2 = fe_select(m2, H, q == 3);
-  const fe s = fe_mul(m1, m2);
-  ge o;
-  o.X = fe_shfl(s, base); o.Y = fe_shfl(s, base + 1); o.Z = fe_shfl(s, base + 2); o.T = fe_shfl(s, base + 3);
-  return o;
+__device__ __forceinline__ fe fe_shfl_xor(const fe& a, int mask) {
+  fe r;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) r.v[i] = __shfl_xor_sync(0xffffffffu, a.v[i], mask);
+  return r;
+}
+
+__device__ __forceinline__ fe fe_small(uint32_t k) { fe r = fe_zero(); r.v[0] = k; return r; }
+
+__device__ __forceinline__ fe qp_identity() {
+  const int q = quad_lane();
+  return fe_small(q == 1 || q == 2 ? 1u : 0u);
+}
+
+// Coordinate q of a point of 32 words (16-byte aligned), and back.
+__device__ __forceinline__ fe qp_load(const uint32_t* p) {
+  const uint4* s = reinterpret_cast<const uint4*>(p + 8 * quad_lane());
+  const uint4 a = s[0], b = s[1];
+  return fe_const(a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w);
+}
+
+__device__ __forceinline__ void qp_store(uint32_t* p, const fe& v) {
+  uint4* d = reinterpret_cast<uint4*>(p + 8 * quad_lane());
+  d[0] = make_uint4(v.v[0], v.v[1], v.v[2], v.v[3]);
+  d[1] = make_uint4(v.v[4], v.v[5], v.v[6], v.v[7]);
+}
+
+// The own coordinate of a point that every lane of the quad holds whole.
+__device__ __forceinline__ fe qp_spread(const ge& p) {
+  const int q = quad_lane();
+  fe r = fe_select(p.X, p.Y, q == 1);
+  r = fe_select(r, p.Z, q == 2);
+  return fe_select(r, p.T, q == 3);
+}
+
+// (X, Y, Z, T) -> (Y-X, Y+X, Z, T)
+__device__ __forceinline__ fe qp_prepare(const fe& v) {
+  const int q = quad_lane();
+  const fe s = fe_addsub(fe_shfl_xor(v, 1), v, q == 0);
+  return fe_select(s, v, q >= 2);
+}
+
+// The cached form (Y-X, Y+X, 2Z, 2dT).
+__device__ __forceinline__ fe qp_cached(const fe& v) {
+  const int q = quad_lane();
+  const fe k = fe_select(fe_small(q == 2 ? 2u : 1u), fe_d2(), q == 3);
+  return fe_mul(qp_prepare(v), k);
+}
+
+// A point from its cached form: (2X, 2Y, 2Z, 2T).
+__device__ __forceinline__ fe qp_from_cached(const fe& c) {
+  const int q = quad_lane();
+  const fe s = fe_select(fe_addsub(fe_shfl_xor(c, 1), c, q == 0), c, q >= 2);
+  return fe_mul(s, fe_select(fe_one(), fe_dinv(), q == 3));
+}
+
+// Negation: of a point (X, T), and of a cached form (the first two exchanged, the last negated).
+__device__ __forceinline__ fe qp_neg(const fe& v) {
+  const int q = quad_lane();
+  return fe_select(v, fe_neg(v), q == 0 || q == 3);
+}
+
+__device__ __forceinline__ fe qp_neg_cached(const fe& c) {
+  const int q = quad_lane();
+  const fe o = fe_shfl_xor(c, 1);
+  return fe_select(fe_select(c, o, q < 2), fe_neg(c), q == 3);
+}
+
+// a + b, b in cached form.  Lanes: A B D C, then E H G F, then E F, G H, F G, E H.
+__device__ __forceinline__ fe qp_add_cached(const fe& a, const fe& c) {
+  const int q = quad_lane();
+  const fe m = fe_mul(qp_prepare(a), c);
+  const fe v = fe_addsub(fe_shfl_xor(m, 1), m, q == 0 || q == 3);
+  const fe u = fe_quad(v, q == 3 ? 1 : q), w = fe_quad(v, q == 3 ? 0 : q == 1 ? 2 : 3);
+  return fe_mul(u, w);
+}
+
+__device__ __forceinline__ fe qp_add(const fe& a, const fe& b) { return qp_add_cached(a, qp_cached(b)); }
+
+// 2a.  Lanes: A = X^2, B = Y^2, ZZ, S = (X+Y)^2, then G = B-A, -H = A+B, -F = 2ZZ-G, E = S-(A+B); the
+// products of these are the doubled point with all four coordinates negated.
+__device__ __forceinline__ fe qp_dbl(const fe& a) {
+  const int q = quad_lane();
+  const fe in = fe_select(a, fe_add(fe_quad(a, 0), fe_quad(a, 1)), q == 3);
+  const fe s = fe_sq(in);
+  const fe t = fe_addsub(fe_shfl_xor(s, 1), s, q == 0);            // lanes 0, 1: G, A+B
+  const fe b = fe_select(s, fe_add(s, s), q == 2);
+  const fe v = fe_select(fe_sub(b, fe_quad(t, q == 2 ? 0 : 1)), t, q < 2);
+  const fe u = fe_quad(v, q == 0 ? 3 : q), w = fe_quad(v, q == 0 ? 2 : q == 3 ? 1 : 0);
+  return fe_mul(u, w);
+}
+
+// X = 0 and Y = Z; the same answer in every lane of the quad.
+__device__ __forceinline__ bool qp_is_identity(const fe& a) {
+  const int q = quad_lane();
+  const bool z = fe_is_zero(fe_select(a, fe_sub(a, fe_quad(a, 2)), q == 1));
+  const uint32_t votes = __ballot_sync(0xffffffffu, z || q >= 2) >> (threadIdx.x & 28);
+  return (votes & 15u) == 15u;
+}
+
+// [8]a = O.
+__device__ __forceinline__ bool qp_is_torsion(fe a) {
+#pragma unroll 1
+  for (int i = 0; i < 3; ++i) a = qp_dbl(a);
+  return qp_is_identity(a);
 }
 
 // Signed 4-bit recoding of a scalar below 2^253: 64 digits in [-8, 8), sum d_i 16^i = k.

@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(T) k_point_group_sums(const uint32_t* pts, con
     pts_load(pts + (size_t)kPtsWords * t, x, y, t2d);
     acc = ge_madd(acc, x, y, t2d);
   }
-  __shared__ uint32_t sp[T][32];
+  __shared__ __align__(16) uint32_t sp[T][32];
   ge_store(sp[threadIdx.x], acc);
   compact::quad_tree(sp, G < T ? (int)G : T);
   if (threadIdx.x < 32) partial[kPointPartialWords * g + threadIdx.x] = sp[0][threadIdx.x];

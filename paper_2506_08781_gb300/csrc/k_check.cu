@@ -51,7 +51,7 @@ void launch_entry_check(cudaStream_t st, const DirectCheckArgs& a) {
 __global__ void __launch_bounds__(kDirectFinishThreads) k_direct_finish(const DirectFinishArgs a) {
   __shared__ uint32_t wsum[kDirectFinishThreads / 32];
   __shared__ unsigned long long red[kDirectFinishThreads / 32][13];
-  __shared__ uint32_t sp[kDirectFinishThreads][32];
+  __shared__ __align__(16) uint32_t sp[kDirectFinishThreads][32];
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // thread tid owns the flags of a contiguous run
   const uint64_t per = (a.n + kDirectFinishThreads - 1) / kDirectFinishThreads;
@@ -120,10 +120,13 @@ __global__ void __launch_bounds__(kDirectFinishThreads) k_direct_finish(const Di
   ge_store(sp[tid], sum);
   compact::quad_tree(sp, nf < kDirectFinishThreads ? (int)nf : kDirectFinishThreads);
   if (tid < 32) {
-    const ge v = ge_add_quad(ge_load(a.unit), ge_neg(ge_load(sp[0])));
+    const fe v = qp_add(qp_load(a.unit), qp_neg(qp_load(sp[0])));
+    __syncwarp();
+    if (tid < 4) qp_store(sp[0], v);
+    __syncwarp();
     if (tid == 0) {
       uint32_t w[8];
-      compact::encode(v, w);
+      compact::encode(ge_load(sp[0]), w);
       for (int k = 0; k < 8; ++k) reinterpret_cast<uint32_t*>(a.out + 32)[k] = w[k];
     }
   }
@@ -181,7 +184,7 @@ __global__ void k_reduce_scalars(const unsigned long long* partial, uint32_t npa
 
 __global__ void k_sum_encode(const uint32_t* partial, uint32_t nparts, uint32_t* point_out, uint8_t* enc_out,
                              uint32_t* bad_out) {
-  __shared__ uint32_t sp[kFinalThreads][32];
+  __shared__ __align__(16) uint32_t sp[kFinalThreads][32];
   __shared__ uint32_t sbad;
   const uint32_t tid = threadIdx.x;
   if (tid == 0) sbad = 0;

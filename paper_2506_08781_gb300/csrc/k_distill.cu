@@ -96,25 +96,22 @@ __device__ __forceinline__ void bisect_pass(const TreeArgs& a, const uint64_t* f
     bool live = w < total;
     const uint64_t wc = live ? w : total - 1;
     const uint64_t k = (fail_in[wc >> j] << j) | (wc & mask);
-    ge P;
+    fe minus_P;
     const uint8_t *e, *s;
     if (tl > 0) {
       const uint64_t node = a.M - (a.M >> (tl - 1)) + k;   // levels 1 .. tl-1 hold M/2 + ... + M/2^(tl-1) nodes
-      P = ge_load4(a.tree_pts + 32 * node);
+      minus_P = qp_minus_extended(a.tree_pts + 32 * node);
       e = a.tree_e + 32 * node;
       s = a.tree_s + 32 * node;
     } else {
       // malformed entries are flagged already; padding leaves hold nothing
       live = live && k < a.n && !flagged(a.skip1, a.skip2, k);
       const uint64_t t = k < a.n ? k : a.n - 1;
-      fe t2d;
-      pts_load(a.pts + (size_t)kPtsWords * t, P.X, P.Y, t2d);
-      P.Z = fe_one();
-      P.T = fe_mul(P.X, P.Y);
+      minus_P = qp_minus_affine(a.pts + (size_t)kPtsWords * t);
       e = a.e + 32 * t;
       s = a.s + 32 * t;
     }
-    const bool ok = check_lanes<LANES>(e, s, P, tY, tG);
+    const bool ok = check_lanes<LANES>(e, s, minus_P, tY, tG);
     if (live && !ok && (threadIdx.x & (LANES - 1)) == 0) {
       if (tl > 0) fail_out[atomicAdd(cnt_out, 1ull)] = k;
       else invalid[k] = 1;
@@ -172,7 +169,7 @@ __global__ void __launch_bounds__(128) k_flagged_windows(const uint32_t* pts, co
                                                          uint32_t* partial) {
   const int w = blockIdx.y;
   const uint32_t quad = threadIdx.x >> 2, nq = blockDim.x >> 2;
-  ge sum = ge_identity();
+  fe sum = qp_identity();
   // block-uniform trip count (quad operations need every lane)
   for (uint64_t i0 = (uint64_t)blockIdx.x * nq; i0 < cnt; i0 += (uint64_t)gridDim.x * nq) {
     const uint64_t i = i0 + quad;
@@ -180,23 +177,19 @@ __global__ void __launch_bounds__(128) k_flagged_windows(const uint32_t* pts, co
     bool neg;
     uint32_t d = weight_digit(z, t, w, pl.c, neg);
     if (i >= cnt || (badR && badR[t])) d = 0;
-    ge P;
-    fe t2d;
-    pts_load(pts + (size_t)kPtsWords * t, P.X, P.Y, t2d);
-    P.Z = fe_one();
-    P.T = fe_mul(P.X, P.Y);
-    if (neg) P = ge_neg(P);
-    ge acc = ge_identity();
+    // +-R_t in cached form
+    fe P = qp_minus_affine(pts + (size_t)kPtsWords * t);
+    P = fe_select(qp_neg_cached(P), P, neg);
+    fe acc = qp_identity();
 #pragma unroll 1
     for (int bit = pl.c - 1; bit >= 0; --bit) {
-      acc = ge_dbl_quad(acc);
-      const ge more = ge_add_quad(acc, P);
-      acc = ge_select(acc, more, ((d >> bit) & 1u) != 0);
+      acc = qp_dbl(acc);
+      acc = fe_select(acc, qp_add_cached(acc, P), ((d >> bit) & 1u) != 0);
     }
-    sum = ge_add_quad(sum, acc);
+    sum = qp_add(sum, acc);
   }
-  __shared__ uint32_t sp[32][32];
-  if ((threadIdx.x & 3) == 0) ge_store(sp[quad], sum);
+  __shared__ __align__(16) uint32_t sp[32][32];
+  qp_store(sp[quad], sum);
   compact::quad_tree(sp, 32);
   const size_t o = ((size_t)w * gridDim.x + blockIdx.x) * kPointPartialWords;
   if (threadIdx.x < 32) partial[o + threadIdx.x] = sp[0][threadIdx.x];
@@ -215,8 +208,8 @@ __global__ void __launch_bounds__(32) k_confirm_windows(const uint32_t* W, const
 #pragma unroll 1
   for (int r0 = 0; r0 < windows; r0 += 8) {
     const int w = r0 + quad, wc = w < windows ? w : windows - 1;
-    const ge d = ge_add_quad(ge_load(W + 32 * (size_t)wc), ge_neg(ge_load(F + 32 * (size_t)wc)));
-    const bool eq = compact::quad_equal(d, ge_load(Pw + 32 * (size_t)wc));
+    const fe d = qp_add(qp_load(W + 32 * (size_t)wc), qp_neg(qp_load(F + 32 * (size_t)wc)));
+    const bool eq = qp_is_torsion(qp_add(d, qp_neg(qp_load(Pw + 32 * (size_t)wc))));
     if (w < windows) ok = ok && eq;
   }
   const bool all = __all_sync(0xffffffffu, ok);
@@ -245,7 +238,7 @@ __global__ void k_gather_flagged(const uint32_t* pts, const uint32_t* z, const u
 // to the batch.
 __global__ void __launch_bounds__(256) k_ccd_points(const uint32_t* pts, const uint8_t* badR, const uint64_t* idx,
                                                     const uint64_t* nf_dev, const uint32_t* unit, uint8_t* enc_out) {
-  __shared__ uint32_t sp[256][32];
+  __shared__ __align__(16) uint32_t sp[256][32];
   ge acc = ge_identity();
   const uint64_t nf = *nf_dev;
   for (uint64_t i = threadIdx.x; i < nf; i += blockDim.x) {
@@ -259,10 +252,13 @@ __global__ void __launch_bounds__(256) k_ccd_points(const uint32_t* pts, const u
   // once per call: compact (out-of-line) point operations, the code being fetched cold
   compact::quad_tree(sp, nf < 1 ? 1 : nf < 256 ? (int)nf : 256);
   if (threadIdx.x < 32) {
-    const ge v = ge_add_quad(ge_load(unit), ge_neg(ge_load(sp[0])));
+    const fe v = qp_add(qp_load(unit), qp_neg(qp_load(sp[0])));
+    __syncwarp();
+    if (threadIdx.x < 4) qp_store(sp[0], v);
+    __syncwarp();
     if (threadIdx.x == 0) {
       uint32_t w[8];
-      compact::encode(v, w);
+      compact::encode(ge_load(sp[0]), w);
       for (int k = 0; k < 8; ++k) {
         enc_out[4 * k] = (uint8_t)w[k]; enc_out[4 * k + 1] = (uint8_t)(w[k] >> 8);
         enc_out[4 * k + 2] = (uint8_t)(w[k] >> 16); enc_out[4 * k + 3] = (uint8_t)(w[k] >> 24);

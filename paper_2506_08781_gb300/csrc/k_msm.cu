@@ -237,15 +237,16 @@ __global__ void __launch_bounds__(128) k_msm_chunk(const uint32_t* buckets, MsmP
   const uint64_t g = quad < total ? quad : total - 1;   // surplus quads repeat the last chunk
   const uint32_t w = (uint32_t)(g / pl.nchunks), j = (uint32_t)(g % pl.nchunks);
   const uint32_t* B = buckets + 32 * ((size_t)w * pl.nb + (size_t)j * kMsmChunk);
-  ge run = ge_identity(), acc = ge_identity();
+  fe run = qp_identity(), acc = qp_identity();
+#pragma unroll 1
   for (int r = kMsmChunk - 1; r >= 1; --r) {
-    run = ge_add_quad(run, ge_load(B + 32 * r));
-    acc = ge_add_quad(acc, run);
+    run = qp_add(run, qp_load(B + 32 * r));
+    acc = qp_add(acc, run);
   }
-  run = ge_add_quad(run, ge_load(B));
-  if ((threadIdx.x & 3) == 0 && quad < total) {
-    ge_store(L + 32 * g, acc);
-    ge_store(T + 32 * g, run);
+  run = qp_add(run, qp_load(B));
+  if (quad < total) {
+    qp_store(L + 32 * g, acc);
+    qp_store(T + 32 * g, run);
   }
 }
 
@@ -257,25 +258,24 @@ __global__ void __launch_bounds__(128) k_msm_chunk(const uint32_t* buckets, MsmP
 // kernels read as G_0 + 16 sum_k 2^k G_{1+k} = W_w.  It replaces the running sums over chunks
 // and the group sums, whose chains of dependent additions set the latency at these sizes.
 __global__ void __launch_bounds__(512) k_msm_direct_groups(const uint32_t* buckets, MsmPlan pl, uint32_t* groups) {
-  extern __shared__ uint32_t sp[];   // one point (32 words) per quad
+  extern __shared__ __align__(16) uint32_t sp[];   // one point (32 words) per quad
   const int w = blockIdx.x;
   const int quad = threadIdx.x >> 2, nq = blockDim.x >> 2;   // nq = 2^(c-1)
   const uint32_t d = (uint32_t)quad + 1;
-  const ge B = ge_load(buckets + 32 * ((size_t)w * pl.nb + d));
-  ge acc = ge_identity();
+  const fe B = qp_cached(qp_load(buckets + 32 * ((size_t)w * pl.nb + d)));
+  fe acc = qp_identity();
 #pragma unroll 1
   for (int bit = pl.c - 1; bit >= 0; --bit) {
-    acc = ge_dbl_quad(acc);
-    const ge sum = ge_add_quad(acc, B);
-    acc = ge_select(acc, sum, ((d >> bit) & 1u) != 0);
+    acc = qp_dbl(acc);
+    acc = fe_select(acc, qp_add_cached(acc, B), ((d >> bit) & 1u) != 0);
   }
-  if ((threadIdx.x & 3) == 0) ge_store(sp + 32 * quad, acc);
+  qp_store(sp + 32 * quad, acc);
   __syncthreads();
 #pragma unroll 1
   for (int h = nq / 2; h > 0; h >>= 1) {
-    const ge sum = ge_add_quad(ge_load(sp + 32 * quad), ge_load(sp + 32 * ((quad + h) % nq)));
+    const fe sum = qp_add(qp_load(sp + 32 * quad), qp_load(sp + 32 * ((quad + h) % nq)));
     __syncthreads();
-    if ((threadIdx.x & 3) == 0 && quad < h) ge_store(sp + 32 * quad, sum);
+    if (quad < h) qp_store(sp + 32 * quad, sum);
     __syncthreads();
   }
   const int ng = 1 + pl.jbits;
@@ -302,21 +302,21 @@ __global__ void __launch_bounds__(512) k_msm_groups(const uint32_t* L, const uin
   const int w = blockIdx.x / ng, grp = blockIdx.x % ng;
   const uint32_t* base = (grp == 0 ? L : T) + 32 * (size_t)w * pl.nchunks;
   const int quad = threadIdx.x >> 2, nq = kGroupThreads / 4;
-  ge acc = ge_identity();
+  fe acc = qp_identity();
+#pragma unroll 1
   for (uint32_t j0 = 0; j0 < pl.nchunks; j0 += nq) {
     const uint32_t j = j0 + quad;
     const bool take = j < pl.nchunks && (grp == 0 || ((j >> (grp - 1)) & 1u));
-    const ge p = take ? ge_load(base + 32 * (size_t)j) : ge_identity();
-    acc = ge_add_quad(acc, p);
+    acc = qp_add(acc, take ? qp_load(base + 32 * (size_t)j) : qp_identity());
   }
-  __shared__ uint32_t sp[kGroupThreads / 4][32];
-  if ((threadIdx.x & 3) == 0) ge_store(sp[quad], acc);
+  __shared__ __align__(16) uint32_t sp[kGroupThreads / 4][32];
+  qp_store(sp[quad], acc);
   __syncthreads();
+#pragma unroll 1
   for (int h = nq / 2; h > 0; h >>= 1) {
-    const ge other = ge_load(sp[(quad + h) % nq]);
-    const ge sum = ge_add_quad(ge_load(sp[quad]), other);
+    const fe sum = qp_add(qp_load(sp[quad]), qp_load(sp[(quad + h) % nq]));
     __syncthreads();
-    if ((threadIdx.x & 3) == 0 && quad < h) ge_store(sp[quad], sum);
+    if (quad < h) qp_store(sp[quad], sum);
     __syncthreads();
   }
   if (threadIdx.x < 32) groups[32 * (size_t)blockIdx.x + threadIdx.x] = sp[0][threadIdx.x];
@@ -325,38 +325,35 @@ __global__ void __launch_bounds__(512) k_msm_groups(const uint32_t* L, const uin
 // Window sums W_w = G_0 + 16 sum_k 2^k G_{1+k} (quad w computes window w), then
 // sum_w 2^{c w} W_w by Horner's rule in quad 0.  One warp; windows are processed in rounds
 // of eight quads.
-__global__ void __launch_bounds__(32) k_msm_final(const uint32_t* groups, MsmPlan pl, uint32_t* out) {
-  __shared__ uint32_t wsum[kMsmMaxWindows][32];
-  const int lane = threadIdx.x & 31, quad = lane >> 2;
-  const int ng = 1 + pl.jbits;
-  for (int r0 = 0; r0 < pl.windows; r0 += 8) {
-    const int w = r0 + quad;
-    const int wc = w < pl.windows ? w : pl.windows - 1;
-    const uint32_t* G = groups + 32 * (size_t)wc * ng;
-    ge acc = ge_load(G + 32 * pl.jbits);       // top bit group
-    for (int k = pl.jbits - 2; k >= 0; --k) acc = ge_add_quad(ge_dbl_quad(acc), ge_load(G + 32 * (1 + k)));
-    for (int s = 0; s < 4; ++s) acc = ge_dbl_quad(acc);   // times kMsmChunk = 16
-    acc = ge_add_quad(acc, ge_load(G));
-    if ((lane & 3) == 0 && w < pl.windows) ge_store(wsum[w], acc);
-    __syncwarp();
-  }
-  ge acc = ge_load(wsum[pl.windows - 1]);
-  for (int w = pl.windows - 2; w >= 0; --w) {
-    for (int s = 0; s < pl.c; ++s) acc = ge_dbl_quad(acc);
-    acc = ge_add_quad(acc, ge_load(wsum[w]));
-  }
-  if (lane == 0) ge_store(out, acc);
-}
-
-// Window sum W_w = G_0 + 16 sum_k 2^k G_{1+k} of window w from its group sums (quad-cooperative
-// Horner over the group bits; every lane of the quad ends with the whole point).
-__device__ __forceinline__ ge window_sum_quad(const uint32_t* groups, const MsmPlan& pl, int w) {
+__device__ __forceinline__ fe window_sum_quad(const uint32_t* groups, const MsmPlan& pl, int w) {
   const int ng = 1 + pl.jbits;
   const uint32_t* G = groups + 32 * (size_t)w * ng;
-  ge acc = ge_load(G + 32 * pl.jbits);
-  for (int k = pl.jbits - 2; k >= 0; --k) acc = ge_add_quad(ge_dbl_quad(acc), ge_load(G + 32 * (1 + k)));
-  for (int i = 0; i < 4; ++i) acc = ge_dbl_quad(acc);   // times kMsmChunk = 16
-  return ge_add_quad(acc, ge_load(G));
+  fe acc = qp_load(G + 32 * pl.jbits);   // top bit group
+#pragma unroll 1
+  for (int k = pl.jbits - 2; k >= 0; --k) acc = qp_add(qp_dbl(acc), qp_load(G + 32 * (1 + k)));
+#pragma unroll 1
+  for (int i = 0; i < 4; ++i) acc = qp_dbl(acc);   // times kMsmChunk = 16
+  return qp_add(acc, qp_load(G));
+}
+
+__global__ void __launch_bounds__(32) k_msm_final(const uint32_t* groups, MsmPlan pl, uint32_t* out) {
+  __shared__ __align__(16) uint32_t wsum[kMsmMaxWindows][32];
+  const int lane = threadIdx.x & 31, quad = lane >> 2;
+#pragma unroll 1
+  for (int r0 = 0; r0 < pl.windows; r0 += 8) {
+    const int w = r0 + quad;
+    const fe acc = window_sum_quad(groups, pl, w < pl.windows ? w : pl.windows - 1);
+    if (w < pl.windows) qp_store(wsum[w], acc);
+    __syncwarp();
+  }
+  fe acc = qp_load(wsum[pl.windows - 1]);
+#pragma unroll 1
+  for (int w = pl.windows - 2; w >= 0; --w) {
+#pragma unroll 1
+    for (int s = 0; s < pl.c; ++s) acc = qp_dbl(acc);
+    acc = qp_add(acc, qp_load(wsum[w]));
+  }
+  if (quad == 0) qp_store(out, acc);
 }
 
 // The window sums W_w of every window into W (32 words each): quad w per window, in rounds
@@ -365,15 +362,16 @@ __global__ void __launch_bounds__(32) k_msm_windows(const uint32_t* groups, MsmP
   const int lane = threadIdx.x & 31, quad = lane >> 2;
   for (int r0 = 0; r0 < pl.windows; r0 += 8) {
     const int w = r0 + quad;
-    const ge acc = window_sum_quad(groups, pl, w < pl.windows ? w : pl.windows - 1);
-    if ((lane & 3) == 0 && w < pl.windows) ge_store(W + 32 * (size_t)w, acc);
+    const fe acc = window_sum_quad(groups, pl, w < pl.windows ? w : pl.windows - 1);
+    if (w < pl.windows) qp_store(W + 32 * (size_t)w, acc);
   }
 }
 
 // Per-window weighted check, group side: quad w forms the window sum W_w and tests
 // [8](W_w - P_w) = O against P_w = [E_w] Y + [S_w] G (k_window_prep); windows are processed in
-// rounds of eight quads.  The window sums go to W (a confirmation needs them).  accept = every window holds, no malformed s (*bad), no undecodable
-// R (*point_bad) and a decodable key.  One warp.
+// rounds of eight quads.  The window sums go to W (a confirmation needs them).  accept = every
+// window holds, no malformed s (*bad), no undecodable R (*point_bad) and a decodable key.  One
+// warp.
 __global__ void __launch_bounds__(32) k_msm_window_check(const uint32_t* groups, MsmPlan pl, const uint32_t* Pw,
                                                          const uint32_t* bad, const uint32_t* point_bad,
                                                          const uint32_t* status, uint32_t* W, uint8_t* accept) {
@@ -382,11 +380,10 @@ __global__ void __launch_bounds__(32) k_msm_window_check(const uint32_t* groups,
   for (int r0 = 0; r0 < pl.windows; r0 += 8) {
     const int w = r0 + quad;
     const int wc = w < pl.windows ? w : pl.windows - 1;
-    const ge acc = window_sum_quad(groups, pl, wc);
-    if ((lane & 3) == 0 && w < pl.windows) ge_store(W + 32 * (size_t)w, acc);
-    ge diff = ge_add_quad(acc, ge_neg(ge_load(Pw + 32 * (size_t)wc)));
-    for (int i = 0; i < 3; ++i) diff = ge_dbl_quad(diff);   // cofactor 8
-    if (w < pl.windows) ok = ok && ge_is_identity(diff);
+    const fe acc = window_sum_quad(groups, pl, wc);
+    if (w < pl.windows) qp_store(W + 32 * (size_t)w, acc);
+    const bool eq = qp_is_torsion(qp_add(acc, qp_neg(qp_load(Pw + 32 * (size_t)wc))));
+    if (w < pl.windows) ok = ok && eq;
   }
   const bool all = __all_sync(0xffffffffu, ok);
   if (lane == 0) *accept = (all && *bad == 0 && !(point_bad && *point_bad) && (*status & kErrKey) == 0) ? 1 : 0;

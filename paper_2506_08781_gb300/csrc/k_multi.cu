@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) k_segment_sums(const
   const uint64_t lo = dlo + (uint64_t)piece * kSegPiece, hi = min(lo + kSegPiece, dhi);
   const bool whole = seg_pieces(dhi - dlo) == 1;   // block-uniform
   if (kPart == kSegPoints) {
-    __shared__ uint32_t sp_[kThreads][32];
+    __shared__ __align__(16) uint32_t sp_[kThreads][32];
     ge acc = ge_identity();
     for (uint64_t t = lo + threadIdx.x; t < hi; t += blockDim.x) {
       if (badR[t] || badS[t]) continue;
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(kSegThreads) k_segment_combine(const uint64_t*
   }
   ge acc = ge_identity();
   for (uint64_t j = threadIdx.x; j < np; j += blockDim.x) acc = ge_add(acc, ge_load(piece_R + 32 * (p0 + j)));
-  __shared__ uint32_t sp_[kSegThreads][32];
+  __shared__ __align__(16) uint32_t sp_[kSegThreads][32];
   ge_store(sp_[threadIdx.x], acc);
   compact::quad_tree(sp_, np < kSegThreads ? (int)np : kSegThreads);
   seg_write<kSegScalars | kSegPoints>(tot, sp_[0], d, out);
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(kFinalThreads) k_multi_window_check(const uint
   const int w = blockIdx.x;
   __shared__ unsigned long long red[kFinalThreads / 32][13];
   __shared__ int8_t dig[64];
-  __shared__ uint32_t pts_[kFinalThreads][32];
+  __shared__ __align__(16) uint32_t pts_[kFinalThreads][32];
   acc13 a;
   acc_zero(a);
   for (uint32_t d = threadIdx.x; d < n_dev; d += blockDim.x)
@@ -296,9 +296,10 @@ __global__ void __launch_bounds__(kFinalThreads) k_multi_window_check(const uint
   ge_store(pts_[threadIdx.x], term);
   compact::quad_tree(pts_, kTableWindows);
   if (threadIdx.x < 32) {
-    ge p1 = ge_load(W + 32 * (size_t)w);
-    if (Wsub) p1 = ge_add_quad(p1, ge_neg(ge_load(Wsub + 32 * (size_t)w)));
-    const bool ok = compact::quad_equal(ge_add_quad(p1, ge_neg(ge_load(P2w + 32 * (size_t)w))), ge_load(pts_[0]));
+    fe p1 = qp_load(W + 32 * (size_t)w);
+    if (Wsub) p1 = qp_add(p1, qp_neg(qp_load(Wsub + 32 * (size_t)w)));
+    p1 = qp_add(p1, qp_neg(qp_load(P2w + 32 * (size_t)w)));
+    const bool ok = qp_is_torsion(qp_add(p1, qp_neg(qp_load(pts_[0]))));
     if (threadIdx.x == 0 && !ok) accept[0] = 0;
   }
 }
@@ -321,9 +322,9 @@ __global__ void __launch_bounds__(kPointThreads) k_table_msm_windows(const uint3
     const uint32_t* kd = k + 8 * ((size_t)win * n + d);
     int carry = 0, digit = 0;
     for (int i = 0; i <= w; ++i) digit = sc_digit4(kd, i, carry);
-    if (digit) acc = ge_add(acc, table_pick(tabs[d], w, digit));
+    acc = table_add(acc, tabs[d], w, digit);
   }
-  __shared__ uint32_t sp[kPointThreads][32];
+  __shared__ __align__(16) uint32_t sp[kPointThreads][32];
   ge_store(sp[threadIdx.x], acc);
   compact::quad_tree(sp, kPointThreads);
   const size_t o = ((size_t)win * gridDim.x + blockIdx.x) * kPointPartialWords;
@@ -338,7 +339,7 @@ __global__ void __launch_bounds__(kPointThreads) k_window_point_sums(const uint3
   ge acc = ge_identity();
   for (uint32_t b = threadIdx.x; b < nblocks; b += blockDim.x)
     acc = ge_add(acc, ge_load(partial + ((size_t)w * nblocks + b) * kPointPartialWords));
-  __shared__ uint32_t sp[kPointThreads][32];
+  __shared__ __align__(16) uint32_t sp[kPointThreads][32];
   ge_store(sp[threadIdx.x], acc);
   compact::quad_tree(sp, nblocks < kPointThreads ? (int)nblocks : kPointThreads);
   if (threadIdx.x < 32) out[32 * (size_t)w + threadIdx.x] = sp[0][threadIdx.x];
@@ -354,7 +355,7 @@ __global__ void __launch_bounds__(kFinalThreads) k_multi_check(const uint32_t* P
                                                                uint8_t* accept) {
   __shared__ unsigned long long red[kFinalThreads / 32][13];
   __shared__ int8_t dig[64];
-  __shared__ uint32_t pts_[kFinalThreads][32];
+  __shared__ __align__(16) uint32_t pts_[kFinalThreads][32];
   acc13 a;
   acc_zero(a);
   for (uint32_t d = threadIdx.x; d < n_dev; d += blockDim.x)
@@ -381,9 +382,10 @@ __global__ void __launch_bounds__(kFinalThreads) k_multi_check(const uint32_t* P
   ge_store(pts_[threadIdx.x], term);
   compact::quad_tree(pts_, kTableWindows);
   if (threadIdx.x < 32) {
-    ge p1 = ge_load(P1);
-    if (P1sub) p1 = ge_add_quad(p1, ge_neg(ge_load(P1sub)));
-    const bool ok = compact::quad_equal(ge_add_quad(p1, ge_neg(ge_load(P2))), ge_load(pts_[0]));
+    fe p1 = qp_load(P1);
+    if (P1sub) p1 = qp_add(p1, qp_neg(qp_load(P1sub)));
+    p1 = qp_add(p1, qp_neg(qp_load(P2)));
+    const bool ok = qp_is_torsion(qp_add(p1, qp_neg(qp_load(pts_[0]))));
     if (threadIdx.x == 0) accept[0] = ok ? 1 : 0;
   }
 }
@@ -397,7 +399,7 @@ __global__ void __launch_bounds__(128) k_device_unit_check(const uint32_t* const
   const uint32_t d = grp < n_dev ? grp : n_dev - 1;   // surplus groups repeat the last device
   const bool ok = check_lanes<LANES>(reinterpret_cast<const uint8_t*>(ss.Eu + 8 * (size_t)d),
                                      reinterpret_cast<const uint8_t*>(ss.Su + 8 * (size_t)d),
-                                     ge_load(ss.Ru + 32 * (size_t)d), tabs[d], tableG) && ss.bad[d] == 0;
+                                     qp_minus_extended(ss.Ru + 32 * (size_t)d), tabs[d], tableG) && ss.bad[d] == 0;
   if ((threadIdx.x & (LANES - 1)) == 0 && grp < n_dev) dev_flag[d] = ok ? 0 : 1;
 }
 
@@ -424,9 +426,9 @@ __global__ void __launch_bounds__(kPointThreads) k_table_msm(const uint32_t* con
     const uint32_t* kd = k + 8 * (size_t)d;
     int carry = 0, digit = 0;
     for (int i = 0; i <= w; ++i) digit = sc_digit4(kd, i, carry);
-    if (digit) acc = ge_add(acc, table_pick(tabs[d], w, digit));
+    acc = table_add(acc, tabs[d], w, digit);
   }
-  __shared__ uint32_t sp[kPointThreads][32];
+  __shared__ __align__(16) uint32_t sp[kPointThreads][32];
   ge_store(sp[threadIdx.x], acc);
   compact::quad_tree(sp, kPointThreads);
   if (threadIdx.x < 32) partial[(uint64_t)blockIdx.x * kPointPartialWords + threadIdx.x] = sp[0][threadIdx.x];

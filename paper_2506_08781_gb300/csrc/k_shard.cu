@@ -80,8 +80,8 @@ __global__ void __launch_bounds__(kShardThreads) k_combine_check(const uint32_t*
                                                                 const uint32_t* status, uint32_t* total,
                                                                 uint8_t* accept) {
   __shared__ int8_t dig_e[64], dig_s[64];
-  __shared__ uint32_t pts_[kShardThreads][32];
-  __shared__ uint32_t sR[32];
+  __shared__ __align__(16) uint32_t pts_[kShardThreads][32];
+  __shared__ __align__(16) uint32_t sR[32];
   __shared__ uint32_t well_formed;
   const int tid = threadIdx.x;
   // a single call's worth of arithmetic from compact (out-of-line) field and point
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kShardThreads) k_combine_check(const uint32_t*
   compact::quad_tree(pts_, 128);
   // [8](R~ - e~Y - s~G) by the first warp's quads (all of them compute it)
   if (tid < 32) {
-    const bool eq = compact::quad_equal(ge_load(sR), ge_load(pts_[0]));
+    const bool eq = compact::quad_equal(sR, pts_[0]);
     if (tid == 0) accept[0] = (eq && well_formed && (*status & kErrKey) == 0) ? 1 : 0;
   }
 }

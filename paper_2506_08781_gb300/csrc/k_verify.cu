@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(kPointThreads, MINB) k_points(const PointArgs 
 #endif
   // the block's sum by quads (a few us less at the end of a small launch than one lane per
   // addition), over as many points as the block can hold
-  __shared__ uint32_t sp[kPointThreads][32];
+  __shared__ __align__(16) uint32_t sp[kPointThreads][32];
   __shared__ uint32_t sbad;
   if (threadIdx.x == 0) sbad = 0;
   __syncthreads();
@@ -376,7 +376,8 @@ __global__ void __launch_bounds__(kPointThreads, MINB) k_points(const PointArgs 
 // launches.  k_table_chain: one quad of lanes per key walks P, 16P, ..., 16^63 P with
 // quad-cooperative doublings (252 of them, at a quarter of a doubling's dependent
 // multiplications each) and writes each 16^w P as table[w][0].  k_table_fill: one quad per
-// (key, window) forms d 16^w P for d = 2..8 by quad-cooperative additions.  The key of
+// (key, window) forms d 16^w P for d = 2..8 by quad additions.  Entries are stored in cached
+// form.  The key of
 // index k is the encoding enc + 8 k, the decoded point pts + kPtsWords * list[k] (affine
 // x, y; k itself without a list), or G (use_base).  An encoding that does not decode gives
 // the identity's table and sets bad_out[k] (when given) or the kErrKey status bit.
@@ -388,7 +389,7 @@ __global__ void __launch_bounds__(128) k_table_chain(const uint32_t* __restrict_
                                                      uint8_t* __restrict__ bad_out) {
   const uint32_t quad = ((uint32_t)blockIdx.x * blockDim.x + threadIdx.x) >> 2;
   const uint32_t k = quad < n ? quad : n - 1;   // surplus quads repeat the last key, unwritten
-  const bool writer = quad < n && (threadIdx.x & 3) == 0;
+  const bool writer = quad < n;
   ge P;
   if (use_base) {
     P = ge_base();
@@ -403,17 +404,22 @@ __global__ void __launch_bounds__(128) k_table_chain(const uint32_t* __restrict_
     for (int i = 0; i < 8; ++i) b[i] = enc[8 * (size_t)k + i];
     const bool ok = ge_decode(b, P);
     if (!ok) P = ge_identity();
-    if (writer) {
+    if (writer && quad_lane() == 0) {
       if (bad_out) bad_out[k] = ok ? 0 : 1;   // the caller reports which key failed
       else if (!ok) atomicOr(status, kErrKey);
     }
   }
   uint32_t* table = dst ? dst[k] : tables + (size_t)k * kTableWords;
-  // every lane runs every quad doubling (full-mask shuffles)
+  fe Q = qp_spread(P);
+  // every lane runs every quad operation (full-mask shuffles)
+#pragma unroll 1
   for (int w = 0; w < kTableWindows; ++w) {
-    if (writer) ge_store(table + (size_t)w * kTableDigits * 32, P);
-    if (w + 1 < kTableWindows)
-      for (int i = 0; i < 4; ++i) P = ge_dbl_quad(P);
+    const fe c = qp_cached(Q);
+    if (writer) qp_store(table + (size_t)w * kTableDigits * 32, c);
+    if (w + 1 < kTableWindows) {
+#pragma unroll 1
+      for (int i = 0; i < 4; ++i) Q = qp_dbl(Q);
+    }
   }
 }
 
@@ -421,14 +427,16 @@ __global__ void __launch_bounds__(128) k_table_fill(uint32_t n, uint32_t* __rest
   const uint64_t total = (uint64_t)n * kTableWindows;
   const uint64_t quad = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 2;
   const uint64_t q = quad < total ? quad : total - 1;
-  const bool writer = quad < total && (threadIdx.x & 3) == 0;
+  const bool writer = quad < total;
   const uint64_t key = q / kTableWindows;
   uint32_t* row = (dst ? dst[key] : tables + key * kTableWords) + (q % kTableWindows) * kTableDigits * 32;
-  const ge Pw = ge_load(row);
-  ge acc = Pw;
+  const fe Pw = qp_load(row);
+  fe acc = qp_from_cached(Pw);
+#pragma unroll 1
   for (int d = 2; d <= kTableDigits; ++d) {
-    acc = ge_add_quad(acc, Pw);
-    if (writer) ge_store(row + (d - 1) * 32, acc);
+    acc = qp_add_cached(acc, Pw);
+    const fe c = qp_cached(acc);
+    if (writer) qp_store(row + (d - 1) * 32, c);
   }
 }
 
@@ -441,7 +449,7 @@ constexpr int kPrepThreads = 128;
 __global__ void __launch_bounds__(128) k_final_prep(const PrepArgs a) {
   __shared__ unsigned long long sums[kPartialWords];
   __shared__ int8_t dig_e[64], dig_s[64];
-  __shared__ uint32_t pts_[kPrepThreads][32];
+  __shared__ __align__(16) uint32_t pts_[kPrepThreads][32];
   __shared__ uint32_t bad_flag;
   const int tid = threadIdx.x;
   if (tid < kPartialWords) sums[tid] = 0;
@@ -528,7 +536,7 @@ __global__ void __launch_bounds__(kWindowThreads) k_window_prep(const unsigned l
                                                                 uint32_t* Pw, uint32_t* bad) {
   __shared__ unsigned long long sums[2][26];
   __shared__ int8_t dig_e[64], dig_s[64];
-  __shared__ uint32_t pts_[kWindowThreads][32];
+  __shared__ __align__(16) uint32_t pts_[kWindowThreads][32];
   const int w = blockIdx.x, tid = threadIdx.x;
   if (tid < 52) sums[tid / 26][tid % 26] = 0;
   __syncthreads();
@@ -566,7 +574,7 @@ __global__ void __launch_bounds__(kWindowThreads) k_window_prep(const unsigned l
 __global__ void k_final_check(const uint32_t* prep, const uint32_t* R, const uint32_t* point_bad,
                               const uint32_t* status, uint8_t* accept) {
   if (blockIdx.x != 0) return;
-  const bool eq = compact::quad_equal(ge_load(R), ge_load(prep));
+  const bool eq = compact::quad_equal(R, prep);
   const bool ok = eq && prep[32] == 0 && !(point_bad && *point_bad) && (*status & kErrKey) == 0;
   if (threadIdx.x == 0) accept[0] = ok ? 1 : 0;
 }
