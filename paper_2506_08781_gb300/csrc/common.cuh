@@ -21,9 +21,7 @@ namespace poslo {
 
 
 constexpr int kHashThreads = 128;
-#ifndef POSLO_HASH_MIN_BLOCKS
-#define POSLO_HASH_MIN_BLOCKS 3   // resident blocks per SM the hash kernel is compiled for
-#endif
+constexpr int kHashBlocksPerSm = 4;   // resident SHA-256 hashing blocks: 128 registers, 47 KiB each
 constexpr int kPointThreads = 128;
 // Block size of the short kernels that run beside the decoding (weights, counting sort):
 // small enough that one of their blocks fits in the registers the three resident decoding
@@ -207,9 +205,15 @@ __device__ __forceinline__ void mdc2_stream(const C& c, const EntryStream& es, u
   for (uint32_t b = 0; b < nb; ++b) {
     const uint32_t o = b << 4;
     uint32_t m[4];
-    if (o + 16 <= es.L) {
+    if (o + 16 <= es.L) {   // five loads, each word the next one's neighbour
+      const uint32_t* p = es.base + (o >> 2);
+      uint32_t v = __ldg(p);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) m[q] = load_msg_word(es, (o >> 2) + q);
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t nx = __ldg(p + (q < 3 ? q + 1 : 3 + (int)es.sh_nz));
+        m[q] = __byte_perm(v, nx, es.sel);
+        v = nx;
+      }
     } else {
 #pragma unroll
       for (int q = 0; q < 4; ++q) m[q] = stream_word(es, o + 4 * q);
