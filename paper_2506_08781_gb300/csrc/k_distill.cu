@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(128) k_tree_leaves(const TreeArgs a) {
   sc e0, e1, s0, s1;
   leaf(a, 2 * k, P0, e0, s0);
   leaf(a, 2 * k + 1, P1, e1, s1);
-  ge_store(a.tree_pts + 32 * k, ge_add(P0, P1));
+  ge_store16(a.tree_pts + 32 * k, ge_add(P0, P1));
   sc_store(a.tree_e + 32 * k, sc_add(e0, e1));
   sc_store(a.tree_s + 32 * k, sc_add(s0, s1));
 }
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(128) k_tree_level(const TreeArgs a, uint64_t i
   const uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= count) return;
   const uint64_t c0 = in_off + 2 * k, c1 = c0 + 1, o = out_off + k;
-  ge_store(a.tree_pts + 32 * o, ge_add(ge_load(a.tree_pts + 32 * c0), ge_load(a.tree_pts + 32 * c1)));
+  ge_store16(a.tree_pts + 32 * o, ge_add(ge_load16(a.tree_pts + 32 * c0), ge_load16(a.tree_pts + 32 * c1)));
   sc_store(a.tree_e + 32 * o, sc_add(sc_load(a.tree_e + 32 * c0), sc_load(a.tree_e + 32 * c1)));
   sc_store(a.tree_s + 32 * o, sc_add(sc_load(a.tree_s + 32 * c0), sc_load(a.tree_s + 32 * c1)));
 }

@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(128, POSLO_ACCUM_MINB) k_msm_accum(const uint3
     const uint32_t d = code & kBktMask;
     if (d != cur) {
       uint32_t* dst = first ? A + 32 * g : buckets + 32 * ((size_t)w * pl.nb + cur + 1);
-      ge_store(dst, acc);
+      ge_store16(dst, acc);
       first = false;
       acc = ge_identity();
       cur = d;
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(128, POSLO_ACCUM_MINB) k_msm_accum(const uint3
     code = ncode;
     skip_c = nskip;
   }
-  ge_store(first ? A + 32 * g : B + 32 * g, acc);
+  ge_store16(first ? A + 32 * g : B + 32 * g, acc);
 }
 
 // Buckets that were not written whole by k_msm_accum: the run in the range holding the
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(128) k_msm_combine(const uint32_t* off, const 
   const uint32_t w = (uint32_t)(b / pl.nb), d = (uint32_t)(b % pl.nb);
   const uint32_t len = d ? cnt[b] : 0u;
   if (len == 0) {
-    ge_store(buckets + 32 * b, ge_identity());
+    ge_store16(buckets + 32 * b, ge_identity());
     return;
   }
   const CombineSpan c = combine_span(off, cnt, pl, b);
@@ -185,9 +185,9 @@ __global__ void __launch_bounds__(128) k_msm_combine(const uint32_t* off, const 
     return;
   }
   const uint64_t g0 = (uint64_t)w * ((n + (1ull << pl.seg_log2) - 1) >> pl.seg_log2);
-  ge acc = ge_load((c.starts_range ? A : B) + 32 * (g0 + c.ts));
-  for (uint64_t t = c.ts + 1; t <= c.te; ++t) acc = ge_add(acc, ge_load(A + 32 * (g0 + t)));
-  ge_store(buckets + 32 * b, acc);
+  ge acc = ge_load16((c.starts_range ? A : B) + 32 * (g0 + c.ts));
+  for (uint64_t t = c.ts + 1; t <= c.te; ++t) acc = ge_add(acc, ge_load16(A + 32 * (g0 + t)));
+  ge_store16(buckets + 32 * b, acc);
 }
 
 __device__ __forceinline__ ge ge_shfl_down(const ge& p, int delta) {
@@ -221,10 +221,10 @@ __global__ void __launch_bounds__(kCombineBigThreads) k_msm_combine_big(const ui
     const uint32_t w = (uint32_t)(b / pl.nb);
     const CombineSpan c = combine_span(off, cnt, pl, b);
     const uint64_t g0 = (uint64_t)w * nseg;
-    ge acc = lane == 0 ? ge_load((c.starts_range ? A : B) + 32 * (g0 + c.ts)) : ge_identity();
-    for (uint64_t t = c.ts + 1 + lane; t <= c.te; t += 32) acc = ge_add(acc, ge_load(A + 32 * (g0 + t)));
+    ge acc = lane == 0 ? ge_load16((c.starts_range ? A : B) + 32 * (g0 + c.ts)) : ge_identity();
+    for (uint64_t t = c.ts + 1 + lane; t <= c.te; t += 32) acc = ge_add(acc, ge_load16(A + 32 * (g0 + t)));
     for (int delta = 16; delta > 0; delta >>= 1) acc = ge_add(acc, ge_shfl_down(acc, delta));
-    if (lane == 0) ge_store(buckets + 32 * b, acc);
+    if (lane == 0) ge_store16(buckets + 32 * b, acc);
   }
 }
 
