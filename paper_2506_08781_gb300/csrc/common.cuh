@@ -775,17 +775,19 @@ struct PrepArgs {
 // ---- kernel declarations ----
 void launch_epoch_seeds(int inst, unsigned grid, unsigned block, cudaStream_t st, const DsNode* ds, int nds,
                         uint64_t e0, uint64_t ne, uint32_t* x0_out, uint32_t* status);
-// Multi-device batches compile their decoding and hashing for this many blocks per SM (128
-// registers a thread), so that three decoding blocks and one hashing block share an SM and
-// the hashing (ALU pipe) runs during the decoding (IMAD pipe) instead of after it.
-constexpr int kCoresidentMinBlocks = 4;
-// What shares the SMs with a hashing launch: nothing of its size; the decoding of one point per
-// entry; the same, both compiled for 128 registers a thread (multi-device batches).
-enum HashPlace { kHashAlone, kHashBeside, kHashCoresident };
+// Resident blocks of the decoding per SM (104 registers a thread); with the hashing of a
+// many-signer batch beside it (128 registers) one fewer, so that three decoding blocks and one
+// hashing block share an SM and the hashing (ALU pipe) runs during the decoding (IMAD pipe)
+// instead of after it: 128 signers of 8,192 entries 4.67 ms, with four decoding blocks 4.74.
+constexpr int kPointBlocksPerSm = 4;
+constexpr int kPointBlocksBeside = 3;
+// What shares the SMs with a hashing launch: nothing of its size, or the decoding of one point
+// per entry.
+enum HashPlace { kHashAlone, kHashBeside };
 unsigned hash_groups(int inst, int sm_count, uint64_t n);
 cudaError_t hash_kernels_init();   // once per device, before the first POSLO+ launch
 void launch_hash(int inst, unsigned groups, cudaStream_t st, HashArgs a, HashPlace place);
-void launch_points(unsigned grid, cudaStream_t st, const PointArgs& a, bool coresident = false);
+void launch_points(unsigned grid, cudaStream_t st, const PointArgs& a);
 struct ZPre { uint32_t w[10]; };   // BE words of "POSLO-Z" || verifier_seed || (byte 39 = 0)
 __global__ void k_weights(const ZPre zp, uint64_t n, uint64_t first, uint32_t* z_out);
 

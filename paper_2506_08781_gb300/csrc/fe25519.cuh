@@ -458,22 +458,22 @@ __device__ __forceinline__ fe fe_select(const fe& a, const fe& b, bool pick_b) {
 // 2^252 - 3.  A stage multiplies by the value it started from, by z^(2^10 - 1) (to reach 50), by
 // z^(2^50 - 1) (250) or by z (last).  One loop instead of a call per stage: the decoding runs as
 // one copy each of the squaring and the product (a few KB of code instead of 48), which a
-// launch of few points fetches from a cold instruction cache.
+// launch of few points fetches from a cold instruction cache.  The factors are indexed at run
+// time and so live in local memory, read eight times, instead of 24 registers held through
+// every squaring.
 __device__ __forceinline__ fe fe_pow_p58(const fe& z) {
   const fe z2 = fe_sq(z);
   const fe z9 = fe_mul(fe_sqn(z2, 2), z);
   fe cur = fe_mul(fe_sq(fe_mul(z9, z2)), z9);   // 2^5 - 1
-  fe z10 = cur, z50 = cur;
+  // what a stage multiplies by: 0 the value it started from, 1 z^(2^10 - 1), 2 z^(2^50 - 1), 3 z
+  fe keep[4];
+  keep[3] = z;
 #pragma unroll 1
   for (int k = 0; k < 8; ++k) {
     // squarings of the stages: 5, 10, 20, 10, 50, 100, 50, 2 (one byte each)
     const int n = (int)(0x023264320a140a05ull >> (8 * k) & 0xff);
-    fe m = fe_select(cur, z10, k == 3);
-    m = fe_select(m, z50, k == 6);
-    m = fe_select(m, z, k == 7);
-    cur = fe_mul(fe_sqn(cur, n), m);
-    z10 = fe_select(z10, cur, k == 0);
-    z50 = fe_select(z50, cur, k == 3);
+    keep[0x00020010u >> (4 * k) & 3] = cur;
+    cur = fe_mul(fe_sqn(cur, n), keep[0x32021010u >> (4 * k) & 3]);
   }
   return cur;
 }

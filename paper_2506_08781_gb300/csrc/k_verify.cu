@@ -390,13 +390,9 @@ __global__ void __launch_bounds__(kHashThreads * GROUPS, MINB) k_hash(const Hash
   }
 }
 
-#ifndef POSLO_POINTS_DYNAMIC
-#define POSLO_POINTS_DYNAMIC 1
-#endif
-
 // Strict decoding of R_t, its affine form for the MSM and its decode flag, and its addition
-// into the thread's unit sum.
-__device__ __forceinline__ void decode_one(const PointArgs& a, uint64_t t, ge& acc, uint32_t& bad) {
+// into the thread's unit sum (32 words at acc).
+__device__ __forceinline__ void decode_one(const PointArgs& a, uint64_t t, uint32_t* acc, uint32_t& bad) {
   const uint4* rp = reinterpret_cast<const uint4*>(a.R + 32 * t);
   const uint4 r0 = __ldg(rp), r1 = __ldg(rp + 1);
   const uint32_t b[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
@@ -414,19 +410,24 @@ __device__ __forceinline__ void decode_one(const PointArgs& a, uint64_t t, ge& a
     dst[4] = make_uint4(t2d.v[0], t2d.v[1], t2d.v[2], t2d.v[3]);
     dst[5] = make_uint4(t2d.v[4], t2d.v[5], t2d.v[6], t2d.v[7]);
   }
-  if (ok && !(a.skip && a.skip[t])) acc = ge_madd(acc, P.X, P.Y, t2d);
+  if (ok && !(a.skip && a.skip[t])) ge_store16(acc, ge_madd(ge_load16(acc), P.X, P.Y, t2d));
 }
 
 // Every R_t: blocks take chunks of kPointChunk points from a shared counter, so a block that
 // starts late (its SM busy with the hashing beside it) simply takes fewer chunks; then the
 // block's unit sum and decode-failure count.
-// MINB: 1 when the decoding runs on its own (146 registers), kCoresidentMinBlocks (128
-// registers) when three of its blocks share each SM with a hashing block.
-template <int MINB>
-__global__ void __launch_bounds__(kPointThreads, MINB) k_points(const PointArgs a) {
-  ge acc = ge_identity();
+//
+// Bound by the IMAD pipe (255 squarings and 28 products a point: 1.38 ms for 2^20 points with
+// every wide product at 4 cycles).  What a thread does not need during the squarings stays out
+// of its registers: its unit sum in its row of shared memory, the exponent chain's factors in
+// local memory.  104 registers instead of 146 let four blocks share an SM instead of three:
+// Distill of 2^20 entries 3.56 -> 3.47 ms.  Five blocks (94 registers) took 3.48 ms, six (80,
+// with the curve equation's terms spilt) 3.49 ms and 7 us more on a batch of 60.
+__global__ void __launch_bounds__(kPointThreads, kPointBlocksPerSm) k_points(const PointArgs a) {
+  __shared__ __align__(16) uint32_t sp[kPointThreads][32];
+  uint32_t* const acc = sp[threadIdx.x];
+  ge_store16(acc, ge_identity());
   uint32_t bad = 0;
-#if POSLO_POINTS_DYNAMIC
   __shared__ uint64_t s_base;
   for (;;) {
     if (threadIdx.x == 0) s_base = (uint64_t)atomicAdd(a.work, 1u) * kPointChunk;
@@ -437,18 +438,11 @@ __global__ void __launch_bounds__(kPointThreads, MINB) k_points(const PointArgs 
     const uint64_t end = min(base + kPointChunk, a.count);
     for (uint64_t t = base + threadIdx.x; t < end; t += blockDim.x) decode_one(a, t, acc, bad);
   }
-#else
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < a.count; t += stride)
-    decode_one(a, t, acc, bad);
-#endif
   // the block's sum by quads (a few us less at the end of a small launch than one lane per
   // addition), over as many points as the block can hold
-  __shared__ __align__(16) uint32_t sp[kPointThreads][32];
   __shared__ uint32_t sbad;
   if (threadIdx.x == 0) sbad = 0;
   __syncthreads();
-  ge_store(sp[threadIdx.x], acc);
   if (bad) atomicAdd(&sbad, bad);
   compact::quad_tree(sp, a.count < 1 ? 1 : a.count < kPointThreads ? (int)a.count : kPointThreads);
   if (threadIdx.x < 32) a.partial[(uint64_t)blockIdx.x * kPointPartialWords + threadIdx.x] = sp[0][threadIdx.x];
@@ -701,9 +695,8 @@ void launch_hash(int inst, unsigned groups, cudaStream_t st, HashArgs a, HashPla
   }
 }
 
-void launch_points(unsigned grid, cudaStream_t st, const PointArgs& a, bool coresident) {
-  if (coresident) k_points<kCoresidentMinBlocks><<<grid, kPointThreads, 0, st>>>(a);
-  else k_points<1><<<grid, kPointThreads, 0, st>>>(a);
+void launch_points(unsigned grid, cudaStream_t st, const PointArgs& a) {
+  k_points<<<grid, kPointThreads, 0, st>>>(a);
 }
 
 }  // namespace poslo

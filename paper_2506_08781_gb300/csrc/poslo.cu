@@ -600,18 +600,12 @@ int run_ytable(poslo_ctx* ctx, const uint8_t* Y, uint32_t** table_out, uint32_t*
   return POSLO_OK;
 }
 
-// Resident decode blocks per SM: below the register-file limit (4) the remaining registers
-// host a hash block, so SHA-256 (ALU pipe) runs beside the field arithmetic (IMAD pipe).
-#ifndef POSLO_POINTS_BLOCKS
-#define POSLO_POINTS_BLOCKS 3
-#endif
-
 // The decoding waits for `after` (an event on the main stream) when given, else for all main
 // stream work so far.
 int run_points(poslo_ctx* ctx, const uint8_t* R, uint64_t count, uint32_t* pts_out, uint8_t* bad_out,
-               uint32_t** partial_out, uint32_t* nblocks_out, cudaEvent_t after = nullptr, bool coresident = false) {
+               uint32_t** partial_out, uint32_t* nblocks_out, cudaEvent_t after = nullptr, int per_sm = kPointBlocksPerSm) {
   int rc;
-  const int blocks = grid_for(ctx, count, kPointThreads, POSLO_POINTS_BLOCKS);
+  const int blocks = grid_for(ctx, count, kPointThreads, per_sm);
   uint32_t* partial;
   if ((rc = ensure_t(ctx, "point_partial", (size_t)blocks * kPointPartialWords * 4, &partial))) return rc;
   if (!after) {
@@ -631,7 +625,7 @@ int run_points(poslo_ctx* ctx, const uint8_t* R, uint64_t count, uint32_t* pts_o
   CU(cudaMemsetAsync(work, 0, 4, ctx->s_points));
   cudaEvent_t tb, te;
   timer_begin(ctx, "points", ctx->s_points, &tb, &te);
-  launch_points((unsigned)blocks, ctx->s_points, a, coresident);
+  launch_points((unsigned)blocks, ctx->s_points, a);
   ++ctx->launch_count;
   CU(cudaGetLastError());
   timer_end(ctx, "points", ctx->s_points, tb, te);
@@ -3158,7 +3152,7 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
     if ((rc = launch_tables_seeds())) return rc;
     // (side stream) decode every R_t, compiled to share the SMs with the hashing
     uint32_t *ppart, npb;
-    if ((rc = run_points(ctx, sb.R, N, pts, badR, &ppart, &npb, nullptr, true))) return rc;
+    if ((rc = run_points(ctx, sb.R, N, pts, badR, &ppart, &npb, nullptr, kPointBlocksBeside))) return rc;
     // the weights z_t alone (they depend only on the batch position), so the MSM's counting
     // sort runs beside the decoding; the segmented hashing (per-entry e_t) on its own stream
     ZPre zp;
@@ -3176,7 +3170,7 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
       a.z_in = z;
       cudaEvent_t tb, te;
       timer_begin(ctx, "hash", ctx->s_hash, &tb, &te);
-      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->s_hash, a, kHashCoresident);
+      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->s_hash, a, kHashBeside);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", ctx->s_hash, tb, te);
