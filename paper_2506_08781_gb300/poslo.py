@@ -426,8 +426,8 @@ class Context:
         ccd = dict(s_v=sv.tobytes(), R_v=Rv.tobytes(),
                    umbrellas=[(umb[64 * l:64 * l + 32].tobytes(), umb[64 * l + 32:64 * l + 64].tobytes())
                               for l in range(n_umbrella)],
-                   invalid=[int(x) for x in inv[:c.n_invalid]])
-        return [bool(v) for v in valid[:n1]], ccd
+                   invalid=inv[:c.n_invalid].tolist())
+        return valid[:n1].astype(bool).tolist(), ccd
 
     def sebver_c(self, b: BatchData, n_umbrella: int, ccd: dict, mode: str):
         """SeBVer in mode 'V', 'U' or 'I' against a ccd from distill_c; returns the bits."""
@@ -440,7 +440,7 @@ class Context:
         bits = np.zeros(max(n, 1), np.uint8)
         cb = self._cbatch(b)
         self._check(self.lib.poslo_sebver_c(self.h, C.byref(cb), n_umbrella, C.byref(c), ord(mode), _ptr(bits)))
-        return [bool(x) for x in bits[:n]]
+        return bits[:n].astype(bool).tolist()
 
     # ------------------------------------------------------------------ serving
     def serve_start(self, workers: int = 2, max_batch_devices: int = 4096, max_batch_entries: int = 1 << 22):
