@@ -131,10 +131,8 @@ __device__ __forceinline__ void bisect_pass(const TreeArgs& a, const uint64_t* f
 // only adds checks of nodes whose ancestors failed: every entry that fails its own check is
 // still found, and entries are flagged only by their own check.
 //
-// A step takes 59 us for 640 checks and about 100 us for 2,048 to 3,700 (throughput of the
-// point additions); as many lanes per check as the grid has for their number keep the latency
-// short (one lane's 16 additions in groups of 8 lanes before: 100 to 120 us a step also with 160
-// checks).
+// A step takes about 40 us for 1,300 checks and 75 for 4,200 (the chains of point additions; as
+// many lanes per check as the grid has for their number keep them short).
 __global__ void __launch_bounds__(128, POSLO_BISECT_MINB) k_bisect_step(const TreeArgs a, BisectState st, int step,
                                                      uint64_t slots, const uint32_t* tY, const uint32_t* tG,
                                                      uint8_t* invalid) {

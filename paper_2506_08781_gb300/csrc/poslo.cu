@@ -1984,15 +1984,18 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
   bool confirmed = false;
   // the ordered list of flagged entries and ccd^v over the others from the local list fidx (its
   // count on the device); ccd^v's point is the batch's unit sum (from the first stage) minus the
-  // flagged entries' points.  On st, then ev_result
-  auto launch_result = [&](cudaStream_t st) -> int {
+  // flagged entries' points.  On st, the scalars' side on another stream (two chains of 44 and 58
+  // us at 2^20 entries with 1,049 flagged), then ev_result
+  auto launch_result = [&](cudaStream_t st, cudaStream_t scalars) -> int {
+    k_sum_scalars<<<sblocks, kHashThreads, 0, scalars>>>(sb.s, n, inv, sp);
+    k_reduce_scalars<<<1, 256, 0, scalars>>>(sp, sblocks, d_ccd);
+    if (scalars != st) CU(cudaEventRecord(ctx->ev_hash, scalars));
     k_shift_list<<<grid_for(ctx, capn, 256, 4), 256, 0, st>>>(fidx, fidx + n, std::min(cap, n), batch->first_index,
                                                               d_idx);
-    k_sum_scalars<<<sblocks, kHashThreads, 0, st>>>(sb.s, n, inv, sp);
-    k_reduce_scalars<<<1, 256, 0, st>>>(sp, sblocks, d_ccd);
     k_ccd_points<<<1, 256, 0, st>>>(pts, badR, fidx, fidx + n, unitR, d_ccd + 32);
     ctx->launch_count += 4;
     CU(cudaGetLastError());
+    if (scalars != st) CU(cudaStreamWaitEvent(st, ctx->ev_hash, 0));
     CU(cudaEventRecord(ctx->ev_result, st));
     return POSLO_OK;
   };
@@ -2065,7 +2068,8 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     k_flags_or<<<grid_for(ctx, n, 256, 4), 256, 0, ctx->s_main>>>(badR, badS, nullptr, n, inv);
     ++ctx->launch_count;
     timer_begin(ctx, "bisect", ctx->s_main, &tb, &te);
-    for (int step = 0; step <= (int)top; ++step) {   // the first step reaches `top`, each other one at least a level
+    // the first step reaches `top`, each other one descends at least two levels (or the last one)
+    for (int step = 0; step <= (int)(top + 1) / 2; ++step) {
       k_bisect_step<<<bgrid, 128, 0, ctx->s_main>>>(ta, bst, step, slots, tableY, ctx->tableG, inv);
       ++ctx->launch_count;
     }
@@ -2077,7 +2081,7 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     if ((rc = run_compact(ctx, inv, n, 0, fidx, n, fidx + n))) return rc;
     CU(cudaMemcpyAsync(&nf, fidx + n, 8, cudaMemcpyDeviceToHost, ctx->s_main));
     CU(cudaStreamSynchronize(ctx->s_main));
-    if ((rc = launch_result(ctx->s_points))) return rc;
+    if ((rc = launch_result(ctx->s_points, ctx->s_hash))) return rc;
     timer_begin(ctx, "confirm", ctx->s_main, &tb, &te);
     const MsmPlan pl1 = msm_plan(ctx, n, 4);
     if (nf == 0) {
@@ -2168,7 +2172,7 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     // the per-entry checks set the flags (direct localisation, or the fallback after a failed
     // confirmation): list them now
     if ((rc = run_compact(ctx, inv, n, 0, fidx, n, fidx + n))) return rc;
-    if ((rc = launch_result(ctx->s_main))) return rc;
+    if ((rc = launch_result(ctx->s_main, ctx->s_main))) return rc;
     CU(cudaMemcpyAsync(&cnt, fidx + n, 8, cudaMemcpyDeviceToHost, ctx->s_main));
     CU(cudaMemcpyAsync(hccd, d_ccd, 64, cudaMemcpyDeviceToHost, ctx->s_main));
     if ((rc = check_status(ctx))) return rc;
