@@ -332,24 +332,26 @@ int validate_batch(poslo_ctx* ctx, const poslo_batch* b) {
 // One verification call indexes its entries with 32-bit indices inside the MSM and the
 // localisation; longer logs go through poslo_distill_stream in chunks.
 constexpr uint64_t kMaxCallEntries = (1ull << 32) - 1;
-// Distill batches up to this many entries are localised by every entry's own check (one
-// launch, eight lanes per entry) rather than by the descent over the segment tree: measured
-// on GB300, 0.18 ms of checking at 4,096 entries and 0.56 ms at 16,384 against 1.0 ms of
-// tree, descent and confirmation; the two meet near 32,768.
+// Distill batches up to this many entries whose weighted check failed are localised by every
+// entry's own check (one launch) rather than by the descent over the segment tree: 0.33 ms at
+// 16,384 entries, where tree, descent and confirmation take 0.3 to 0.4 ms for a few flips.
 constexpr uint64_t kDirectCheckMax = 16384;
+
+// Flagged entries up to which a confirmation subtracts them window by window (one quad per
+// entry and window) instead of by an MSM over them and Horner's rule over the windows.
+constexpr uint64_t kConfirmWindowsMax = 4096;
 
 // Batches of at most this many entries are checked entry by entry at once, without the weighted
 // check of the batch before it (no weights, no MSM): the definition itself, in one launch whose
 // latency at this size is below that of the MSM's chain of short kernels, and the same work
-// whether the batch is valid or not.  Measured on GB300 (weighted check first / direct, us):
-// Distill of a valid batch 300 / 186 at 1,024 entries, 297 / 254 at 4,096, 305 / 304 at 6,000,
-// 308 / 374 at 8,192, with flips 510 / 199 at 1,024, 568 / 287 at 4,096; many signers with one
-// flipped entry 1,252 / 209 at 300 entries, 1,344 / 382 at 5,000, 1,418 / 512 at 8,000.
-// Flagged entries up to which a confirmation subtracts them window by window (one quad per
-// entry and window) instead of by an MSM over them and Horner's rule over the windows.
-constexpr uint64_t kConfirmWindowsMax = 4096;
-constexpr uint64_t kDirectFirstMax = 4096;        // Distill
-constexpr uint64_t kMultiDirectFirstMax = 8192;   // many signers
+// whether the batch is valid or not.  Measured on GB300, direct / weighted check first, us:
+//   Distill, valid       226 / 268 at 6,000 entries, 262 / 270 at 8,192, 293 / 278 at 12,000
+//   Distill, 0.1 % flips 253 / 489,                  287 / 518,          319 / 549
+//   32 signers, valid    380 / 468 at 12,000, 466 / 501 at 16,384 (a flip: 381 / 819, 471 / 871)
+// so Distill's line is where a valid batch is still the faster of the two, and the many signers'
+// the largest batch of the lane-parallel check.
+constexpr uint64_t kDirectFirstMax = 8192;         // Distill
+constexpr uint64_t kMultiDirectFirstMax = 16384;   // many signers
 static_assert(kDirectFirstMax <= kDirectCheckMax && kMultiDirectFirstMax <= kMultiGroupCheckMax, "sizes of the checks");
 
 // Host inputs are copied R_t first: ev_staged marks their arrival, so the decoding (the

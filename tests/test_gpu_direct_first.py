@@ -84,3 +84,14 @@ def test_many_signers_at_the_edges(ctx, sizes, flips):
         with pytest.raises(poslo.PosloError) as e:
             ctx.aver_multi(*args, cap=1)
         assert e.value.code == poslo.POSLO_EBUFSMALL
+
+
+@pytest.mark.parametrize("n,flips", [(8192, 0), (8192, 9), (8192, 8192), (8193, 9)])
+def test_distill_at_the_upper_edge(ctx, n, flips):
+    Y, msgs, s, R, ds = _log(n, n, first=3)
+    bad = synth.apply_tamper(msgs, synth.tamper_plan(n, msgs, flips)) if flips else msgs
+    want = X.distill_f(Y, bad.data, bad.offs, 3, N2, s.tobytes(), R.tobytes(), ds)
+    b = ctx.make_batch(poslo.VARIANT_F, N2, Y, bad.data, bad.offs, s, R, ds, first_index=3)
+    for _ in range(2):
+        idx, cs, cR = ctx.distill(b)
+        assert ([int(t) for t in idx], cs, cR) == want

@@ -36,6 +36,12 @@ def _shift(s, t, delta):
     ([8000, 8385, 5], [7999, 8000], None),
     ([9000, 500, 300], [9100], (17, 8000)),
     ([9000, 500, 300], [], (17, 8000)),
+    ([16385, 500, 300], [], None),
+    ([16385, 500, 300], [16500], None),
+    ([16385, 500, 300], [16500], (17, 8000)),
+    ([16385, 500, 300], [5, 17100], None),
+    ([9000, 7384], [8999], None),
+    ([9000, 7385], [8999], None),
 ])
 def test_flagged_signers_beside_and_behind(ctx, sizes, flips, pair):
     data, lens, ss, Rs, keys, stacks = [], [], [], [], [], []
