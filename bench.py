@@ -151,19 +151,19 @@ def probe_int_peaks(device: int) -> dict:
 # Algorithmic integer work per entry for the roofline (counted from the algorithms, not
 # from the compiled code):
 #   decoding R_t (k_points): 255 squarings and 21 multiplications in F_p, plus the 7
-#     multiplications of its mixed addition into the unit sum.  Counted per half of a
-#     32x32-bit product: a squaring has 28 cross products and 8 diagonal squares (low and
-#     high halves) and a fold by 38 (8 low + 8 high + 1 low): 45 low, 44 high; a
-#     multiplication has 64 products and the fold: 73 low, 72 high.
-#   mad.hi issues at half the rate of mad.lo on this GPU (probed), so the work is expressed
-#     in mad.lo issue slots: low + high x (mad.lo rate / mad.hi rate).
+#     multiplications of its mixed addition into the unit sum.  Counted in 32x32 -> 64 bit
+#     products: a squaring has 28 cross products, 8 diagonal squares and a fold by 38 (8),
+#     44 in all; a multiplication has 64 products and the fold, 72; each has one more low
+#     half (the fold by 19).
+#   A 64-bit product (mad.lo.cc / madc.hi.cc fused into one wide multiply-add) takes two
+#     mad.lo issue slots on this GPU, so the work is expressed in those: 2 x wide + low.
 #   SHA-256: 1,384 ALU instructions per compression with 3-input LOP3/IADD3 and funnel
 #     shifts (64 rounds x 14 + 48 schedule words x 10 + 8); compressions per entry =
 #     1 (PRF) + ceil((L + 25) / 64) (H)
-SQ_LO, SQ_HI, MUL_LO, MUL_HI = 45, 44, 73, 72
+SQ_WIDE, MUL_WIDE = 44, 72
 DECODE_SQ, DECODE_MUL = 255, 21 + 7
-IMAD_LO_PER_DECODE = DECODE_SQ * SQ_LO + DECODE_MUL * MUL_LO    # 13,519
-IMAD_HI_PER_DECODE = DECODE_SQ * SQ_HI + DECODE_MUL * MUL_HI    # 13,236
+WIDE_PER_DECODE = DECODE_SQ * SQ_WIDE + DECODE_MUL * MUL_WIDE    # 13,236
+IMAD_SLOTS_PER_DECODE = 2 * WIDE_PER_DECODE + DECODE_SQ + DECODE_MUL
 ALU_PER_COMPRESSION = 64 * 14 + 48 * 10 + 8
 # DRAM bytes (read + write) of one k_points launch over 2^20 entries, from an ncu capture:
 # the 32 MB of encodings read once; of the 100 MB of decoded points written, the part that has
@@ -526,12 +526,12 @@ def bench_stream(device: int) -> dict:
 # Thread instructions per AES-128 of the table cipher with its on-the-fly key schedule, counted
 # from the algorithm (not the compiled code): each of the 16 round lookups and 4 key-schedule
 # S-box lookups is a byte extract, an address computation and a shared-memory read (3); a full
-# round adds 12 rotations, 8 three-input XORs and 15 key-schedule operations (masks, shifts,
-# the XOR chain, Rcon): 9 x (60 + 12 + 8 + 15) = 855; the last round's 16 S-box reads with their
-# masks and shifts (4 x 20) + 4 XORs + its key schedule (27) = 111; the initial AddRoundKey 4;
-# the MMO/MDC-2 feed-forward XOR 4: about 974.  The kernel is bound by instruction issue (the
-# ALU and shared-memory pipes share the 4 schedulers of an SM), so this count is its roofline.
-AES_INSTR = 9 * (16 * 3 + 4 * 3 + 12 + 8 + 15) + (4 * 20 + 4 + 27) + 4 + 4
+# round adds 8 three-input XORs and 15 key-schedule operations (masks, shifts, the XOR chain,
+# Rcon): 9 x (60 + 8 + 15) = 747; the last round's 16 S-box reads with their masks and shifts
+# (4 x 20) + 4 XORs + its key schedule (27) = 111; the initial AddRoundKey 4; the MMO/MDC-2
+# feed-forward XOR 4: 866 (the four rotated tables leave no rotations).  Instruction issue is one
+# bound; the 200 table reads (one shared-memory wavefront a lane) are the other, nearly met.
+AES_INSTR = 9 * (16 * 3 + 4 * 3 + 8 + 15) + (4 * 20 + 4 + 27) + 4 + 4
 
 
 CCD_UMBRELLAS = 64
@@ -1117,8 +1117,7 @@ def run_ours(args):
     dom = "points" if "points" in kernels else None
     roof = None
     if dom in ("points", "check") and peaks:
-        hi_cost = peaks["imad_lo_ops"] / peaks["imad_hi_ops"]
-        work = n * (IMAD_LO_PER_DECODE + IMAD_HI_PER_DECODE * hi_cost)
+        work = n * IMAD_SLOTS_PER_DECODE
         ach = work / (kernels[dom]["ms_per_launch"] * 1e-3) / 1e9
         pk = peaks["imad_lo_ops"] / 1e9
         roof = {"bound": "alu", "pipe": "IMAD", "kernel": dom, "achieved": ach, "peak": pk, "unit": "Gop/s",
@@ -1126,8 +1125,8 @@ def run_ours(args):
                 "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_points launch "
                                   "at 2^20 entries",
                 "peak_source": "probed mad.lo.u32 issue rate on this GPU (probe/peaks.cu)",
-                "work": f"{IMAD_LO_PER_DECODE:,} mad.lo + {IMAD_HI_PER_DECODE:,} mad.hi per R_t decode and its "
-                        f"unit-sum addition; mad.hi counted as {hi_cost:.2f} mad.lo issue slots (probed rate ratio)",
+                "work": f"{WIDE_PER_DECODE:,} 64-bit products per R_t decode and its unit-sum addition, two mad.lo "
+                        f"issue slots each, and one mad.lo per field product",
                 "timing": "k_points duration on its own stream during the timed steps (it shares the GPU with "
                           "the hashing and the counting sort, so this understates the kernel alone)"}
     elif dom == "hash" and peaks:
