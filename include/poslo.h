@@ -451,7 +451,8 @@ void poslo_reset_kernel_times(poslo_ctx* ctx);
 /* ---- CUDA-graph replay (no counterpart in the paper) ------------------------------------ */
 
 /* poslo_aver_multi and poslo_distill run their work up to the first host decision (the
- * combined weighted check) as a fixed sequence of launches.  When a call has the same shape
+ * combined weighted check; of small batches, every entry's own check) as a fixed sequence of
+ * launches.  When a call has the same shape
  * as the previous call of that entry point on this context -- for poslo_aver_multi the
  * device count, segment tables, seeds layout, batch pointers (device-resident inputs) and
  * MSM plan; for poslo_distill a device-resident batch with the same pointers, n, n2,
