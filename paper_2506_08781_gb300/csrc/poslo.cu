@@ -673,7 +673,7 @@ int run_points_rest(poslo_ctx* ctx, const PointsRest& rest) {
 
 // Pippenger plan: the window c comes from the context (poslo_params.msm_window) or from the
 // autotuned table for this size class (see poslo_msm_autotune); the default before tuning is
-// c = log2(n) - 4 clamped to [8, 16].
+// c = log2(n) - 4 clamped to [8, 16] (16 already from 2^19.5 entries with 127-bit weights).
 MsmPlan msm_plan_c(int c, int sw, int seg_log2 = kMsmSegLog2Min) {
   MsmPlan pl;
   pl.c = c;
@@ -727,7 +727,12 @@ MsmPlan msm_plan(poslo_ctx* ctx, uint64_t n, int sw) {
     const int lg = log2_floor(n);
     auto it = ctx->msm_tuned.find(lg * 16 + sw);
     if (it != ctx->msm_tuned.end()) return msm_plan_c(it->second & 0xff, sw, it->second >> 8);
-    c = msm_balanced_width(std::min(16, std::max(8, lg - 4)), sw);
+    // weights of 127 bits from 2^19.5 entries: 8 windows of 16 bits instead of 9 of 15, whose last has
+    // 7 bits (its 128 counters also slow the counting, 72 -> 210 us).  Distill of 750,000 entries
+    // 2.72 -> 2.62 ms, of 1,000,000 3.53 -> 3.34; at 500,000 1.91 -> 1.92, and rounding up at the
+    // narrower widths gave between -1 and 2.5 %, so only here
+    const bool wide = sw == 4 && lg == 19 && n >= 741455;
+    c = msm_balanced_width(std::min(16, std::max(8, lg - 4 + (wide ? 1 : 0))), sw);
   }
   MsmPlan pl = msm_plan_c(c, sw);
   pl.seg_log2 = msm_seg_default(pl, n, ctx->sm_count);
