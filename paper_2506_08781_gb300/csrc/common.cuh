@@ -779,7 +779,7 @@ void launch_epoch_seeds(int inst, unsigned grid, unsigned block, cudaStream_t st
 // Resident blocks of the decoding per SM (104 registers a thread); with the hashing of a
 // many-signer batch beside it (128 registers) one fewer, so that three decoding blocks and one
 // hashing block share an SM and the hashing (ALU pipe) runs during the decoding (IMAD pipe)
-// instead of after it: 128 signers of 8,192 entries 4.67 ms, with four decoding blocks 4.74.
+// instead of after it: 128 signers of 1,000,000 entries together 4.67 ms, with four decoding blocks 4.74.
 // (One signer's batch starts its decoding before the seeds and the weights, as soon as the
 // points have landed, and there the same split measured 3.45 - 3.57 ms against 3.47 of 2^20
 // entries, and 736 us against 718 of 40,013: not taken.)

@@ -656,7 +656,7 @@ int run_points(poslo_ctx* ctx, const uint8_t* R, uint64_t count, uint32_t* pts_o
 
 // Behind the hashing on the hashing stream: the decoding's remaining blocks (they share its chunk
 // counter, so they take over part of what is left; none left is none taken), then the decoding's
-// events on the points stream.  128 signers of 8,192 entries: 4.41 -> 4.35 ms.
+// events on the points stream.  128 signers of 1,000,000 entries together: 4.41 -> 4.35 ms.
 int run_points_rest(poslo_ctx* ctx, const PointsRest& rest) {
   if (rest.blocks) {
     CU(cudaStreamWaitEvent(ctx->s_hash, ctx->ev_rest, 0));
@@ -3212,7 +3212,7 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
   auto stage1 = [&]() -> int {
     int rc;
     if ((rc = launch_tables_seeds())) return rc;
-    // (side stream) decode every R_t, compiled to share the SMs with the hashing
+    // (side stream) decode every R_t, three blocks per SM with the hashing beside them
     uint32_t *ppart, npb;
     PointsRest rest;
     if ((rc = run_points(ctx, sb.R, N, pts, badR, &ppart, &npb, nullptr, &rest))) return rc;
@@ -3254,7 +3254,7 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
     } else {
       // beside the last launches of the MSM, Horner's rule over the windows among them (one
       // warp), instead of behind them: with the entry checks beside the confirmation below,
-      // 128 signers of 8,192 entries, two of them with a flip, 4.64 -> 4.41 ms
+      // 128 signers of 1,000,000 entries together, two with a flip, 4.64 -> 4.41 ms
       CU(cudaStreamWaitEvent(ctx->s_hash, ctx->ev_summed, 0));
     }
     cudaStream_t ts = per_window ? ctx->s_main : ctx->s_hash;   // the devices' sums
