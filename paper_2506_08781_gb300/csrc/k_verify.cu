@@ -2,6 +2,7 @@
 // window tables and the final cofactored check.
 #include "common.cuh"
 #include "compact.cuh"
+#include "stage.h"
 
 namespace poslo {
 
@@ -97,24 +98,21 @@ __global__ void k_weights(const ZPre zp, uint64_t n, uint64_t first, uint32_t* z
 // warp's loads touches 32 lines), and a last block's tail words come from a column of shared
 // memory instead of selects: 2^20 x U[32, 256] bytes 422 -> 375 us, weighted 464 -> 407 us, 16
 // bytes 184 -> 170 us.  Tiles of more than kStageMax bytes (and malformed ones) are read
-// directly.  The copy keeps the
-// bytes' alignment modulo 16 and reads no 4-byte word without a message byte in it.
+// directly.  The copy keeps the bytes' alignment modulo 16 and reads no 4-byte word without a
+// message byte in it (stage.h).
 constexpr uint32_t kStageBytes = 40960;              // with the rest below 48 KiB: four blocks per SM
 constexpr uint32_t kStageMax = kStageBytes - 16 - 112;   // a last block is read up to 112 bytes past its message
 constexpr int kTailRows = 6;                         // x || 0x80 shifted into place (5 words), a zero word
 
 __device__ __forceinline__ void stage_tile(uint32_t* stage, const uint8_t* src, uint32_t total) {
-  const uint32_t a0 = (uint32_t)(reinterpret_cast<uintptr_t>(src) & 15u), end = a0 + total;
+  const uint32_t a0 = (uint32_t)(reinterpret_cast<uintptr_t>(src) & 15u);
   const uint8_t* s16 = src - a0;
-  const uint32_t lo = (a0 + 15) >> 4, hi = end >> 4;   // whole granules
-  for (uint32_t i = lo + threadIdx.x; i < hi; i += blockDim.x)
+  const uint32_t hi = stage_granule_hi(a0, total);
+  for (uint32_t i = stage_granule_lo(a0) + threadIdx.x; i < hi; i += blockDim.x)
     reinterpret_cast<uint4*>(stage)[i] = __ldg(reinterpret_cast<const uint4*>(s16) + i);
-  if (threadIdx.x < 8) {   // the granules at the two ends, word by word
-    const bool tail = threadIdx.x >= 4;
-    const uint32_t g = tail ? hi : 0u, w = 4 * g + (threadIdx.x & 3);
-    const bool partial = tail ? (end & 15u) != 0 && !(hi == 0 && a0 != 0) : a0 != 0;
-    if (partial && 4 * w + 4 > a0 && 4 * w < end) stage[w] = __ldg(reinterpret_cast<const uint32_t*>(s16) + w);
-  }
+  uint32_t w;
+  if (threadIdx.x < 8 && stage_end_word(a0, total, threadIdx.x, w))
+    stage[w] = __ldg(reinterpret_cast<const uint32_t*>(s16) + w);
 }
 
 // The 16 words of the block at word offset ob of the padded stream m || x || 0x80 || 0..: message
