@@ -67,6 +67,7 @@ int ensure(poslo_ctx* ctx, const char* name, size_t bytes, void** out) {
       cudaStreamSynchronize(ctx->s_main);
       cudaStreamSynchronize(ctx->s_table);
       cudaStreamSynchronize(ctx->s_points);
+      cudaStreamSynchronize(ctx->s_hash);
       cudaFree(b.p);
       ctx->mem_used -= b.cap;
       b.p = nullptr;
@@ -252,6 +253,22 @@ int run_replayable(poslo_ctx* ctx, poslo_host::GraphSlot& g, const std::vector<u
   CU(cudaGraphLaunch(g.exec, ctx->s_main));
   return POSLO_OK;
 }
+
+// Nothing that a verification call has launched is still running when it returns: a call that
+// succeeds ends synchronised and disarms this, and an early return (a workspace that the memory
+// budget refuses while other streams already work, say) waits here for every stream, because what
+// is running reads the caller's arrays, which the caller may release, and writes buffers that the
+// next call uses on other streams.
+struct DrainOnError {
+  poslo_ctx* ctx;
+  bool copies = false;   // the copy stream too (distill_stream; a service's staging thread owns it otherwise)
+  bool armed = true;
+  ~DrainOnError() {
+    if (!armed) return;
+    for (cudaStream_t st : {ctx->s_main, ctx->s_table, ctx->s_points, ctx->s_hash}) cudaStreamSynchronize(st);
+    if (copies) cudaStreamSynchronize(ctx->s_copy);
+  }
+};
 
 uint32_t log2_exact(uint32_t n) {
   if (n == 0 || (n & (n - 1))) return 0xffffffffu;
@@ -1418,6 +1435,7 @@ int poslo_hash_entries(poslo_ctx* ctx, const poslo_batch* batch, uint8_t* e_out)
   if ((rc = validate_batch(ctx, batch))) return rc;
   if (batch->on_device && (reinterpret_cast<uintptr_t>(e_out) & 15))
     return fail(ctx, POSLO_EINVAL, "device-resident e_out must be 16-byte aligned");
+  DrainOnError drain{ctx};
   if ((rc = reset_status(ctx))) return rc;
   Staged sb;
   if ((rc = stage_batch(ctx, batch, sb))) return rc;
@@ -1428,7 +1446,9 @@ int poslo_hash_entries(poslo_ctx* ctx, const poslo_batch* batch, uint8_t* e_out)
   if ((rc = run_hash(ctx, batch, sb, d_e, false, false, nullptr, &partial, &nb, true))) return rc;
   if (!batch->on_device && batch->n)
     CU(cudaMemcpyAsync(e_out, d_e, 32 * batch->n, cudaMemcpyDeviceToHost, ctx->s_main));
-  return check_status(ctx);
+  if ((rc = check_status(ctx))) return rc;
+  drain.armed = false;
+  return POSLO_OK;
 }
 
 int poslo_aver(poslo_ctx* ctx, const poslo_batch* batch, uint32_t agg_mode, uint8_t* accept) {
@@ -1440,6 +1460,7 @@ int poslo_aver(poslo_ctx* ctx, const poslo_batch* batch, uint32_t agg_mode, uint
   if (agg_mode == POSLO_AGG_WEIGHTED && !F) return fail(ctx, POSLO_EINVAL, "weighted aggregation needs POSLO-F");
   if (agg_mode > POSLO_AGG_WEIGHTED) return fail(ctx, POSLO_EINVAL, "bad aggregation mode");
   const bool weighted = agg_mode == POSLO_AGG_WEIGHTED;
+  DrainOnError drain{ctx};
   if ((rc = reset_status(ctx))) return rc;
   Staged sb;
   if ((rc = stage_batch(ctx, batch, sb))) return rc;
@@ -1487,6 +1508,7 @@ int poslo_aver(poslo_ctx* ctx, const poslo_batch* batch, uint32_t agg_mode, uint
   CU(cudaMemcpyAsync(&h_acc, d_acc, 1, cudaMemcpyDeviceToHost, ctx->s_main));
   if ((rc = check_status(ctx))) return rc;
   kforget.armed = false;   // the key decoded: its table is sound
+  drain.armed = false;
   *accept = h_acc;
   return POSLO_OK;
 }
@@ -1505,6 +1527,7 @@ int poslo_aver_partial(poslo_ctx* ctx, const poslo_batch* batch, uint32_t agg_mo
   if (agg_mode > POSLO_AGG_WEIGHTED) return fail(ctx, POSLO_EINVAL, "bad aggregation mode");
   const bool weighted = agg_mode == POSLO_AGG_WEIGHTED;
   const uint64_t n = batch->n;
+  DrainOnError drain{ctx};
   if ((rc = reset_status(ctx))) return rc;
   Staged sb;
   if ((rc = stage_batch(ctx, batch, sb))) return rc;
@@ -1623,6 +1646,7 @@ int poslo_aver_partial(poslo_ctx* ctx, const poslo_batch* batch, uint32_t agg_mo
   uint32_t* h = reinterpret_cast<uint32_t*>(ctx->h_small);   // page-locked: no staging, one sync
   CU(cudaMemcpyAsync(h, rec, 4 * kShardWords, cudaMemcpyDeviceToHost, ctx->s_main));
   if ((rc = check_status(ctx))) return rc;
+  drain.armed = false;
   memcpy(out->e, h, 32);
   memcpy(out->s, h + 8, 32);
   memcpy(out->R, h + 16, 128);
@@ -1648,6 +1672,7 @@ int poslo_combine_check(poslo_ctx* ctx, const uint8_t Y[32], const poslo_partial
     n_all += parts[i].n;
   }
   int rc;
+  DrainOnError drain{ctx};
   if ((rc = reset_status(ctx))) return rc;
   uint32_t* tableY;
   std::vector<const uint32_t*> ktab;
@@ -1689,6 +1714,7 @@ int poslo_combine_check(poslo_ctx* ctx, const uint8_t Y[32], const poslo_partial
   CU(cudaMemcpyAsync(ctx->h_small + sizeof(poslo_partial), d_acc, 1, cudaMemcpyDeviceToHost, ctx->s_main));
   if ((rc = check_status(ctx))) return rc;
   kforget.armed = false;   // the key decoded: its table is sound
+  drain.armed = false;
   *accept = ctx->h_small[sizeof(poslo_partial)];
   if (total) {
     memcpy(total->e, h, 32);
@@ -1715,6 +1741,7 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
   if (batch->n > kMaxCallEntries) return fail(ctx, POSLO_EINVAL, "more than 2^32 - 1 entries in one call");
   const uint64_t n = batch->n;
   const uint64_t n1 = std::max<uint64_t>(n, 1);
+  DrainOnError drain{ctx};
   if ((rc = reset_status(ctx))) return rc;
   Staged sb;
   if ((rc = stage_batch(ctx, batch, sb))) return rc;
@@ -1885,6 +1912,7 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     CU(cudaMemcpyAsync(ctx->h_small, d_out, kDirectOutHeader + 8 * first, cudaMemcpyDeviceToHost, ctx->s_main));
     if ((rc = check_status(ctx))) return rc;
     kforget.armed = false;   // the key decoded: its table is sound
+    drain.armed = false;
     uint64_t cnt;
     memcpy(&cnt, ctx->h_small + 64, 8);
     const uint64_t got = std::min(cnt, capd);
@@ -1977,6 +2005,7 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
   // h_acc covers "no malformed entry and the weighted equation holds": then no entry is
   // invalid and ccd^v is the unit sums of the whole batch, already read
   if (h_acc) {
+    drain.armed = false;
     *n_invalid = 0;
     if (ccd_s) memcpy(ccd_s, hccd, 32);
     if (ccd_R) memcpy(ccd_R, hccd + 32, 32);
@@ -2184,6 +2213,7 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     CU(cudaMemcpyAsync(hccd, d_ccd, 64, cudaMemcpyDeviceToHost, ctx->s_main));
     if ((rc = check_status(ctx))) return rc;
   }
+  drain.armed = false;
   const uint64_t got = std::min(cnt, cap);
   if (got && invalid_idx) CU(cudaMemcpy(invalid_idx, d_idx, 8 * got, cudaMemcpyDeviceToHost));
   *n_invalid = cnt;
@@ -2209,6 +2239,7 @@ int poslo_agg(poslo_ctx* ctx, const uint8_t* scalars, const uint8_t* points, uin
     return POSLO_OK;
   }
   int rc;
+  DrainOnError drain{ctx};
   if ((rc = reset_status(ctx))) return rc;
   const void *dp, *dsc;
   if ((rc = stage(ctx, "agg_pts_in", points, 32 * n, on_device, ctx->s_main, &dp))) return rc;
@@ -2233,6 +2264,7 @@ int poslo_agg(poslo_ctx* ctx, const uint8_t* scalars, const uint8_t* points, uin
   CU(cudaMemcpyAsync(h, d_out, 64, cudaMemcpyDeviceToHost, ctx->s_main));
   CU(cudaMemcpyAsync(&bad, d_bad, 4, cudaMemcpyDeviceToHost, ctx->s_main));
   if ((rc = check_status(ctx))) return rc;
+  drain.armed = false;
   if (bad) return fail(ctx, POSLO_EINVAL, "%u points do not decode", bad);
   memcpy(s_out, h, 32);
   memcpy(R_out, h + 32, 32);
@@ -2246,11 +2278,13 @@ int poslo_msm(poslo_ctx* ctx, const uint8_t* points, const uint8_t* scalars, uin
   if (on_device && n && ((reinterpret_cast<uintptr_t>(points) | reinterpret_cast<uintptr_t>(scalars)) & 15))
     return fail(ctx, POSLO_EINVAL, "device-resident points and scalars must be 16-byte aligned");
   int rc;
+  DrainOnError drain{ctx};
   if ((rc = reset_status(ctx))) return rc;
   const void *dp, *ds;
   if ((rc = stage(ctx, "msm_pts_in", points, 32 * n, on_device, ctx->s_main, &dp))) return rc;
   if ((rc = stage(ctx, "msm_sc_in", scalars, 32 * n, on_device, ctx->s_main, &ds))) return rc;
   if (n == 0) {
+    drain.armed = false;
     out[0] = 1;
     memset(out + 1, 0, 31);
     return POSLO_OK;
@@ -2278,6 +2312,7 @@ int poslo_msm(poslo_ctx* ctx, const uint8_t* points, const uint8_t* scalars, uin
   CU(cudaMemcpyAsync(h, d_out, 32, cudaMemcpyDeviceToHost, ctx->s_main));
   CU(cudaMemcpyAsync(&bad_cnt, d_bad_cnt, 4, cudaMemcpyDeviceToHost, ctx->s_main));
   if ((rc = check_status(ctx))) return rc;
+  drain.armed = false;
   if (bad_cnt) return fail(ctx, POSLO_EINVAL, "%u points do not decode", bad_cnt);
   memcpy(out, h, 32);
   return POSLO_OK;
@@ -2373,6 +2408,7 @@ int poslo_distill_stream(poslo_ctx* ctx, const poslo_batch* batch, uint64_t chun
     max_bytes = std::max<uint64_t>(max_bytes, batch->offs[hi] - batch->offs[lo]);
     max_n = std::max(max_n, hi - lo);
   }
+  DrainOnError drain{ctx, true};
   // two sets of staging buffers: messages, offsets (rebased to the chunk), s, R
   uint8_t *msgs[2], *sv[2], *Rv[2];
   uint64_t* offs[2];
@@ -2424,6 +2460,7 @@ int poslo_distill_stream(poslo_ctx* ctx, const poslo_batch* batch, uint64_t chun
     total += got;
   }
   CU(cudaStreamSynchronize(ctx->s_copy));
+  drain.armed = false;
   *n_invalid = total;
   *accept = total == 0 ? 1 : 0;
   if (total > cap || (total && !invalid_idx))
@@ -2513,6 +2550,7 @@ int poslo_distill_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrell
   if (!ctx || !valid || !ccd || !ccd->s_v || !ccd->R_v || !ccd->umbrellas)
     return fail(ctx, POSLO_EINVAL, "bad distill_c arguments");
   int rc;
+  DrainOnError drain{ctx};
   Staged sb;
   uint64_t n1 = 0;
   uint32_t* tableY;
@@ -2558,6 +2596,7 @@ int poslo_distill_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrell
   CU(cudaMemcpyAsync(&cnt, d_cnt, 8, cudaMemcpyDeviceToHost, ctx->s_main));
   if ((rc = check_status(ctx))) return rc;
   kforget.armed = false;   // the key decoded: its table is sound
+  drain.armed = false;
   store_le_words(hw.data(), ccd->s_v);
   memcpy(ccd->R_v, he.data(), 32);
   for (uint32_t l = 0; l < n_umbrella; ++l) {
@@ -2579,6 +2618,7 @@ int poslo_sebver_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrella
       (mode == POSLO_SEBVER_U && !ccd->umbrellas))
     return fail(ctx, POSLO_EINVAL, "bad sebver_c arguments");
   int rc;
+  DrainOnError drain{ctx};
   Staged sb;
   uint64_t n1 = 0;
   uint32_t* tableY;
@@ -2602,6 +2642,7 @@ int poslo_sebver_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrella
   if (nchk == 0) {
     if ((rc = check_status(ctx))) return rc;
     kforget.armed = false;   // the key decoded: its table is sound
+    drain.armed = false;
     return POSLO_OK;
   }
   uint8_t *d_mask, *s_chk, *R_chk, *bad, *d_bits;
@@ -2651,6 +2692,7 @@ int poslo_sebver_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrella
   CU(cudaMemcpyAsync(bits, d_bits, nchk, cudaMemcpyDeviceToHost, ctx->s_main));
   if ((rc = check_status(ctx))) return rc;
   kforget.armed = false;   // the key decoded: its table is sound
+  drain.armed = false;
   return POSLO_OK;
 }
 
@@ -2891,6 +2933,7 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
   if (N && (!mb->offs || !mb->s || !mb->R)) return fail(ctx, POSLO_EINVAL, "missing batch arrays");
   if (mb->on_device && N && !device_aligned(mb->offs, mb->s, mb->R))
     return fail(ctx, POSLO_EINVAL, "device-resident offs must be 8-byte aligned, s and R 16-byte aligned");
+  DrainOnError drain{ctx};
   if ((rc = reset_status(ctx))) return rc;
   // ---- stage the concatenated batch and the segment tables
   poslo_batch view{};
@@ -3182,6 +3225,7 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
     CU(cudaMemcpyAsync(ctx->h_small, d_idx, 8 * (1 + first), cudaMemcpyDeviceToHost, ctx->s_main));
     if ((rc = check_status(ctx))) return rc;
     if ((rc = check_keys())) return rc;
+    drain.armed = false;
     if (settled) (*settled)(any.data());
     for (uint32_t d = 0; d < nd; ++d) accept[d] = any[d] ? 0 : 1;
     uint64_t cnt;
@@ -3425,6 +3469,7 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
       write_pairs(g.data(), got);
     }
   }
+  drain.armed = false;
   *n_invalid = cnt;
   if (cnt > cap) return fail(ctx, POSLO_EBUFSMALL, "%llu invalid entries, room for %llu", (unsigned long long)cnt,
                              (unsigned long long)cap);
