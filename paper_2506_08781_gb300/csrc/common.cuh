@@ -14,13 +14,13 @@
 
 #include "aes128.cuh"
 #include "ge25519.cuh"
+#include "hash_grid.h"
 #include "sc25519.cuh"
 #include "sha256.cuh"
 
 namespace poslo {
 
 
-constexpr int kHashThreads = 128;
 constexpr int kHashBlocksPerSm = 4;   // resident SHA-256 hashing blocks: 128 registers, 47 KiB each
 constexpr int kPointThreads = 128;
 // Block size of the short kernels that run beside the decoding (weights, counting sort):
@@ -790,7 +790,7 @@ constexpr int kPointBlocksBeside = 3;
 enum HashPlace { kHashAlone, kHashBeside };
 unsigned hash_groups(int inst, int sm_count, uint64_t n);
 cudaError_t hash_kernels_init();   // once per device, before the first POSLO+ launch
-void launch_hash(int inst, unsigned groups, cudaStream_t st, HashArgs a, HashPlace place);
+void launch_hash(int inst, unsigned groups, int sm_count, cudaStream_t st, HashArgs a, HashPlace place);
 void launch_points(unsigned grid, cudaStream_t st, const PointArgs& a);
 struct ZPre { uint32_t w[10]; };   // BE words of "POSLO-Z" || verifier_seed || (byte 39 = 0)
 __global__ void k_weights(const ZPre zp, uint64_t n, uint64_t first, uint32_t* z_out);

@@ -52,7 +52,6 @@ __global__ void k_epoch_seeds(const DsNode* __restrict__ ds, int nds, uint64_t e
 // the order, so that the warps of a group carry like amounts of work.  Per entry, one loop
 // drives every SHA-256 compression (the PRF block, the message blocks, and the weight block in
 // weighted mode) through a single inlined copy of the compression function.
-constexpr int kHashTile = 256;
 constexpr int kHashClasses = 32;   // one per lane: the prefix sums are a warp scan
 constexpr int kHashPer = kHashTile / kHashThreads;
 static_assert(kHashPer == 2, "a thread takes one entry from each end of the order");
@@ -162,7 +161,7 @@ __global__ void __launch_bounds__(kHashThreads * GROUPS, MINB) k_hash(const Hash
   __shared__ uint32_t s_cnt_[GROUPS][kHashClasses], s_off_[GROUPS][kHashClasses];
   const int g = GROUPS == 1 ? 0 : (int)(threadIdx.x / kHashThreads);
   const uint32_t tid = threadIdx.x % kHashThreads;
-  const uint32_t group = blockIdx.x * GROUPS + g;
+  const uint32_t group = hash_group(blockIdx.x, g, gridDim.x);
   uint16_t* s_order = s_order_[g];
   uint32_t *s_cnt = s_cnt_[g], *s_off = s_off_[g];
   uint32_t* tail = tails + (INST == kInstAes ? 0 : tid);
@@ -666,9 +665,7 @@ void launch_epoch_seeds(int inst, unsigned grid, unsigned block, cudaStream_t st
 constexpr int kAesGroupsAlone = 4, kAesGroupsBeside = 2;
 
 unsigned hash_groups(int inst, int sm_count, uint64_t n) {
-  const uint64_t need = (n + kHashThreads - 1) / kHashThreads;
-  const uint64_t cap = (uint64_t)sm_count * (inst == kInstAes ? kAesGroupsAlone : kHashBlocksPerSm);
-  return (unsigned)(need < 1 ? 1 : need < cap ? need : cap);
+  return hash_groups_of(n, (uint32_t)sm_count * (inst == kInstAes ? kAesGroupsAlone : kHashBlocksPerSm));
 }
 
 cudaError_t hash_kernels_init() {
@@ -679,14 +676,14 @@ cudaError_t hash_kernels_init() {
                               (int)kAesWideBytes);
 }
 
-void launch_hash(int inst, unsigned groups, cudaStream_t st, HashArgs a, HashPlace place) {
+void launch_hash(int inst, unsigned groups, int sm_count, cudaStream_t st, HashArgs a, HashPlace place) {
   a.ngroups = groups;
   if (inst == kInstAes) {
     if (place == kHashAlone)
-      k_hash<kInstAes, 1, kAesGroupsAlone><<<(groups + kAesGroupsAlone - 1) / kAesGroupsAlone,
+      k_hash<kInstAes, 1, kAesGroupsAlone><<<hash_blocks(groups, kAesGroupsAlone, sm_count),
                                              kHashThreads * kAesGroupsAlone, kAesWideBytes, st>>>(a);
     else
-      k_hash<kInstAes, 2, kAesGroupsBeside><<<(groups + kAesGroupsBeside - 1) / kAesGroupsBeside,
+      k_hash<kInstAes, 2, kAesGroupsBeside><<<hash_blocks(groups, kAesGroupsBeside, sm_count),
                                               kHashThreads * kAesGroupsBeside, kAesWideBytes, st>>>(a);
   } else {
     k_hash<kInstSha, kHashBlocksPerSm, 1><<<groups, kHashThreads, 0, st>>>(a);

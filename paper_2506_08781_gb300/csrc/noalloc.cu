@@ -128,7 +128,7 @@ extern "C" int poslo_hash_entries_noalloc(const poslo_batch* batch, uint8_t* e_o
   a.e_out = e_out;
   a.partial = partial;
   a.status = status;
-  launch_hash(kInstSha, (unsigned)blocks, st, a, kHashAlone);
+  launch_hash(kInstSha, (unsigned)blocks, sms, st, a, kHashAlone);
   if (cudaGetLastError() != cudaSuccess) return POSLO_EDEVICE;
   uint32_t h_status = 0;
   if (cudaMemcpyAsync(&h_status, status, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess) return POSLO_EDEVICE;

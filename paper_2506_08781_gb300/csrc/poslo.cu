@@ -485,7 +485,7 @@ int run_hash(poslo_ctx* ctx, const poslo_batch* b, const Staged& sb, uint8_t* e_
   a.status = ctx->status;
   cudaEvent_t tb, te;
   timer_begin(ctx, "hash", ctx->s_main, &tb, &te);
-  launch_hash((int)ctx->inst, (unsigned)blocks, ctx->s_main, a, alone ? kHashAlone : kHashBeside);
+  launch_hash((int)ctx->inst, (unsigned)blocks, ctx->sm_count, ctx->s_main, a, alone ? kHashAlone : kHashBeside);
   ++ctx->launch_count;
   CU(cudaGetLastError());
   timer_end(ctx, "hash", ctx->s_main, tb, te);
@@ -1596,7 +1596,7 @@ int poslo_aver_partial(poslo_ctx* ctx, const poslo_batch* batch, uint32_t agg_mo
     cudaEvent_t tb, te;
     if (!weighted) {
       timer_begin(ctx, "hash", ctx->s_main, &tb, &te);
-      launch_hash((int)ctx->inst, nhb, ctx->s_main, a, F ? kHashBeside : kHashAlone);
+      launch_hash((int)ctx->inst, nhb, ctx->sm_count, ctx->s_main, a, F ? kHashBeside : kHashAlone);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", ctx->s_main, tb, te);
@@ -1613,7 +1613,7 @@ int poslo_aver_partial(poslo_ctx* ctx, const poslo_batch* batch, uint32_t agg_mo
       MsmState ms;
       if ((rc = run_msm_sort(ctx, ctx->s_main, z, 4, nullptr, n, ms))) return rc;
       timer_begin(ctx, "hash", ctx->s_hash, &tb, &te);
-      launch_hash((int)ctx->inst, nhb, ctx->s_hash, a, kHashBeside);
+      launch_hash((int)ctx->inst, nhb, ctx->sm_count, ctx->s_hash, a, kHashBeside);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", ctx->s_hash, tb, te);
@@ -1874,7 +1874,7 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
       if ((rc = launch_seeds())) return rc;
       cudaEvent_t tb, te;
       timer_begin(ctx, "hash", ctx->s_main, &tb, &te);
-      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->s_main, ha, kHashBeside);
+      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->sm_count, ctx->s_main, ha, kHashBeside);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", ctx->s_main, tb, te);
@@ -1963,7 +1963,7 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     {
       cudaEvent_t tb, te;
       timer_begin(ctx, "hash", hs, &tb, &te);
-      launch_hash((int)ctx->inst, (unsigned)hblocks, hs, a, kHashBeside);
+      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->sm_count, hs, a, kHashBeside);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", hs, tb, te);
@@ -3200,7 +3200,7 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
       if ((rc = run_points(ctx, sb.R, N, pts, badR, &ppart, &npb))) return rc;
       cudaEvent_t tb, te;
       timer_begin(ctx, "hash", ctx->s_main, &tb, &te);
-      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->s_main, ha, kHashBeside);
+      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->sm_count, ctx->s_main, ha, kHashBeside);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", ctx->s_main, tb, te);
@@ -3277,7 +3277,7 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
       a.z_in = z;
       cudaEvent_t tb, te;
       timer_begin(ctx, "hash", ctx->s_hash, &tb, &te);
-      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->s_hash, a, kHashBeside);
+      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->sm_count, ctx->s_hash, a, kHashBeside);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", ctx->s_hash, tb, te);

@@ -5,10 +5,12 @@
 #pragma once
 #include <cstdint>
 
+#ifndef POSLO_HD
 #ifdef __CUDACC__
 #define POSLO_HD __host__ __device__ __forceinline__
 #else
 #define POSLO_HD inline
+#endif
 #endif
 
 namespace poslo {
