@@ -152,6 +152,7 @@ __device__ __forceinline__ EntryStream entry_stream(const uint8_t* m, uint32_t L
 }
 
 // SHA-256(m || x) for one entry; returns the 8 state words.
+template <bool IMAD>
 __device__ __forceinline__ void hash_entry(const uint8_t* m, uint32_t L, const uint32_t x[4], uint32_t st[8]) {
   const EntryStream es = entry_stream(m, L, x);
   const uint32_t total = L + 16;
@@ -171,7 +172,7 @@ __device__ __forceinline__ void hash_entry(const uint8_t* m, uint32_t L, const u
         w[15] |= total << 3;
       }
     }
-    sha256_compress(st, w);
+    sha256_compress<IMAD>(st, w);
   }
 }
 
@@ -188,10 +189,10 @@ __device__ __forceinline__ void prf_node_i(const C& c, const uint32_t z[4], uint
   else prf_node(z, bit, out);
 }
 
-template <int INST, class C>
+template <int INST, bool IMAD = true, class C>
 __device__ __forceinline__ void prf_entry_i(const C& c, const uint32_t x0[4], uint32_t j, uint32_t out[4]) {
   if constexpr (INST == kInstAes) prf_entry_aes(c, x0, j, out);
-  else prf_entry(x0, j, out);
+  else prf_entry<IMAD>(x0, j, out);
 }
 
 // MDC-2-AES-128 over the padded stream: (L + 16 + 16) / 16 blocks (the 0x80 byte always
@@ -225,14 +226,14 @@ __device__ __forceinline__ void mdc2_stream(const C& c, const EntryStream& es, u
 }
 
 // H(m || x) as 8 little-endian digest words for the instantiation.
-template <int INST, class C>
+template <int INST, bool IMAD = true, class C>
 __device__ __forceinline__ void entry_digest(const C& c, const uint8_t* m, uint32_t L, const uint32_t x[4],
                                              uint32_t dig[8]) {
   if constexpr (INST == kInstAes) {
     mdc2_stream(c, entry_stream(m, L, x), dig);
   } else {
     uint32_t st[8];
-    hash_entry(m, L, x, st);
+    hash_entry<IMAD>(m, L, x, st);
 #pragma unroll
     for (int q = 0; q < 8; ++q) dig[q] = bswap32(st[q]);
   }
@@ -446,7 +447,8 @@ __device__ __forceinline__ void store_words_bytes(uint8_t* b, const uint32_t v[8
   }
 }
 
-// r_i^j = SHA-256(r || le32(i) || le32(j) || 0x00) mod q: one block of 41 bytes.
+// r_i^j = SHA-256(r || le32(i) || le32(j) || 0x00) mod q: one block of 41 bytes (one thread walks
+// an epoch's: latency counts, sha256_compress).
 __device__ __forceinline__ sc nonce_c(const uint32_t rw[8], uint32_t i, uint32_t j) {
   uint32_t w[16];
 #pragma unroll
@@ -459,7 +461,7 @@ __device__ __forceinline__ sc nonce_c(const uint32_t rw[8], uint32_t i, uint32_t
   w[15] = 41 * 8;
   uint32_t st[8];
   sha256_init(st);
-  sha256_compress(st, w);
+  sha256_compress<false>(st, w);
   uint32_t d[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) d[k] = bswap32(st[k]);

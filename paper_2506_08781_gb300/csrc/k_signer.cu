@@ -121,10 +121,10 @@ __global__ void k_sign_c(const SignCArgs a) {
   for (uint32_t j = 0; j < a.n2; ++j) {
     const uint64_t t = k * a.n2 + j;
     uint32_t x[4];
-    prf_entry_i<INST>(c, x0, j, x);
+    prf_entry_i<INST, false>(c, x0, j, x);
     const uint64_t o0 = a.offs[t] - a.base_off, o1 = a.offs[t + 1] - a.base_off;
     uint32_t d[8];
-    entry_digest<INST>(c, a.msgs + o0, (uint32_t)(o1 - o0), x, d);
+    entry_digest<INST, false>(c, a.msgs + o0, (uint32_t)(o1 - o0), x, d);
     const sc e = sc_reduce256(d);
     acc = sc_add(acc, sc_sub(nonce_c(rw, (uint32_t)i, j), sc_mul(e, y)));
   }
