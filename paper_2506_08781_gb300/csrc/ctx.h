@@ -122,8 +122,9 @@ namespace poslo_host {
 // poslo_aver_multi with the devices' window tables given (device pointers, one per device,
 // host array); with key_tables = nullptr the tables are built from the keys (poslo.cu).
 // When settled is given, it is called once the devices that need no entry-level localisation
-// are known (flagged[d] = 0: device d is accepted, its result is final), before the
-// localisation of the others runs; a service publishes those results early.
+// are known (flagged[d] = 0: device d is accepted, its result is final), without waiting for the
+// localisation of the others, which may be running by then; a service publishes those results
+// early.  (A small batch is checked entry by entry at once: its results are known together.)
 int aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const uint32_t* const* key_tables, uint8_t* accept,
                uint64_t* invalid_pairs, uint64_t cap, uint64_t* n_invalid,
                const std::function<void(const uint8_t* flagged)>* settled = nullptr);

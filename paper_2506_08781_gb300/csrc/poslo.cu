@@ -3439,10 +3439,9 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
     }
     uint8_t confirmed = 0;
     CU(cudaMemcpyAsync(&confirmed, d_acc, 1, cudaMemcpyDeviceToHost, ctx->s_main));
-    rc = check_status(ctx);
-    if (localised) CU(cudaStreamSynchronize(ctx->s_table));
-    if (rc) return rc;
+    if ((rc = check_status(ctx))) return rc;
     if (!confirmed) {   // cancelling errors: settle every device
+      if (localised) CU(cudaStreamSynchronize(ctx->s_table));   // the lists are rewritten
       std::fill(flag.begin(), flag.end(), 1);
       list_flagged();
       localised = false;
@@ -3450,7 +3449,9 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
   } else {
     list_flagged();
   }
+  // the other devices' answers need not wait for the entry checks that run beside the confirmation
   if (settled) (*settled)(flag.data());
+  if (localised) CU(cudaStreamSynchronize(ctx->s_table));
   for (uint32_t d = 0; d < nd; ++d) accept[d] = 1;
   const uint32_t nfl = (uint32_t)fl.size();
   uint64_t cnt = 0;

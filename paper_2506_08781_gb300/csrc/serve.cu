@@ -187,9 +187,9 @@ void run_batch(Server* S, poslo_ctx* w, TakenBatch& B) {
   std::vector<uint8_t> acc(nd);
   std::vector<uint64_t> pairs(2 * std::max<uint64_t>(total, 1));
   uint64_t cnt = 0;
-  // requests whose device passes the device-level checks are final before the entry-level
-  // localisation of the others: publish them at once (a reader may then release them, so
-  // they are not touched again here)
+  // requests whose device passes the device-level checks are final whatever the entry-level
+  // localisation of the others finds: publish them without waiting for it (a reader may then
+  // release them, so they are not touched again here; the batch's device copy is the worker's)
   std::vector<uint8_t> published(nd, 0);
   const std::function<void(const uint8_t*)> settled = [&](const uint8_t* flagged) {
     {
