@@ -157,14 +157,16 @@ def probe_int_peaks(device: int) -> dict:
 #     half (the fold by 19).
 #   A 64-bit product (mad.lo.cc / madc.hi.cc fused into one wide multiply-add) takes two
 #     mad.lo issue slots on this GPU, so the work is expressed in those: 2 x wide + low.
-#   SHA-256: 1,384 ALU instructions per compression with 3-input LOP3/IADD3 and funnel
-#     shifts (64 rounds x 14 + 48 schedule words x 10 + 8); compressions per entry =
-#     1 (PRF) + ceil((L + 25) / 64) (H)
+#   SHA-256: what a compression cannot do off the ALU pipe: per round 6 rotations, a 3-input
+#     XOR after each three of them, the choice, the majority and the addition of the round
+#     constant (11), per schedule word 4 rotations, 2 shifts and two 3-input XORs (8):
+#     64 x 11 + 48 x 8 = 1,088.  The other additions have register operands only and run on
+#     the IMAD pipe beside it.  Compressions per entry = 1 (PRF) + ceil((L + 25) / 64) (H)
 SQ_WIDE, MUL_WIDE = 44, 72
 DECODE_SQ, DECODE_MUL = 255, 21 + 7
 WIDE_PER_DECODE = DECODE_SQ * SQ_WIDE + DECODE_MUL * MUL_WIDE    # 13,236
 IMAD_SLOTS_PER_DECODE = 2 * WIDE_PER_DECODE + DECODE_SQ + DECODE_MUL
-ALU_PER_COMPRESSION = 64 * 14 + 48 * 10 + 8
+ALU_PER_COMPRESSION = 64 * 11 + 48 * 8
 # DRAM bytes (read + write) of one k_points launch over 2^20 entries, from an ncu capture:
 # the 32 MB of encodings read once; of the 100 MB of decoded points written, the part that has
 # left L2 by the end of the launch.
@@ -523,15 +525,16 @@ def bench_stream(device: int) -> dict:
 
 # ------------------------------------------------------------------------------ POSLO-C, hash-bound
 
-# Thread instructions per AES-128 of the table cipher with its on-the-fly key schedule, counted
-# from the algorithm (not the compiled code): each of the 16 round lookups and 4 key-schedule
-# S-box lookups is a byte extract, an address computation and a shared-memory read (3); a full
-# round adds 8 three-input XORs and 15 key-schedule operations (masks, shifts, the XOR chain,
-# Rcon): 9 x (60 + 8 + 15) = 747; the last round's 16 S-box reads with their masks and shifts
-# (4 x 20) + 4 XORs + its key schedule (27) = 111; the initial AddRoundKey 4; the MMO/MDC-2
-# feed-forward XOR 4: 866 (the four rotated tables leave no rotations).  Instruction issue is one
-# bound; the 200 table reads (one shared-memory wavefront a lane) are the other, nearly met.
-AES_INSTR = 9 * (16 * 3 + 4 * 3 + 8 + 15) + (4 * 20 + 4 + 27) + 4 + 4
+# POSLO+ hashing, per AES-128 of the table cipher with its on-the-fly key schedule, counted from
+# the algorithm (not the compiled code).  Table reads: 16 round lookups and 4 key-schedule S-box
+# lookups in each of 10 rounds, 200, of which a shared-memory wavefront serves the 32 lanes of a
+# warp: one wavefront a cycle and SM is the kernel's bound.  Instructions: a lookup is a byte
+# permute (the address) and the read; a full round adds 8 three-input XORs for its columns and 7
+# operations of the key schedule (3 permutes to join the S-box bytes, 4 XORs); the last round joins
+# its columns from S-box bytes (4 x 3 permutes and an XOR); AddRoundKey at the start and the
+# MMO/MDC-2 feed-forward are 4 XORs each: 400 + 9 x 15 + 23 + 8 = 566.
+AES_LOOKUPS = 10 * (16 + 4)
+AES_INSTR = 2 * AES_LOOKUPS + 9 * (8 + 7) + (4 * 4 + 7) + 4 + 4
 
 
 CCD_UMBRELLAS = 64
@@ -614,19 +617,22 @@ def bench_hash_bound(device: int, steps: int, warmup: int) -> dict:
             ctx.close()
             if inst == poslo.INST_AES:
                 aes = int(np.sum(2 * ((L + 32) // 16) + 2))           # MDC-2 blocks x 2 + the PRF's 2
-                work = {"unit": "G thread-instructions/s", "per_launch": aes * AES_INSTR, "pipe": "issue",
-                        "peak_note": "4 warp instructions per clock per SM (32 threads each)",
-                        "aes_calls": aes, "instr_per_aes": AES_INSTR}
-                peak = 4 * 32 * 152 * 2.07e9
+                work = {"unit": "G table reads/s", "per_launch": aes * AES_LOOKUPS, "pipe": "shared memory",
+                        "peak_note": "one wavefront (32 reads) per clock per SM"}
+                peak = 32 * 152 * 2.07e9
+                issue = aes * AES_INSTR / (hash_ms * 1e-3) / (4 * 32 * 152 * 2.07e9)
             else:
                 work = {"unit": "G ALU ops/s", "per_launch": compressions(msgs) * ALU_PER_COMPRESSION,
                         "pipe": "ALU (LOP3/SHF/IADD3)", "peak_note": "64 ops per clock per SM"}
                 peak = 64 * 152 * 2.07e9
+                issue = None
             ach = work["per_launch"] / (hash_ms * 1e-3)
             row[name] = {"entries_per_s": N_ENTRIES / (ms * 1e-3), "ms_per_aver": ms, "hash_kernel_ms": hash_ms,
                          "hash_roofline": {"bound": work["pipe"], "achieved": ach / 1e9, "peak": peak / 1e9,
                                            "unit": work["unit"], "frac": ach / peak,
                                            "peak_source": work["peak_note"] + " at 2070 MHz, 152 SMs"}}
+            if issue is not None:   # the next bound: four warp instructions per clock per SM
+                row[name]["hash_roofline"].update(aes_calls=aes, instr_per_aes=AES_INSTR, frac_of_issue=issue)
             if label.startswith("U"):
                 row[name]["distill_c"] = bench_distill_c(ctx_inst=inst, device=device, km=km, msgs=msgs, Y=Y,
                                                          epoch_R=epoch_R, s_ep=s_ep, steps=steps, warmup=warmup)
@@ -1135,7 +1141,7 @@ def run_ours(args):
         pk = peaks["lop3_ops"] / 1e9
         roof = {"bound": "alu", "pipe": "ALU", "kernel": dom, "achieved": ach, "peak": pk, "unit": "Gop/s",
                 "frac": ach / pk, "traffic": None, "peak_source": "probed lop3 issue rate on this GPU",
-                "work": "1,384 ALU ops per SHA-256 compression"}
+                "work": f"{ALU_PER_COMPRESSION:,} ALU ops per SHA-256 compression"}
     clocks = clk.summary()
 
     if rank == 0:
