@@ -44,8 +44,8 @@ __global__ void __launch_bounds__(kCcdThreads) k_scalar_group_sums(const uint8_t
 }
 
 // enc[g] = encoding of the sum of the decoded points pts[g G .. (g+1) G) that are neither
-// flagged in skip nor undecodable (bad), and the sum itself in the decoding's partial format
-// (kPointPartialWords, bad count 0), so that the sum over all groups needs no second pass over
+// flagged in skip nor undecodable (bad), and (given partial) the sum itself in the decoding's
+// partial format (kPointPartialWords, bad count 0), so that the sum over all groups needs no second pass over
 // the points.  One block of T threads per group: latency-bound, G / T additions of a lane, a
 // tree by quads and one inversion (64 groups of 64 points: 74 -> 35 us; all 4,096 points in one
 // block before: 177 us).
@@ -65,9 +65,9 @@ __global__ void __launch_bounds__(T) k_point_group_sums(const uint32_t* pts, con
   __shared__ __align__(16) uint32_t sp[T][32];
   ge_store(sp[threadIdx.x], acc);
   compact::quad_tree(sp, G < T ? (int)G : T);
-  if (threadIdx.x < 32) partial[kPointPartialWords * g + threadIdx.x] = sp[0][threadIdx.x];
+  if (partial && threadIdx.x < 32) partial[kPointPartialWords * g + threadIdx.x] = sp[0][threadIdx.x];
   if (threadIdx.x == 0) {
-    partial[kPointPartialWords * g + 32] = 0;
+    if (partial) partial[kPointPartialWords * g + 32] = 0;
     uint32_t b[8];
     compact::encode(ge_load(sp[0]), b);
     for (int k = 0; k < 8; ++k) reinterpret_cast<uint32_t*>(enc + 32 * g)[k] = b[k];

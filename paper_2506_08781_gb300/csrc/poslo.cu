@@ -2481,22 +2481,17 @@ void store_le_words(const uint32_t* w, uint8_t* out) {
     for (int b = 0; b < 4; ++b) out[4 * k + b] = (uint8_t)(w[k] >> (8 * b));
 }
 
-// Shared part of C.Distill and SeBVer: checks the batch (whole epochs, per-epoch s~_i and
-// R~_i), stages it, starts the key table, and leaves the per-epoch sums e~_i (n1 x 32 bytes,
-// limbs little-endian) in *esum.
-// The key's window table comes from the key cache; a table this call builds into a new cache
-// slot is forgotten again (kforget) unless the caller disarms it once the key has decoded.
 // Main stream: ok[k] = s_k canonical, R_k decodable (badR) and [8](R_k - e_k Y - s_k G) = O for n
-// independent checks; inv[k] = 1 - ok[k], badS scratch of n bytes.
+// independent checks; inv[k] = 1 - ok[k].  ok holds the checks' non-canonical flags until the flip.
 void launch_check_list(poslo_ctx* ctx, const uint8_t* e, const uint8_t* s, const uint32_t* pts, const uint8_t* badR,
-                       uint8_t* badS, uint64_t n, const uint32_t* tableY, uint8_t* inv, uint8_t* ok) {
-  k_noncanonical<<<(unsigned)((n + 255) / 256), 256, 0, ctx->s_main>>>(s, n, badS);
+                       uint64_t n, const uint32_t* tableY, uint8_t* inv, uint8_t* ok) {
+  k_noncanonical<<<(unsigned)((n + 255) / 256), 256, 0, ctx->s_main>>>(s, n, ok);
   DirectCheckArgs a{};
   a.e = e;
   a.s = s;
   a.pts = pts;
   a.badR = badR;
-  a.badS = badS;
+  a.badS = ok;
   a.n = n;
   a.tableY = tableY;
   a.tableG = ctx->tableG;
@@ -2506,6 +2501,11 @@ void launch_check_list(poslo_ctx* ctx, const uint8_t* e, const uint8_t* s, const
   ctx->launch_count += 3;
 }
 
+// Shared part of C.Distill and SeBVer: checks the batch (whole epochs, per-epoch s~_i and
+// R~_i), stages it, starts the key table, and leaves the per-epoch sums e~_i (n1 x 32 bytes,
+// limbs little-endian) in *esum.
+// The key's window table comes from the key cache; a table this call builds into a new cache
+// slot is forgotten again (kforget) unless the caller disarms it once the key has decoded.
 int ccd_common(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrella, Staged& sb, uint64_t& n1,
                uint32_t** tableY, uint8_t** esum, std::vector<uint32_t>& kmiss, KeyForget& kforget) {
   int rc;
@@ -2563,30 +2563,34 @@ int poslo_distill_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrell
   uint8_t *badR, *ok, *inv, *encs;
   uint64_t* d_idx;
   if ((rc = ensure_t(ctx, "ccd_pts", 4 * kPtsWords * n1, &pts))) return rc;
-  if ((rc = ensure_t(ctx, "ccd_badR", 2 * n1, &badR))) return rc;
-  uint8_t* badS = badR + n1;
+  if ((rc = ensure_t(ctx, "ccd_badR", n1, &badR))) return rc;
   if ((rc = ensure_t(ctx, "ccd_ok", 2 * n1, &ok))) return rc;
   inv = ok + n1;
   if ((rc = ensure_t(ctx, "ccd_words", 32 * (1 + (size_t)n_umbrella), &words))) return rc;
   if ((rc = ensure_t(ctx, "ccd_encs", 32 * (1 + (size_t)n_umbrella), &encs))) return rc;
-  if ((rc = ensure_t(ctx, "ccd_usums", 4 * kPointPartialWords * (size_t)n_umbrella, &usums))) return rc;
   const uint64_t capn = std::max<uint64_t>(std::min<uint64_t>(ccd->cap, n1), 1);
   if ((rc = ensure_t(ctx, "ccd_idx", 8 * capn + 8, &d_idx))) return rc;
   uint64_t* d_cnt = d_idx + capn;
   if ((rc = run_points(ctx, sb.R, n1, pts, badR, &ppart, &npb, ctx->ev_staged))) return rc;
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_points, 0));
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_table, 0));
-  // b_i for every epoch, then the umbrellas (groups 1..n^u) and from their sums ccd^v (group 0)
-  launch_check_list(ctx, esum, sb.s, pts, badR, badS, n1, tableY, inv, ok);
+  // b_i for every epoch and ccd^i, then the umbrellas (groups 1..n^u) and from their sums ccd^v
+  // (group 0); its points from the epochs again when the memory budget has no room for the sums
+  launch_check_list(ctx, esum, sb.s, pts, badR, n1, tableY, inv, ok);
+  const uint64_t first_epoch = batch->first_index / batch->n2;
+  if ((rc = run_compact(ctx, inv, n1, first_epoch, d_idx, std::min<uint64_t>(ccd->cap, n1), d_cnt))) return rc;
+  if (ensure_t(ctx, "ccd_usums", 4 * kPointPartialWords * (size_t)n_umbrella, &usums) != POSLO_OK) {
+    cudaGetLastError();
+    usums = nullptr;
+  }
   k_scalar_group_sums<<<n_umbrella, kCcdThreads, 0, ctx->s_main>>>(sb.s, g, n1, inv, words + 8);
   launch_point_group_sums(n_umbrella, ctx->s_main, pts, badR, g, n1, inv, encs + 32, usums);
   k_scalar_group_sums<<<1, kCcdThreads, 0, ctx->s_main>>>(reinterpret_cast<const uint8_t*>(words + 8), n_umbrella,
                                                           n_umbrella, nullptr, words);
-  k_sum_encode<<<1, kFinalThreads, 0, ctx->s_main>>>(usums, n_umbrella, nullptr, encs, nullptr);
+  if (usums) k_sum_encode<<<1, kFinalThreads, 0, ctx->s_main>>>(usums, n_umbrella, nullptr, encs, nullptr);
+  else launch_point_group_sums(1, ctx->s_main, pts, badR, n1, n1, inv, encs, nullptr);
   ctx->launch_count += 4;
   CU(cudaGetLastError());
-  const uint64_t first_epoch = batch->first_index / batch->n2;
-  if ((rc = run_compact(ctx, inv, n1, first_epoch, d_idx, std::min<uint64_t>(ccd->cap, n1), d_cnt))) return rc;
   std::vector<uint32_t> hw(8 * (1 + (size_t)n_umbrella));
   std::vector<uint8_t> he(32 * (1 + (size_t)n_umbrella));
   uint64_t cnt = 0;
@@ -2654,7 +2658,7 @@ int poslo_sebver_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrella
   if ((rc = ensure_t(ctx, "seb_s", 32 * nchk, &s_chk))) return rc;
   if ((rc = ensure_t(ctx, "seb_R", 32 * nchk, &R_chk))) return rc;
   if ((rc = ensure_t(ctx, "seb_pts", 4 * kPtsWords * nchk, &pts))) return rc;
-  if ((rc = ensure_t(ctx, "seb_bad", 4 * nchk, &bad))) return rc;
+  if ((rc = ensure_t(ctx, "seb_bad", 2 * nchk, &bad))) return rc;
   d_bits = bad + nchk;
   CU(cudaMemcpyAsync(d_mask, mask.data(), n1, cudaMemcpyHostToDevice, ctx->s_main));
   if (mode == POSLO_SEBVER_V) {
@@ -2686,8 +2690,8 @@ int poslo_sebver_c(poslo_ctx* ctx, const poslo_batch* batch, uint32_t n_umbrella
   if ((rc = run_points(ctx, R_chk, nchk, pts, bad, &ppart, &npb))) return rc;
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_points, 0));
   CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_table, 0));
-  launch_check_list(ctx, reinterpret_cast<const uint8_t*>(e_chk), s_chk, pts, bad, bad + 2 * nchk, nchk, tableY,
-                    bad + 3 * nchk, d_bits);
+  // (the points are decoded: their encodings make room for the flags)
+  launch_check_list(ctx, reinterpret_cast<const uint8_t*>(e_chk), s_chk, pts, bad, nchk, tableY, R_chk, d_bits);
   CU(cudaGetLastError());
   CU(cudaMemcpyAsync(bits, d_bits, nchk, cudaMemcpyDeviceToHost, ctx->s_main));
   if ((rc = check_status(ctx))) return rc;
