@@ -65,6 +65,7 @@ struct HashArgs {
   const uint32_t* z_in;        // optional (weighted): z_t already computed (k_weights); read, not hashed
   uint8_t* sbad_out;           // optional: n bytes, 1 = s_t is not canonical
   uint32_t ngroups;            // groups of kHashThreads threads, one partial each (set by launch_hash)
+  HashSteps steps;             // their numbering over the grid (set by launch_hash)
   unsigned long long* partial; // per group: 13 u64 limb sums of e, 13 of s, 1 bad count (27 u64)
   uint32_t* status;            // device status word (kErrInput for decreasing offsets)
   // multi-device batches (n_seg > 0): entry t belongs to the device d with

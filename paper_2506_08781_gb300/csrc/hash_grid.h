@@ -34,6 +34,16 @@ POSLO_HD uint32_t hash_blocks(uint32_t groups, uint32_t per_block, uint32_t sms)
   return groups <= sms ? groups : full > sms ? full : sms;
 }
 
-POSLO_HD uint32_t hash_group(uint32_t block, uint32_t g, uint32_t blocks) { return g * blocks + block; }
+// Group g of block b has number b * block_step + g * group_step: across the blocks first, or in a
+// row when every place of the grid has a group.  Then all SMs have work either way, and in a row
+// the last round's tiles end on some SMs before the others, where what is launched behind the
+// hashing begins: POSLO+-C Distill of 2^20 entries 1.04 ms, 1.10 across, of 600,000 0.70 and 0.75
+// (hashing alone of 262,144 entries is 231 us in a row and 211 across).
+struct HashSteps {
+  uint32_t block_step, group_step;
+};
+POSLO_HD HashSteps hash_steps(uint32_t groups, uint32_t blocks, uint32_t per_block) {
+  return groups == blocks * per_block ? HashSteps{per_block, 1u} : HashSteps{1u, blocks};
+}
 
 }  // namespace poslo

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kHashThreads * GROUPS, MINB) k_hash(const Hash
   __shared__ uint32_t s_cnt_[GROUPS][kHashClasses], s_off_[GROUPS][kHashClasses];
   const int g = GROUPS == 1 ? 0 : (int)(threadIdx.x / kHashThreads);
   const uint32_t tid = threadIdx.x % kHashThreads;
-  const uint32_t group = hash_group(blockIdx.x, g, gridDim.x);
+  const uint32_t group = blockIdx.x * a.steps.block_step + g * a.steps.group_step;
   uint16_t* s_order = s_order_[g];
   uint32_t *s_cnt = s_cnt_[g], *s_off = s_off_[g];
   uint32_t* tail = tails + (INST == kInstAes ? 0 : tid);
@@ -677,17 +677,16 @@ cudaError_t hash_kernels_init() {
 }
 
 void launch_hash(int inst, unsigned groups, int sm_count, cudaStream_t st, HashArgs a, HashPlace place) {
+  const uint32_t per = inst != kInstAes ? 1 : place == kHashAlone ? kAesGroupsAlone : kAesGroupsBeside;
+  const uint32_t blocks = hash_blocks(groups, per, sm_count);
   a.ngroups = groups;
-  if (inst == kInstAes) {
-    if (place == kHashAlone)
-      k_hash<kInstAes, 1, kAesGroupsAlone><<<hash_blocks(groups, kAesGroupsAlone, sm_count),
-                                             kHashThreads * kAesGroupsAlone, kAesWideBytes, st>>>(a);
-    else
-      k_hash<kInstAes, 2, kAesGroupsBeside><<<hash_blocks(groups, kAesGroupsBeside, sm_count),
-                                              kHashThreads * kAesGroupsBeside, kAesWideBytes, st>>>(a);
-  } else {
-    k_hash<kInstSha, kHashBlocksPerSm, 1><<<groups, kHashThreads, 0, st>>>(a);
-  }
+  a.steps = hash_steps(groups, blocks, per);
+  if (inst != kInstAes)
+    k_hash<kInstSha, kHashBlocksPerSm, 1><<<blocks, kHashThreads, 0, st>>>(a);
+  else if (place == kHashAlone)
+    k_hash<kInstAes, 1, kAesGroupsAlone><<<blocks, kHashThreads * kAesGroupsAlone, kAesWideBytes, st>>>(a);
+  else
+    k_hash<kInstAes, 2, kAesGroupsBeside><<<blocks, kHashThreads * kAesGroupsBeside, kAesWideBytes, st>>>(a);
 }
 
 void launch_points(unsigned grid, cudaStream_t st, const PointArgs& a) {

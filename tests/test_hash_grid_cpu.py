@@ -19,11 +19,12 @@ int main() {
   for (uint64_t n : ns)
     for (uint32_t per : {1u, 2u, 4u}) {
       const uint32_t groups = hash_groups_of(n, 4 * SMS), blocks = hash_blocks(groups, per, SMS);
+      const HashSteps steps = hash_steps(groups, blocks, per);
       std::set<uint32_t> ids, busy;
       uint32_t in_range = 0;
       for (uint32_t b = 0; b < blocks; ++b)
         for (uint32_t g = 0; g < per; ++g) {
-          const uint32_t id = hash_group(b, g, blocks);
+          const uint32_t id = b * steps.block_step + g * steps.group_step;
           if (id >= groups) continue;
           ++in_range;
           ids.insert(id);
