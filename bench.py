@@ -170,7 +170,7 @@ ALU_PER_COMPRESSION = 64 * 11 + 48 * 8
 # DRAM bytes (read + write) of one k_points launch over 2^20 entries, from an ncu capture:
 # the 32 MB of encodings read once; of the 100 MB of decoded points written, the part that has
 # left L2 by the end of the launch.
-POINTS_DRAM_BYTES_2P20 = 33_746_176 + 44_258_304
+POINTS_DRAM_BYTES_2P20 = 33_633_792 + 53_569_792
 
 
 def make_workload(n=N_ENTRIES, seed=SEED, tamper=0, rank=0, world=1):

@@ -32,8 +32,8 @@
  * any byte.  Every call is synchronous: it returns when its outputs are in
  * the caller's buffers.  Calls on one context must not overlap (they share its streams and
  * workspace); different contexts are independent.  A call returns POSLO_OK or a negative
- * poslo_status; poslo_last_error() then describes the failure.  "Signature invalid" is not
- * an error: it is an output bit or index.
+ * poslo_status; poslo_last_error() then describes the failure, and nothing the call launched is
+ * running any more.  "Signature invalid" is not an error: it is an output bit or index.
  */
 #ifndef POSLO_H_
 #define POSLO_H_

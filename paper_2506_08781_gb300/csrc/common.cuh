@@ -24,8 +24,9 @@ namespace poslo {
 constexpr int kHashBlocksPerSm = 4;   // resident SHA-256 hashing blocks: 128 registers, 47 KiB each
 constexpr int kPointThreads = 128;
 // Block size of the short kernels that run beside the decoding (weights, counting sort):
-// small enough that one of their blocks fits in the registers the three resident decoding
-// blocks of an SM leave free, so they progress during the decoding instead of after it.
+// small enough that their blocks (48 registers a thread, 6,144 a block) fit in the 12,288
+// registers that four resident decoding blocks of an SM leave free, so they progress during the
+// decoding instead of after it.
 #ifndef POSLO_SIDE_THREADS
 #define POSLO_SIDE_THREADS 128
 #endif
@@ -739,8 +740,11 @@ __device__ __forceinline__ bool entry_check_lanes(const uint8_t* e32, const uint
 }
 
 // Lanes per check for n checks in one launch: the fewer the checks, the more lanes shorten each
-// one's chain of additions (1,024 checks: 31 us with 32 lanes); beyond some 2,048 the additions'
-// throughput counts and the choice makes less than 3 %.
+// one's chain of additions (1,024 checks: 31 us with 32 lanes); the more checks, the more their
+// additions' throughput counts, and fewer lanes save the additions of the tree.  Distill with 16
+// lanes / 8, us: 2,100 entries 151 / 173, 3,000 165 / 186, 4,000 185 / 187; from 4,097 on with 8
+// lanes / 16: 8,192 entries 251 / 252, 16,384 with a flip 639 / 651.  32 signers of 2,100 entries
+// 234 / 248, of 4,000 261 / 266.
 constexpr uint64_t kLanes32Max = 2048, kLanes16Max = 4096;
 
 // ---- Distill segment tree (k_distill.cu) ----

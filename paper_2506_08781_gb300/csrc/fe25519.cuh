@@ -487,7 +487,8 @@ __device__ __forceinline__ fe fe_pow_p58(const fe& z) {
 // matrix (u v; q r) of entries at most 2^30, which then moves f, g (exactly) and the
 // coefficients d, e with d z = f, e z = g (mod p): (u d + v e + m p) / 2^30, with m chosen to
 // make the division exact.  Numbers are nine signed limbs of 30 bits; in them p is 2^15 at limb
-// 8 and -19 at limb 0.  |m| <= 2^29, so d and e grow by at most p / 2 a batch.
+// 8 and -19 at limb 0.  |m| <= 2^29, so d and e grow by at most p / 2 a batch.  (Signed limbs of
+// 30 bits with 30 steps collected in a matrix are also how libsecp256k1's modinv32 lays this out.)
 // One thread's chain: about 20 batches of some 1,500 cycles, where the 255 squarings and 11
 // products of z^(p-2) took 95,000 cycles.
 static __device__ __noinline__ fe fe_inv(const fe& z) {

@@ -3,9 +3,9 @@
 // One context owns its CUDA streams: the main stream runs the seeds, weights, counting sort
 // and MSM and the final check; a side stream builds the window table of the public key Y
 // while hashing runs; a third stream decodes and sums the commitments R_t; a fourth hashes
-// the messages during the decoding.  The hash kernel is
-// bound by the integer ALU pipe (SHA-256) and the point kernel by the IMAD pipe (field
-// multiplication), so running them concurrently lets both pipes issue on every SM.
+// the messages.  The hash kernel is bound by the integer ALU pipe (SHA-256) and the point kernel
+// by the IMAD pipe (field multiplication); in a many-signer batch, whose decoding takes three
+// blocks per SM, the two share the SMs.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -355,7 +355,10 @@ constexpr uint64_t kMaxCallEntries = (1ull << 32) - 1;
 constexpr uint64_t kDirectCheckMax = 16384;
 
 // Flagged entries up to which a confirmation subtracts them window by window (one quad per
-// entry and window) instead of by an MSM over them and Horner's rule over the windows.
+// entry and window) instead of by an MSM over them and Horner's rule over the windows.  Distill
+// window by window / by the MSM, ms, of 150,000 entries: 1.74 / 1.96 with 4,097 flips, 1.96 / 2.13
+// with 6,000, 2.49 / 2.54 with 12,000; of 2^20: 4.98 / 5.22, 5.25 / 5.43, 6.23 / 6.25.  The two
+// meet near 12,000, so the line is on the safe side of where they cross.
 constexpr uint64_t kConfirmWindowsMax = 4096;
 
 // Batches of at most this many entries are checked entry by entry at once, without the weighted
@@ -1951,8 +1954,9 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     }
     CU(cudaEventRecord(ctx->ev_main, ctx->s_main));
     CU(cudaStreamWaitEvent(ctx->s_hash, ctx->ev_main, 0));
-    // (measured: hashing beside the decoding, 4.78 ms per 2^20-entry step, beats hashing on the
-    // main stream before the sort, 4.88 ms, and beside the bucket accumulation, 4.95 ms)
+    // (four decoding blocks leave an SM no registers for a hashing block, so the hashing starts as
+    // the decoding's last blocks end and runs beside the sort's; with three decoding blocks and
+    // hashing beside them this call took as long, see kPointBlocksBeside)
     cudaStream_t hs = ctx->s_hash;
     HashArgs a = ha;
     a.weighted = 1;
