@@ -792,9 +792,10 @@ void launch_epoch_seeds(int inst, unsigned grid, unsigned block, cudaStream_t st
 // entries, and 736 us against 718 of 40,013: not taken.)
 constexpr int kPointBlocksPerSm = 4;
 constexpr int kPointBlocksBeside = 3;
-// What shares the SMs with a hashing launch: nothing of its size, or the decoding of one point
-// per entry.
-enum HashPlace { kHashAlone, kHashBeside };
+// What shares the SMs with a hashing launch: nothing of its size; the decoding of one point per
+// entry; or the decoding and an MSM's launches, which such a call waits for longer than for its
+// hashing (its POSLO+ blocks then keep to few SMs, hash_blocks).
+enum HashPlace { kHashAlone, kHashBeside, kHashApart };
 unsigned hash_groups(int inst, int sm_count, uint64_t n);
 cudaError_t hash_kernels_init();   // once per device, before the first POSLO+ launch
 void launch_hash(int inst, unsigned groups, int sm_count, cudaStream_t st, HashArgs a, HashPlace place);

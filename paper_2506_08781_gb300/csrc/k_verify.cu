@@ -680,7 +680,7 @@ cudaError_t hash_kernels_init() {
 
 void launch_hash(int inst, unsigned groups, int sm_count, cudaStream_t st, HashArgs a, HashPlace place) {
   const uint32_t per = inst != kInstAes ? 1 : place == kHashAlone ? kAesGroupsAlone : kAesGroupsBeside;
-  const uint32_t blocks = hash_blocks(groups, per, sm_count);
+  const uint32_t blocks = hash_blocks(groups, per, place == kHashApart ? 0 : sm_count);
   a.ngroups = groups;
   a.steps = hash_steps(groups, blocks, per);
   if (inst != kInstAes)

@@ -1616,7 +1616,7 @@ int poslo_aver_partial(poslo_ctx* ctx, const poslo_batch* batch, uint32_t agg_mo
       MsmState ms;
       if ((rc = run_msm_sort(ctx, ctx->s_main, z, 4, nullptr, n, ms))) return rc;
       timer_begin(ctx, "hash", ctx->s_hash, &tb, &te);
-      launch_hash((int)ctx->inst, nhb, ctx->sm_count, ctx->s_hash, a, kHashBeside);
+      launch_hash((int)ctx->inst, nhb, ctx->sm_count, ctx->s_hash, a, kHashApart);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", ctx->s_hash, tb, te);
@@ -1967,7 +1967,7 @@ int poslo_distill(poslo_ctx* ctx, const poslo_batch* batch, uint64_t* invalid_id
     {
       cudaEvent_t tb, te;
       timer_begin(ctx, "hash", hs, &tb, &te);
-      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->sm_count, hs, a, kHashBeside);
+      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->sm_count, hs, a, kHashApart);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", hs, tb, te);
@@ -3285,7 +3285,7 @@ int poslo_host::aver_multi(poslo_ctx* ctx, const poslo_multi_batch* mb, const ui
       a.z_in = z;
       cudaEvent_t tb, te;
       timer_begin(ctx, "hash", ctx->s_hash, &tb, &te);
-      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->sm_count, ctx->s_hash, a, kHashBeside);
+      launch_hash((int)ctx->inst, (unsigned)hblocks, ctx->sm_count, ctx->s_hash, a, kHashApart);
       ++ctx->launch_count;
       CU(cudaGetLastError());
       timer_end(ctx, "hash", ctx->s_hash, tb, te);
